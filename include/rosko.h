@@ -81,10 +81,10 @@ typedef enum {
  *         value run on the tensor-core dense-panel path, the others on the
  *         sparse path; >= 1001 = never.  At pack time the same field is the
  *         minimum density for which a dense copy is kept.
- *   dense_n_r      C columns per tensor-core CTA tile (128 or 256).
- *   dense_split_k  CTAs over which the stream-K tensor-core path divides its
- *         (tile, K slab) work (default: one per SM); a tile whose K range
- *         is divided is added into C with atomics.
+ *   dense_n_r      C columns per tensor-core tile (128 or 256).
+ *   dense_split_k  CTAs over which the tensor-core path divides its (tile, K
+ *         slab) work, at most one per SM (default: one per SM); a tile whose
+ *         K range is divided is added into C with atomics.
  *   order traversal of a panel inside a B slab by the CUDA-core path:
  *         1 = column order, Alg. 2 as printed (one B row per packed column,
  *         the C row picked by a run-time switch over loc_m);
@@ -95,8 +95,10 @@ typedef enum {
  *         128-row tile touches (the tile's col_ind); needs m_r = 16,
  *         m_c = 128.
  *   mode  a rosko_sched_mode.
- *   dense_m_c  C rows per tensor-core CTA tile: 128 (one MMA per K step) or
- *         256 (two 128-row MMAs sharing each staged B slab).
+ *   dense_m_c  128 or 256.  The tile height follows from the work: a pair
+ *         of CTAs computes 256 rows together (128 in each, sharing every
+ *         staged B slab) whenever there are at least two 128-row tiles and
+ *         two CTAs, else one CTA computes 128.
  * A field <= 0 means "library chooses" (except in ROSKO_SCHED_FORCED, where
  * the sparse fields must be set and dense fields <= 0 still mean default).
  */
@@ -187,13 +189,14 @@ rosko_status rosko_pack_transposed(const void* A_dev, rosko_dtype a_dtype, int64
  * released in stream order).  The FP32 (dequantised) INT8 result stays on
  * the CUDA-core path.
  * Stream order: when C must be zero-filled first (tiles or rows cut along K
- * and added), the fill is a small kernel ahead of a tensor-core launch, else
- * a memset.  The tensor-core kernel is launched as a programmatic dependent
- * of that fill (it reads A and B at once and writes C only after the fill),
- * and the row-direct kernel as a programmatic dependent of whatever kernel
- * precedes it on `stream` (it reads nothing before that kernel has
- * completed).  Both keep ordinary stream-order semantics for the caller;
- * they only let the launch overlap its predecessor's tail.
+ * and added), the fill is a small kernel ahead of a tensor-core launch (of
+ * the cut tiles only, unless the sparse part adds too), else a memset.  Every
+ * kernel of the call is launched as a programmatic dependent of whatever
+ * kernel precedes it on `stream`: it is scheduled while that one ends and
+ * reads and writes nothing before it has completed (the tensor-core kernel
+ * after a fill reads A and B while the fill runs and writes C after it).
+ * This keeps ordinary stream-order semantics for the caller; it only takes
+ * the launch latency out of the gap between two kernels.
  * The row-direct traversal numbers its work items (row pieces x column
  * strips of n_r columns) with 31 bits; beyond that it returns
  * ROSKO_ERR_UNSUPPORTED.
@@ -229,9 +232,9 @@ rosko_status rosko_spmm_plan(rosko_packed_t A, const void* B_dev, rosko_dtype b_
 /*
  * rosko_spmm_batched - C_i = A_i . B_i (or C_i += ...) for `count` <= 64
  * independent problems (pruned layers of different shapes).  The dense-panel
- * tiles of all problems run in one persistent tensor-core launch per CTA-tile
- * shape (at most four: 128 or 256 columns x 128 or 256 rows, each problem
- * taking the shape its tile or the analytic rule gives it), whose work list
+ * tiles of all problems run in one persistent tensor-core launch per tile
+ * width (128 or 256 columns, each problem taking the width its tile or the
+ * analytic rule gives it), whose work list
  * (per-problem TMA descriptors and sizes) is passed in the kernel
  * parameters; the row-direct sparse remainders share one launch, other
  * remainders run one launch per problem.  Per-problem arrays: A, B (device),

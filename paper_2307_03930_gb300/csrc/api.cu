@@ -157,15 +157,18 @@ CUresult encode_tiled(CUtensorMap* map, CUtensorMapDataType dt, cuuint32_t rank,
   return g_encode(map, dt, rank, gaddr, dims, strides, box, estrides, il, sw, l2, oob);
 }
 
-// Tensor-core dense-panel tiles (measured on GB300, stream-K kernel):
+// Tensor-core dense-panel tiles (the kernel runs them on CTA pairs, 256 rows
+// at a time, as soon as there are two row tiles):
 //  * K of fewer than 16 slabs (K < 1024): cutting tiles along K buys little
-//    and costs a zero fill of C and reduce-adds, so every tile is owned whole
-//    by one CTA (one per tile, or one per SM walking several); 128-wide
-//    tiles give more of them;
-//  * otherwise 256 columns per tile (half the L2 -> SM traffic of A against
-//    128) and either 256 rows when each CTA gets enough K work, or 128 rows
-//    with one tile per CTA when the tiles nearly fill the GPU, or 128 rows
-//    with the (tile, slab) units shared by one CTA per SM (stream-K).
+//    and costs a zero fill of C and reduce-adds, so every tile is owned whole;
+//    128-wide tiles give more of them;
+//  * otherwise 256 columns per tile (a pair's 256 x 256 tile moves 64 bytes
+//    per tensor-pipe cycle into each SM, a 256 x 128 tile 96, more than the
+//    ~70 that the L2 -> SM path sustains), on one whole tile per pair when
+//    the tiles nearly fill the GPU (2048^3: 16.4 against 22.3 us cut over
+//    every SM), else with the (tile, slab) units shared by one CTA per SM.
+// *mc_out is the rule's own 256 / 128 figure (enough K work per CTA for 256
+// rows of accumulator in one CTA); it no longer changes the launch.
 void dense_config(int64_t n_tiles, int64_t N, int64_t K, int sms, int* TN_out, int* ctas_out,
                   int* mc_out, bool chunked) {
   const int64_t slabs = (K + 63) / 64;
@@ -180,15 +183,6 @@ void dense_config(int64_t n_tiles, int64_t N, int64_t K, int sms, int* TN_out, i
   }
   *TN_out = N > 128 ? 256 : 128;
   const int64_t ntn = (N + *TN_out - 1) / *TN_out;
-  // 256-row tiles (two MMAs per B stage: a third less L2 -> SM traffic per
-  // flop, eight MMAs per ring step) hold their accumulator in all of TMEM,
-  // so the 256 KB epilogue of a CTA (~28 B/clk per SM through the TMA store
-  // path) overlaps no MMAs.  They pay when each CTA has enough K work to
-  // amortise it: ~20 double slabs or more (1024x4096x4096: 33.7 against
-  // 37.5 us; 512x4608x3136, 12 per CTA: 26.9 against 23.0 us).
-  // (INT8 codes drain the accumulator every 1,024 K: that needs the second
-  // TMEM set to overlap the drains, so their tiles stay 128 rows high;
-  // 11008x4096x2048 at 90 %: 205 against 268 us)
   const int64_t pair_units = (n_tiles + 1) / 2 * ntn * slabs;
   if (!chunked && pair_units >= 20LL * sms) {
     *mc_out = 256;
@@ -196,9 +190,7 @@ void dense_config(int64_t n_tiles, int64_t N, int64_t K, int sms, int* TN_out, i
     return;
   }
   *mc_out = 128;
-  // one whole tile per CTA when the tiles nearly fill the GPU (no K split:
-  // no zero fill of C, no reductions, a store epilogue; 2048^3: 21.4 against
-  // 23.7 us), else stream-K over every SM
+  // one whole tile per pair: no zero fill of C, no reductions, a store epilogue
   const int64_t tiles = n_tiles * ntn;
   *ctas_out = (4 * tiles >= 3 * (int64_t)sms && tiles <= sms) ? (int)tiles : sms;
 }
@@ -603,11 +595,11 @@ rosko_status spmm_run(rosko_packed_s* A, const void* B_dev, rosko_dtype b_dtype,
       return ROSKO_ERR_UNSUPPORTED;
   }
   // (INT8 tensor-core tiles add every K chunk into C)
-  const bool zero_c =
-      !accumulate && ((n_sparse > 0 && (L.split > 1 || direct_cut)) ||
-                      (!skip_dense && n_dense > 0 &&
-                       (p == ROSKO_I8 || dense_needs_zero(n_dense, N, A->K, t.dense_n_r,
-                                                          t.dense_split_k, t.dense_m_c / 128))));
+  const bool zero_sparse = !accumulate && n_sparse > 0 && (L.split > 1 || direct_cut);
+  const bool zero_dense =
+      !accumulate && !skip_dense && n_dense > 0 &&
+      (p == ROSKO_I8 || dense_needs_zero(n_dense, N, A->K, t.dense_n_r, t.dense_split_k));
+  const bool zero_c = zero_sparse || zero_dense;
   if (flags & kRunPlanOnly) {
     // report the split and the resolved schedule, launch nothing
     rosko_plan* out = g_plan_out;
@@ -633,16 +625,16 @@ rosko_status spmm_run(rosko_packed_s* A, const void* B_dev, rosko_dtype b_dtype,
           cudaSuccess)
     return ROSKO_ERR_CUDA;
   if (run_dense) {
-    const ZeroFill* z = fill ? &zf : nullptr;
+    // BF16 without a sparse part that adds: only the cut tiles are zeroed
+    const bool cut_only = fill && !zero_sparse && p == ROSKO_BF16;
+    const ZeroFill* z = fill && !cut_only ? &zf : nullptr;
     rosko_status s =
         p == ROSKO_I8
             ? dense_spmm_i8_launch(A, n_dense, static_cast<const int8_t*>(B_dev), N, ldb,
                                    static_cast<int32_t*>(C_dev), ldc, t.dense_n_r,
-                                   t.dense_split_k, t.dense_m_c / 128, z, st)
-            : dense_spmm_launch(A->dense_A, A->n_copy * 128, A->Kpad, A->tile_order_dev, n_dense,
-                                A->K, B_dev, N, ldb, static_cast<float*>(C_dev), ldc, A->M,
-                                accumulate, t.dense_n_r, t.dense_split_k, t.dense_m_c / 128,
-                                zero_c, z, st);
+                                   t.dense_split_k, z, st)
+            : dense_spmm_launch(A, n_dense, B_dev, N, ldb, static_cast<float*>(C_dev), ldc,
+                                accumulate, t.dense_n_r, t.dense_split_k, cut_only, z, st);
     if (s != ROSKO_OK) return s;
   }
   if (L.order == 3) {
@@ -688,9 +680,11 @@ rosko_status spmm_batched_impl(int32_t count, rosko_packed_s* const* A, const vo
   std::vector<char> active((size_t)count, 0), dense_any((size_t)count, 0);
   std::vector<char> direct_cut((size_t)count, 0);
   rest.resize((size_t)count);
-  // dense tiles run in one launch per CTA-tile shape (TN x 128 MH): each
-  // problem takes the shape the analytic rule (or its tile) gives it
-  std::vector<int> job_tn, job_mh;
+  // dense tiles run in one launch per tile width: each problem takes the
+  // width the analytic rule (or its tile) gives it; a launch runs on CTA pairs
+  // as soon as one of its problems has two row tiles
+  std::vector<int> job_tn;
+  int group_cg[2] = {1, 1};
   for (int32_t i = 0; i < count; ++i) {
     bool done = false;
     rosko_status v = spmm_validate(A[i], B[i], b_dt, N[i], ldb[i], nullptr, C[i], c_dt, ldc[i],
@@ -732,7 +726,7 @@ rosko_status spmm_batched_impl(int32_t count, rosko_packed_s* const* A, const vo
       jobs.push_back(j);
       job_of.push_back(i);
       job_tn.push_back(tn);
-      job_mh.push_back(mc / 128);
+      group_cg[tn / 256] = std::max(group_cg[tn / 256], dense_group(nd));
       dense_any[(size_t)i] = 1;
     }
     // the sparse remainder keeps this problem's tile; spmm_run recomputes the
@@ -759,18 +753,18 @@ rosko_status spmm_batched_impl(int32_t count, rosko_packed_s* const* A, const vo
   std::vector<char> zeroed((size_t)count, 0);
   if (!accumulate) {
     std::vector<char> need((size_t)count, 0);
-    for (int g = 0; g < 4; ++g) {
-      const int tn = (g & 1) ? 256 : 128, mh = (g & 2) ? 2 : 1;
+    for (int g = 0; g < 2; ++g) {
+      const int tn = g ? 256 : 128;
       std::vector<DenseJob> gj;
       std::vector<int> gi;
       for (size_t k = 0; k < jobs.size(); ++k)
-        if (job_tn[k] == tn && job_mh[k] == mh) {
+        if (job_tn[k] == tn) {
           gj.push_back(jobs[k]);
           gi.push_back(job_of[k]);
         }
       if (gj.empty()) continue;
       std::unique_ptr<bool[]> nj(new bool[gj.size()]);
-      dense_batch_needs_zero(gj.data(), (int)gj.size(), tn, sms, mh, nj.get());
+      dense_batch_needs_zero(gj.data(), (int)gj.size(), tn, group_cg[g], nj.get());
       for (size_t k = 0; k < gj.size(); ++k)
         if (nj[k]) need[(size_t)gi[k]] = 1;
     }
@@ -786,13 +780,13 @@ rosko_status spmm_batched_impl(int32_t count, rosko_packed_s* const* A, const vo
       zeroed[(size_t)i] = 1;
     }
   }
-  for (int g = 0; g < 4; ++g) {
-    const int tn = (g & 1) ? 256 : 128, mh = (g & 2) ? 2 : 1;
+  for (int g = 0; g < 2; ++g) {
+    const int tn = g ? 256 : 128;
     std::vector<DenseJob> gj;
     for (size_t k = 0; k < jobs.size(); ++k)
-      if (job_tn[k] == tn && job_mh[k] == mh) gj.push_back(jobs[k]);
+      if (job_tn[k] == tn) gj.push_back(jobs[k]);
     if (gj.empty()) continue;
-    rosko_status s = dense_batch_launch(gj.data(), (int)gj.size(), tn, sms, mh, st);
+    rosko_status s = dense_batch_launch(gj.data(), (int)gj.size(), tn, group_cg[g], st);
     if (s != ROSKO_OK) return s;
   }
   // sparse remainders (the dense tiles were launched above): the row-direct

@@ -183,12 +183,12 @@ bool sparse_config_supported(rosko_dtype p_dt, rosko_dtype b_dt, rosko_dtype c_d
 int sparse_default_V(rosko_dtype p_dt, int R, int order);
 
 // spmm_dense_tc.cu
-rosko_status dense_spmm_launch(const void* dense_A, int64_t dense_rows, int64_t Kpad,
-                               const int32_t* tile_order_dev, int64_t n_tiles, int64_t K,
-                               const void* B, int64_t N, int64_t ldb, float* C, int64_t ldc,
-                               int64_t M, int accumulate, int TN, int ctas, int MH,
-                               bool c_zeroed, const ZeroFill* zf,
-                               cudaStream_t st);
+// The first n_tiles dense copies of h times B.  ctas: CTAs to use at most
+// (<= 0: one per SM).  zf: zero-fill all of C first; zero_cut: only the tiles
+// that the split cuts (dense_needs_zero).
+rosko_status dense_spmm_launch(const rosko_packed_s* h, int64_t n_tiles, const void* B, int64_t N,
+                               int64_t ldb, float* C, int64_t ldc, int accumulate, int TN,
+                               int ctas, bool zero_cut, const ZeroFill* zf, cudaStream_t st);
 // One row-direct (order 4) sparse SpMM of a batch: the panels of h listed in
 // panel_list (NULL: all rows), B and C of this problem.
 struct DirectJob {
@@ -218,8 +218,7 @@ int direct_pick(const rosko_packed_s* h, const int32_t* panel_list, int64_t n_pa
 // One launch over all jobs (count <= 64, same handle / B / C types, V
 // columns per lane); C of jobs with cut rows must be zeroed by the caller
 // unless they accumulate.
-rosko_status direct_batch_launch(const DirectJob* jobs, int count, int V, cudaStream_t st,
-                                 bool pdl = false);
+rosko_status direct_batch_launch(const DirectJob* jobs, int count, int V, cudaStream_t st);
 // One dense-panel SpMM of a batch (see dense_batch_launch).
 struct DenseJob {
   const void* dense_A;
@@ -233,7 +232,6 @@ struct DenseJob {
   int accumulate;
   int kchunk = 0;    // K slabs per exact-integer chunk (INT8 codes), 0: none
   int out_i32 = 0;   // C is INT32 (INT8 codes through the BF16 pipe)
-  int pdl = 0;       // launch as a programmatic dependent of the previous kernel
 };
 // INT8 x INT8 -> INT32 through the BF16 tensor pipe: B is converted to BF16
 // (exact) in stream-ordered scratch, the handle's dense copies hold the INT8
@@ -241,18 +239,16 @@ struct DenseJob {
 // and added into C, which the caller has zeroed unless it accumulates.
 rosko_status dense_spmm_i8_launch(const rosko_packed_s* h, int64_t n_tiles, const int8_t* B,
                                   int64_t N, int64_t ldb, int32_t* C, int64_t ldc, int TN,
-                                  int ctas, int MH, const ZeroFill* zf, cudaStream_t st);
-// One persistent stream-K launch over all jobs' dense tiles (count <= 64);
-// C of jobs whose tiles the split cuts must be zeroed by the caller unless
-// they accumulate (dense_batch_needs_zero).
-rosko_status dense_batch_launch(const DenseJob* jobs, int count, int TN, int ctas, int MH,
-                                cudaStream_t st);
-void dense_batch_needs_zero(const DenseJob* jobs, int count, int TN, int ctas, int MH,
-                            bool* out);
-// stream-K grid size and whether some dense tile is split between CTAs
-// (MH = 128-row halves per CTA tile: 1 or 2)
-int64_t dense_grid(int64_t n_tiles, int64_t N, int64_t K, int TN, int ctas, int MH);
-bool dense_needs_zero(int64_t n_tiles, int64_t N, int64_t K, int TN, int ctas, int MH);
+                                  int ctas, const ZeroFill* zf, cudaStream_t st);
+// One persistent launch over all jobs' dense tiles (count <= 64) by workers of
+// cg CTAs; C of jobs whose tiles the split cuts must be zeroed by the caller
+// unless they accumulate (dense_batch_needs_zero).
+rosko_status dense_batch_launch(const DenseJob* jobs, int count, int TN, int cg, cudaStream_t st);
+void dense_batch_needs_zero(const DenseJob* jobs, int count, int TN, int cg, bool* out);
+// CTAs per worker (1 or 2) of a launch over n_tiles row tiles, and whether its
+// split over `ctas` CTAs cuts a tile
+int dense_group(int64_t n_tiles);
+bool dense_needs_zero(int64_t n_tiles, int64_t N, int64_t K, int TN, int ctas);
 
 // api.cu
 rosko_status spmm_validate(rosko_packed_s* A, const void* B_dev, rosko_dtype b_dtype, int64_t N,

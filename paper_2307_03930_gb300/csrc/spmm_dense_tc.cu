@@ -2,34 +2,49 @@
 //
 // Row tiles of A (128 rows = several packed panels) whose density is high
 // enough that a dense contraction beats row skipping on CUDA cores are kept
-// as dense BF16 copies.  For such a tile the whole K-first schedule of
-// Sec. 4.2 runs on the tensor core: the 128 x TN C tile lives in tensor memory
-// (TMEM) for the full K range, K slabs of A (128 x 64, K-major) and B
-// (64 x TN, N-major: B is row-major K x N) stream through a ring of shared
-// memory stages filled by TMA, one elected thread issues tcgen05.mma
-// (M = 128, N = TN, K = 16 per instruction) and C is written once.
+// as dense BF16 copies.  For such tiles the whole K-first schedule of
+// Sec. 4.2 runs on the tensor core: the C tile lives in tensor memory (TMEM)
+// for the full K range, K slabs of A (128 x 64, K-major) and B (64 x TN,
+// N-major: B is row-major K x N) stream through a ring of shared memory
+// stages filled by TMA, one elected thread issues tcgen05.mma (K = 16 per
+// instruction) and C is written once.
+//
+// Workers.  A worker is a pair of CTAs on two neighbouring SMs (CG = 2,
+// cta_group::2) whenever the work has at least two row tiles, else one CTA
+// (CG = 1).  A pair computes a 256 x TN tile of C: each CTA loads its own 128
+// rows of A and half of B's columns, the MMA (M = 256, N = TN) reads both
+// halves of B from the two shared memories, and each CTA's TMEM receives its
+// own 128 x TN half of C.  What bounds this kernel is feeding the tensor
+// pipe: a 128 x 256 x 64 slab takes 512 cycles of it; one CTA alone has to
+// write 48 KB into shared memory and read 48 KB of operands in that time
+// (96 + 96 bytes per cycle of 128), a CTA of a pair 32 KB (64 + 64), and the
+// L2 -> SM traffic falls by the same third.  The smaller stages also make the
+// ring six slabs deep instead of four.
 //
 // Warp roles: 0 = TMA producer, 1 = MMA issuer (and TMEM owner), 2.. =
-// epilogue (warp w reads TMEM lanes 32 (w % 4) .. 32 (w % 4) + 31; with 8
-// epilogue warps two share a lane quarter and split its columns).  The
-// producer and MMA warps wait as whole warps (converged) and one lane
-// issues.  Each ring step costs such a warp a few hundred cycles (measured:
-// a wait on a completed mbarrier, an arrive or a commit, and the wake-up of
-// the other side), about the 512 tensor-pipe cycles of the four MMAs of a
-// 128-row K slab, so with 128-row tiles both warps move two stages per step
-// (the producer's two lanes issue their stages' copies side by side).
+// epilogue (warp w reads TMEM lanes 32 (w % 4) .. 32 (w % 4) + 31).  The
+// producer and MMA warps wait as whole warps and one elected lane issues
+// (elect.sync, see elect_one: with a plain `lane == 0` branch a slab's four
+// MMAs took 640-670 cycles to issue, more than the 512 that the pipe needs;
+// elected, the loop runs at 508, and 11008x4096x2048 went from 115 to 96 us).
+// In a pair both CTAs run a producer (their copies complete on the even CTA's
+// barrier) and an epilogue; the even CTA's MMA warp issues for both and its
+// commits arrive on both CTAs' barriers.
 //
-// Schedule: persistent stream-K.  The (tile, K slab) units of all dense tiles
-// are cut into one equal contiguous share per SM, so small-M problems (few
-// row tiles) still fill every SM in one wave.  A share covers the K ranges of
-// one or two tiles; two TMEM accumulators alternate so that the epilogue of
-// one range overlaps the MMAs of the next.  A tile whose K range is cut
-// between CTAs is added into C; a tile owned whole is stored.  C is then
-// zero-filled by a small kernel launched just before this one, of which this
-// launch is a programmatic dependent: the ring fills and MMAs start at once
-// and only the epilogue waits (griddepcontrol.wait) for the fill, which thus
-// runs under the MMAs.  The first ring fill is issued by thread 0 before the
-// TMEM allocation and the block barrier, overlapping its cold DRAM latency.
+// Schedule.  Workers are persistent.  A single problem with at least as many
+// tiles as workers gives each worker one whole tile per round, in an order
+// that keeps the tiles of a round a compact block of C (8 column tiles wide),
+// so that a round reads few distinct slabs of A and B; what is left (fewer
+// tiles than workers, or the whole of a batch) is cut into one equal
+// contiguous share per worker along (tile, K slab), so every worker finishes
+// together and layers with few row tiles still fill the GPU.  A share's ends
+// snap to the tile boundary when it is closer than kMinPiece slabs.  A tile
+// whose K range is cut is added into C by its pieces; only those tiles are
+// zero-filled first, by a small kernel of which this launch is a programmatic
+// dependent: the ring fills and MMAs start at once and only the epilogue
+// waits (griddepcontrol.wait), so the fill runs under the MMAs.  Every other
+// tile is stored.  Two TMEM accumulators alternate so that the epilogue of
+// one range overlaps the MMAs of the next.
 //
 // Epilogue: each epilogue warp moves its 32 TMEM lanes (C rows) 32 columns
 // at a time into a 32 x 32 FP32 staging tile in shared memory (128-byte
@@ -49,33 +64,59 @@
 namespace rosko {
 namespace {
 
-constexpr int kTM = 128;             // rows of a dense tile (MMA M)
+constexpr int kTM = 128;             // rows of a dense tile
 constexpr int kTK = 64;              // K per stage: 64 BF16 = one 128-byte swizzle row
 constexpr uint32_t kABytes = kTM * kTK * 2;   // 16 KB
 constexpr uint32_t kStageC = 32 * 32 * 4;      // one 32 x 32 FP32 staging tile
-// Epilogue warps: 4 (one per TMEM lane quarter, two staging tiles each) or
-// 8 (two per quarter, each writing half of the columns, one staging tile
-// each); the staging space is the same 32 KB either way.  Measured on GB300
-// the two run the epilogue in the same time (it is bound by the TMA stores
-// and L2 reductions, not by the warps), so the smaller block is kept.
+// Epilogue warps: 4 (one per TMEM lane quarter), two staging tiles each.
+// Eight warps ran the epilogue in the same time (it is bound by the TMA
+// stores and L2 reductions, ~28 bytes per cycle per SM, not by the warps).
 constexpr int kEpiWarps = 4;
-constexpr int kStagePerWarp = 8 / kEpiWarps;
-constexpr uint32_t kEpiBytes = 8 * kStageC;
+constexpr int kStagePerWarp = 2;
+constexpr uint32_t kEpiBytes = kEpiWarps * kStagePerWarp * kStageC;
 constexpr int kThreads = 64 + 32 * kEpiWarps;
+// A tile's cost in K slabs is at least its epilogue's time (128 KB per
+// 128 x 256 accumulator at ~28 B/clk: about nine slabs of 512 cycles; the
+// same ratio for 128-column tiles).
+constexpr int kEpiCost = 9;
+// Stream-K pieces shorter than this many K slabs cost more in reductions
+// (every piece adds its partial tile into C) than they gain in balance.
+constexpr int kMinPiece = 8;
+// Column tiles of a round's block (see the schedule above).
+constexpr int kGroupN = 8;
 
 // One problem of the batch (a single SpMM is a batch of one).
 struct DenseProb {
   const int32_t* tile_order;  // dense copy c holds rows tile_order[c]*128 ...
   float* C;
-  int64_t ldc, M, N;
-  int64_t unit0;     // first unit of this problem in the batch's unit space
+  int64_t ldc;
+  int M, N;
   int n_copy;        // 128-row tiles (dense copies) in the work
-  int n_ntiles;      // TN-wide column tiles
+  int mtiles;        // worker tiles: ceil(n_copy / CG) rows of them
+  int ntn;           // TN-wide column tiles
+  int tiles;         // mtiles * ntn
   int slabs;         // K slabs of 64 per tile
-  int accumulate, vec_ok;
+  int cost;          // max(slabs, kEpiCost)
+  int cost0;         // first cost unit of this problem in the shared space
+  int accumulate;
   int tma_c;         // C tensor map usable (16-byte aligned rows)
   int b3d;           // B tensor map is 3-D (64 columns x K x N / 64 chunks)
 };
+
+// The split of the work between the workers.  Rounds of whole tiles (one
+// problem only): tile r * workers + w for r < rounds; then the tiles from
+// tile0 on, cut along the cost space [0, units).
+// cut = 0: every share ends on a tile boundary (a batch with at least two
+// tiles per worker: its problems would otherwise be zero-filled whole).
+struct DenseSplit {
+  int count, workers, rounds, tile0, units, cut;
+};
+
+// A position in the cut part of the work: problem, tile in it, K slab.
+struct DensePos {
+  int q, tile, slab;
+};
+constexpr int kMaxWorkers = 160;   // persistent: at most one per SM
 
 // The whole batch travels in the kernel parameters (no device allocation):
 // per problem its A and B tensor maps and its scalars.
@@ -85,111 +126,119 @@ struct DenseTable {
   CUtensorMap tmB[NP];
   CUtensorMap tmC[NP];   // FP32 C, 32 x 32 boxes, 128-byte swizzle
   DenseProb p[NP];
-  int count;
-  int64_t units;
-  int stages;
-  int aligned;   // CTA ranges start and end on tile boundaries (no tile is cut)
+  DenseSplit split;
+  // where each worker's share begins (computed on the host: the divisions
+  // cost a worker about a microsecond at its start)
+  DensePos start[kMaxWorkers + 1];
   // INT8 codes through the BF16 pipe: accumulator segments end every
   // `kchunk` K slabs (0: only at tile ends), so that every FP32 partial sum
   // stays an exact integer, and C is INT32 (partials converted and added)
   int kchunk;
   int out_i32;
+  // 1: the launch follows a zero fill of C that started after everything
+  // before it had completed, so A and B may be read at once
+  int early_ab;
   int* status;
 };
 
-// Stream-K split of the (tile, K slab) units: CTA b owns [b U / G, (b+1) U / G).
-// U < 2^31 and b <= G < 2^16 (checked on the host), so floor(U b / G) is
-// (U / G) b + ((U % G) b) / G in 32-bit unsigned divisions (a 64-bit
-// division is a long software sequence that every CTA would pay at start).
-__device__ __forceinline__ int64_t unit_begin(int64_t U, int64_t b, int64_t G) {
-  const uint32_t u = (uint32_t)U, g = (uint32_t)G, bb = (uint32_t)b;
-  const uint32_t q = u / g, r = u - q * g;
-  return (int64_t)q * bb + (int64_t)((r * bb) / g);
-}
-
-// Advance the problem index q (monotone in u) so that u belongs to problem q.
-template <int NP>
-__device__ __forceinline__ void advance_problem(const DenseTable<NP>& T, int64_t u, int& q) {
-  while (q + 1 < T.count && u >= T.p[q + 1].unit0) ++q;
-}
-
-// First tile boundary at or after unit x (tile = `slabs` consecutive units).
-template <int NP>
-__device__ __forceinline__ int64_t tile_boundary(const DenseTable<NP>& T, int64_t x) {
-  if (x >= T.units) return T.units;
+// Where worker b's share begins (b = workers: the end of the work).  The
+// cost space is divided evenly (U < 2^31 and b <= workers < 2^16, so
+// floor(U b / G) is (U / G) b + ((U % G) b) / G in 32-bit divisions); a cut
+// closer than kMinPiece slabs to a tile boundary moves onto it, as does every
+// cut of a tile whose cost is its epilogue.
+inline DensePos dense_pos(const DenseSplit& S, const DenseProb* p, int b) {
+  DensePos r = {S.count, 0, 0};
+  if (b >= S.workers) return r;
+  const uint32_t U = (uint32_t)S.units, G = (uint32_t)S.workers;
+  const uint32_t quo = U / G, rem = U - quo * G;
+  const uint32_t x = quo * (uint32_t)b + rem * (uint32_t)b / G;
+  if (x >= U) return r;
   int q = 0;
-  advance_problem(T, x, q);
-  const uint32_t slabs = (uint32_t)T.p[q].slabs;
-  const uint32_t r = (uint32_t)(x - T.p[q].unit0) % slabs;
-  return r ? x + (slabs - r) : x;
+  while (q + 1 < S.count && x >= (uint32_t)p[q + 1].cost0) ++q;
+  const uint32_t lx = x - (uint32_t)p[q].cost0, cost = (uint32_t)p[q].cost;
+  int tile = (int)(lx / cost);
+  int slab = (int)(lx - (uint32_t)tile * cost);
+  if (!S.cut || p[q].slabs != (int)cost) {
+    tile += 2 * slab >= (int)cost ? 1 : 0;
+    slab = 0;
+  } else if (slab < kMinPiece) {
+    slab = 0;
+  } else if ((int)cost - slab < kMinPiece) {
+    ++tile;
+    slab = 0;
+  }
+  tile += S.tile0;
+  if (tile >= p[q].tiles) {
+    ++q;
+    tile = 0;
+  }
+  r.q = q;
+  r.tile = tile;
+  r.slab = slab;
+  return r;
 }
 
-// Position of a unit inside the batch: problem q, row-tile group mt, column
-// tile nt, K slab (unit = (nt * mtiles + mt) * slabs + slab within problem q).
-// Set once per role with divisions, then advanced by increments only.
-struct Cursor {
-  int q, mt, nt, slab;
-  int mtiles, ntiles, slabs;
-  int b3d;   // problem q's B tensor map is 3-D (kept in a register: the
-             // parameter table is indexed by q, a run-time value)
+// Row and column of a worker tile: column groups of kGroupN tiles, inside a
+// group columns fastest.
+__host__ __device__ inline void dense_tile_at(const DenseProb& p, int tile, int* mt, int* nt) {
+  const int per = kGroupN * p.mtiles;
+  const int g = tile / per;
+  const int r = tile - g * per;
+  const int w = p.ntn - g * kGroupN < kGroupN ? p.ntn - g * kGroupN : kGroupN;
+  *mt = r / w;
+  *nt = g * kGroupN + (r - *mt * w);
+}
+
+// A worker's segments: the K slabs [s0, s1) of one tile each, in the same
+// order for its three roles.
+struct DenseSeg {
+  int q, mt, nt, s0, s1;
+  bool whole;
 };
-
-template <int NP, int MH>
-__device__ __forceinline__ void cursor_load(const DenseTable<NP>& T, Cursor& c) {
-  const DenseProb& P = T.p[c.q];
-  c.mtiles = (P.n_copy + MH - 1) / MH;
-  c.ntiles = P.n_ntiles;
-  c.slabs = P.slabs;
-  c.b3d = P.b3d;
-}
-
-template <int NP, int MH>
-__device__ __forceinline__ Cursor cursor_at(const DenseTable<NP>& T, int64_t u) {
-  Cursor c;
-  c.q = 0;
-  advance_problem(T, u, c.q);
-  cursor_load<NP, MH>(T, c);
-  const uint32_t lu = (uint32_t)(u - T.p[c.q].unit0);
-  const uint32_t tile = lu / (uint32_t)c.slabs;
-  c.slab = (int)(lu - tile * (uint32_t)c.slabs);
-  c.nt = (int)(tile / (uint32_t)c.mtiles);
-  c.mt = (int)(tile - (uint32_t)c.nt * (uint32_t)c.mtiles);
-  return c;
-}
-
-// Move to the first slab of the next tile (next problem after its last tile).
-template <int NP, int MH>
-__device__ __forceinline__ void cursor_next_tile(const DenseTable<NP>& T, Cursor& c) {
-  c.slab = 0;
-  if (++c.mt == c.mtiles) {
-    c.mt = 0;
-    if (++c.nt == c.ntiles) {
-      c.nt = 0;
-      if (c.q + 1 < T.count) {
+template <int NP>
+struct SegIter {
+  const DenseTable<NP>& T;
+  int worker, round;
+  DensePos c, e;
+  __device__ __forceinline__ SegIter(const DenseTable<NP>& t, int w)
+      : T(t), worker(w), round(0), c(t.start[w]), e(t.start[w + 1]) {}
+  __device__ __forceinline__ bool next(DenseSeg& s) {
+    int tile;
+    if (round < T.split.rounds) {
+      s.q = 0;
+      tile = round * T.split.workers + worker;
+      s.s0 = 0;
+      s.s1 = T.p[0].slabs;
+      ++round;
+    } else {
+      if (c.q > e.q || (c.q == e.q && (c.tile > e.tile || (c.tile == e.tile && c.slab >= e.slab))))
+        return false;
+      s.q = c.q;
+      tile = c.tile;
+      s.s0 = c.slab;
+      s.s1 = (c.q == e.q && c.tile == e.tile) ? e.slab : T.p[c.q].slabs;
+      c.slab = 0;
+      if (++c.tile == T.p[c.q].tiles) {
+        c.tile = 0;
         ++c.q;
-        cursor_load<NP, MH>(T, c);
       }
     }
+    dense_tile_at(T.p[s.q], tile, &s.mt, &s.nt);
+    s.whole = s.s0 == 0 && s.s1 == T.p[s.q].slabs;
+    return true;
   }
-}
+};
 
-template <int NP, int MH>
-__device__ __forceinline__ void cursor_next(const DenseTable<NP>& T, Cursor& c) {
-  if (++c.slab == c.slabs) cursor_next_tile<NP, MH>(T, c);
-}
-
-// MH = 128-row halves per CTA tile (1: 128 x TN, 2: 256 x TN sharing each B
-// stage between two MMAs, which halves B's shared-memory bytes per flop).
-template <int TN, int NP, int MH>
-__global__ void __launch_bounds__(kThreads, 1)
-    dense_panel_kernel(const __grid_constant__ DenseTable<NP> T) {
-  constexpr uint32_t kBBytes = (uint32_t)TN * kTK * 2;
-  constexpr uint32_t kStageBytes = MH * kABytes + kBBytes;
-  constexpr int NBUF = (MH * TN * 2 <= 512) ? 2 : 1;   // TMEM accumulator sets
+template <int TN, int NP, int CG>
+__global__ void __cluster_dims__(CG, 1, 1) __launch_bounds__(kThreads, 1)
+    dense_panel_kernel(const __grid_constant__ DenseTable<NP> T, int S) {
+  constexpr int BN = TN / CG;                             // B columns this CTA loads
+  constexpr uint32_t kBBytes = (uint32_t)BN * kTK * 2;
+  constexpr uint32_t kStageBytes = kABytes + kBBytes;
+  constexpr int NBUF = 2;                                 // TMEM accumulators
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  const int S = T.stages;
   uint8_t* stage_c = smem + (size_t)S * kStageBytes;   // 1024-aligned: stages are 1 KB multiples
   uint64_t* full = reinterpret_cast<uint64_t*>(stage_c + kEpiBytes);
   uint64_t* empty = full + S;
@@ -197,221 +246,185 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint64_t* acc_empty = acc_full + 2;  // [2] epilogue -> MMA: accumulator drained
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + 2);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  // one thread fills ring stage sj with unit cj: A (MH x 128 rows; rows past
-  // the last copy are zero-filled) and TN / 64 chunks of 64 B columns, one
-  // 3-D box when N is a multiple of 64 (x = column in chunk, y = k,
-  // z = chunk), else one 2-D box each
-  auto issue_stage = [&](const Cursor& cj, int sj) {
-    uint8_t* a_dst = smem + (size_t)sj * kStageBytes;
-    uint8_t* b_dst = a_dst + MH * kABytes;
-    const int k0 = cj.slab * kTK;
-    mbar_arrive_expect_tx(&full[sj], kStageBytes);
-    tma_load_2d(a_dst, &T.tmA[cj.q], k0, cj.mt * MH * kTM, &full[sj]);
-    if (cj.b3d) {
-      tma_load_3d(b_dst, &T.tmB[cj.q], 0, k0, cj.nt * (TN / 64), &full[sj]);
-    } else {
-#pragma unroll
-      for (int jj = 0; jj < TN / 64; ++jj)
-        tma_load_2d(b_dst + jj * (kTK * 128), &T.tmB[cj.q], cj.nt * TN + 64 * jj, k0, &full[sj]);
-    }
-  };
-  int64_t u0 = unit_begin(T.units, blockIdx.x, gridDim.x);
-  int64_t u1 = unit_begin(T.units, blockIdx.x + 1, gridDim.x);
-  if (T.aligned) {
-    // many tiles: whole tiles per CTA (no zero fill, no reductions into C)
-    u0 = tile_boundary(T, u0);
-    u1 = tile_boundary(T, u1);
-  }
-  if (u0 >= u1) return;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
+  const int rank = CG == 2 ? (int)cluster_rank() : 0;
+  const int worker = (int)blockIdx.x / CG;
+  // the next launch in the stream may be scheduled from now on (it waits for
+  // this grid in its own pdl_wait)
+  if (threadIdx.x == 0) pdl_trigger();
 
-  if (threadIdx.x == 32) {
-    // descriptor fetches overlap the barrier and TMEM set-up
-    int q0 = 0;
-    advance_problem(T, u0, q0);
-    prefetch_tensormap(&T.tmA[q0]);
-    prefetch_tensormap(&T.tmB[q0]);
-    if (T.p[q0].tma_c) prefetch_tensormap(&T.tmC[q0]);
+  // Set-up, overlapped per warp: the producer initialises the barriers and
+  // starts its copies as soon as both CTAs' barriers exist, while warp 1
+  // allocates TMEM (the epilogue's and MMA warps' barrier 1 hands it over).
+  // Launched as a programmatic dependent, all of it also overlaps the tail of
+  // the launch before it.
+  if (warp == 0) {
+    if (lane == 0) {
+      for (int s = 0; s < S; ++s) {
+        mbar_init(&full[s], 1);
+        mbar_init(&empty[s], 1);
+      }
+      for (int b = 0; b < 2; ++b) {
+        mbar_init(&acc_full[b], 1);
+        mbar_init(&acc_empty[b], CG * kEpiWarps);
+      }
+      fence_barrier_init();
+    }
+    __syncwarp();
   }
-  if (threadIdx.x == 0) {
-    for (int s = 0; s < S; ++s) {
-      mbar_init(&full[s], 1);
-      mbar_init(&empty[s], 1);
-    }
-    for (int b = 0; b < 2; ++b) {
-      mbar_init(&acc_full[b], 1);
-      mbar_init(&acc_empty[b], kEpiWarps);
-    }
-    fence_barrier_init();
-    // (a programmatic dependent only of a zero fill of C, whose start means
-    // that every launch before it has completed: A and B are final here)
-    // the first ring fill goes out now: its (cold, DRAM) latency overlaps
-    // the TMEM allocation and the block barrier
-    Cursor c = cursor_at<NP, MH>(T, u0);
-    for (int64_t u = u0; u < u1 && u < u0 + S; ++u) {
-      issue_stage(c, (int)(u - u0));
-      cursor_next<NP, MH>(T, c);
-    }
-  }
+  // the peer's copies and commits arrive on this CTA's barriers: both CTAs
+  // must have initialised theirs
+  if constexpr (CG == 2) cluster_arrive();
+  else __syncthreads();
   if (warp == 1) {
-    tc::tmem_alloc(tmem_slot, NBUF * MH * TN);
-    tc::tmem_relinquish();
+    tc::tmem_alloc<CG>(tmem_slot, NBUF * TN);
+    tc::tmem_relinquish<CG>();
+    tc::fence_before_sync();
   }
-  tc::fence_before_sync();
-  __syncthreads();
-  tc::fence_after_sync();
-  const uint32_t tmem = *tmem_slot;
+  SegIter<NP> it(T, worker);
+  DenseSeg sg;
+  if constexpr (CG == 2) cluster_wait();
+  uint32_t tmem = 0;
+  if (warp != 0) {
+    asm volatile("bar.sync 1, %0;" ::"n"(kThreads - 32) : "memory");
+    tc::fence_after_sync();
+    tmem = *tmem_slot;
+  }
 
   if (warp == 0) {
     // ---------------- TMA producer -----------------------------------------
-    // The whole warp walks the ring (waits are warp-wide, so the warp stays
-    // converged); lane 0 issues the copies.
-    // the first min(S, units) stages were filled at start
-    const int64_t pre = std::min<int64_t>(S, u1 - u0);
-    int64_t i = pre;
-    int st = (int)(pre % S);
-    uint32_t ph = pre == S ? 1u : 0u;   // ring stage and its phase parity
-    bool ok = true;
-    Cursor c = cursor_at<NP, MH>(T, u0 + pre < u1 ? u0 + pre : u0);
-    // two stages per iteration (the MMA warp takes them in pairs too): each
-    // ring step costs this warp a few hundred cycles
-    constexpr int kPair = MH == 1 ? 2 : 1;
-    for (int64_t u = u0 + pre; u < u1;) {
-      const int n = (kPair == 2 && u + 1 < u1) ? 2 : 1;
-      const int st2 = st + 1 == S ? 0 : st + 1;
-      const uint32_t ph2 = st + 1 == S ? ph ^ 1u : ph;
-      bool got = i < S || mbar_wait_bounded(&empty[st], ph ^ 1u, T.status);
-      if (n == 2 && i + 1 >= S) got = got && mbar_wait_bounded(&empty[st2], ph2 ^ 1u, T.status);
-      if (!__all_sync(0xffffffffu, got)) {
-        ok = false;
-        break;
-      }
-      // lane j fills stage j of the pair: the two stages' copies are issued
-      // by one instruction stream, side by side
-      Cursor c1 = c;
-      cursor_next<NP, MH>(T, c1);
-      if (lane < n) issue_stage(lane ? c1 : c, lane ? st2 : st);
-      // row tiles fastest: CTAs that run together share B in L2
-      if (n == 2) {
-        c = c1;
-        cursor_next<NP, MH>(T, c);
+    if (!T.early_ab) pdl_wait();   // A and B may be the previous launch's output
+    // One thread fills ring stage sj with K slab `slab` of a tile: A (this
+    // CTA's 128 rows; rows past the last copy are zero-filled) and its BN / 64
+    // chunks of 64 B columns, one 3-D box when N is a multiple of 64
+    // (x = column in chunk, y = k, z = chunk), else one 2-D box each.
+    const uint32_t full0 = CG == 2 ? cluster_addr(full, 0) : smem_u32(full);
+    auto issue_stage = [&](const DenseSeg& sg, bool b3d, int slab, int sj) {
+      uint8_t* a_dst = smem + (size_t)sj * kStageBytes;
+      uint8_t* b_dst = a_dst + kABytes;
+      const int k0 = slab * kTK;
+      const int arow = (sg.mt * CG + rank) * kTM;
+      const int bcol = sg.nt * TN + rank * BN;
+      if constexpr (CG == 2) {
+        // both CTAs' bytes are counted by the even CTA's barrier
+        const uint32_t bar = full0 + (uint32_t)sj * 8u;
+        if (rank == 0) mbar_arrive_expect_tx(&full[sj], 2 * kStageBytes);
+        tma_load_2d_pair(a_dst, &T.tmA[sg.q], k0, arow, bar);
+        if (b3d) {
+          tma_load_3d_pair(b_dst, &T.tmB[sg.q], 0, k0, bcol / 64, bar);
+        } else {
+#pragma unroll
+          for (int jj = 0; jj < BN / 64; ++jj)
+            tma_load_2d_pair(b_dst + jj * (kTK * 128), &T.tmB[sg.q], bcol + 64 * jj, k0, bar);
+        }
       } else {
-        c = c1;
+        mbar_arrive_expect_tx(&full[sj], kStageBytes);
+        tma_load_2d(a_dst, &T.tmA[sg.q], k0, arow, &full[sj]);
+        if (b3d) {
+          tma_load_3d(b_dst, &T.tmB[sg.q], 0, k0, bcol / 64, &full[sj]);
+        } else {
+#pragma unroll
+          for (int jj = 0; jj < BN / 64; ++jj)
+            tma_load_2d(b_dst + jj * (kTK * 128), &T.tmB[sg.q], bcol + 64 * jj, k0, &full[sj]);
+        }
       }
-      __syncwarp();
-      for (int j = 0; j < n; ++j) {
+    };
+    int st = 0;
+    uint32_t ph = 1;   // parity of the stage's last release (fresh: passes)
+    bool ok = true;
+    while (ok && it.next(sg)) {
+      const bool b3d = T.p[sg.q].b3d != 0;
+      for (int s = sg.s0; s < sg.s1; ++s) {
+        if (!__all_sync(0xffffffffu, mbar_wait_bounded(&empty[st], ph, T.status))) {
+          ok = false;
+          break;
+        }
+        if (elect_one()) issue_stage(sg, b3d, s, st);
+        __syncwarp();
         if (++st == S) {
           st = 0;
           ph ^= 1u;
         }
       }
-      u += n;
-      i += n;
     }
-    if (!ok && lane == 0) {
-      // consumers gave up: wait (bounded) for our copies in flight to land
-      for (int64_t j = (i > S ? i - S : 0); j < i; ++j)
-        mbar_wait_bounded(&full[j % S], (uint32_t)(j / S) & 1u, T.status);
+    // every copy has landed and every commit on this CTA's barriers has
+    // arrived once each stage is released (bounded; a stage that was never
+    // filled passes at once)
+    for (int j = 0; j < S; ++j) {
+      if (!mbar_wait_bounded(&empty[st], ph, T.status)) break;
+      if (++st == S) {
+        st = 0;
+        ph ^= 1u;
+      }
     }
+    __syncwarp();
   } else if (warp == 1) {
     // ---------------- MMA issuer --------------------------------------------
     // The warp waits together; lane 0 issues the MMAs and the commits.  The
-    // smem descriptors of stage 0 are built once; stage s, K step kk and
-    // half hh only move the start address (a 14-bit field in 16-byte units:
-    // shared memory is below 256 KB, so the sum never carries out of it).
-    constexpr uint32_t idesc = tc::idesc_bf16_f32(kTM, TN, false, true);
+    // smem descriptors of stage 0 are built once; stage s and K step kk only
+    // move the start address (a 14-bit field in 16-byte units: shared memory
+    // is below 256 KB, so the sum never carries out of it).
+    constexpr uint32_t idesc = tc::idesc_bf16_f32(CG * kTM, TN, false, true);
     const uint32_t sbase = smem_u32(smem);
     // A: K-major, 128-byte swizzle, 8-row groups 1024 B apart; a K step of
     // 16 BF16 is 32 bytes inside the swizzle row.  B: N-major (row k of B =
     // 128 bytes of 64 N values), 128-byte swizzle; 64-wide N chunks are
     // 64 rows x 128 B = 8 KB apart (LBO), 8-row K groups 1024 B apart (SBO);
     // a K step of 16 rows = 2 KB.
-    const uint64_t a_desc0 = tc::smem_desc(sbase, 16, 1024, 2);
-    const uint64_t b_desc0 = tc::smem_desc(sbase + MH * kABytes, kTK * 128, 1024, 2);
-    int seg = -1;
+    const uint64_t a_desc0 = tc::smem_desc(sbase, 16, 1024, 2) & ~uint64_t(0x3FFF);
+    const uint64_t b_desc0 = tc::smem_desc(sbase + kABytes, kTK * 128, 1024, 2) & ~uint64_t(0x3FFF);
     int st = 0;
     uint32_t ph = 0;
     bool ok = true;
-    Cursor c = cursor_at<NP, MH>(T, u0);
-    int bsel = NBUF - 1;      // accumulator set of the current segment
-    uint32_t bph = 1;         // its acc_empty parity (flips each reuse)
+    int b = NBUF - 1;          // accumulator of the current segment
+    uint32_t bph = 0;          // parity of its last release (fresh: passes)
     const int kc = T.kchunk;
-    // 128-row tiles: two K slabs per iteration when both belong to the same
-    // accumulator segment.  Every ring step (a wait on a full stage, a
-    // commit) costs this warp a few hundred cycles, about what the four MMAs
-    // of one 128-row slab take on the tensor pipe.  (A 256-row stage already
-    // holds eight MMAs; pairing its three stages would leave the ring too
-    // shallow to cover the commit -> producer -> consumer round trip.)
-    constexpr int kPair = MH == 1 ? 2 : 1;
-    auto seg_end_after = [&](int64_t uu, int sl) {
-      return (uu + 1 == u1) || sl + 1 == c.slabs || (kc && (sl + 1) % kc == 0);
-    };
-    for (int64_t u = u0; u < u1;) {
-      const int slab = c.slab;
-      const bool first = (u == u0) || slab == 0 || (kc && slab % kc == 0);
-      const bool end1 = seg_end_after(u, slab);
-      const int n = (end1 || kPair == 1) ? 1 : 2;   // slabs this iteration
-      const bool last = n == 1 ? end1 : seg_end_after(u + 1, slab + 1);
-      if (first) {
-        ++seg;
-        if (++bsel == NBUF) {
-          bsel = 0;
+    while (rank == 0 && ok && it.next(sg)) {
+      for (int c0 = sg.s0; ok && c0 < sg.s1;) {
+        // slabs [c0, c1) sum in one accumulator
+        const int c1 = kc ? min(sg.s1, (c0 / kc + 1) * kc) : sg.s1;
+        if (++b == NBUF) {
+          b = 0;
           bph ^= 1u;
         }
-        // the epilogue must have drained this accumulator (segment seg - NBUF)
-        if (seg >= NBUF &&
-            !__all_sync(0xffffffffu, mbar_wait_bounded(&acc_empty[bsel], bph ^ 1u, T.status))) {
+        // the epilogue (of both CTAs) must have drained this accumulator
+        if (!__all_sync(0xffffffffu, mbar_wait_bounded<CG == 2>(&acc_empty[b], bph, T.status))) {
           ok = false;
           break;
         }
         tc::fence_after_sync();
-      }
-      const int st2 = st + 1 == S ? 0 : st + 1;
-      const uint32_t ph2 = st + 1 == S ? ph ^ 1u : ph;
-      bool got = mbar_wait_bounded(&full[st], ph, T.status);
-      if (n == 2) got = got && mbar_wait_bounded(&full[st2], ph2, T.status);
-      if (!__all_sync(0xffffffffu, got)) {
-        ok = false;
-        break;
-      }
-      tc::fence_after_sync();
-      if (lane == 0) {
-        const uint32_t d_tmem = tmem + (uint32_t)(bsel * MH * TN);
-#pragma unroll
-        for (int j = 0; j < 2; ++j) {
-          if (j == n) break;
-          const int sj = j ? st2 : st;
-          const uint64_t so = (uint64_t)((sj * kStageBytes) >> 4);
-#pragma unroll
-          for (int kk = 0; kk < kTK / 16; ++kk) {
-            const uint64_t bd = b_desc0 + so + (uint64_t)((kk * 16 * 128) >> 4);
-#pragma unroll
-            for (int hh = 0; hh < MH; ++hh) {
-              const uint64_t ad = a_desc0 + so + (uint64_t)((hh * kABytes + kk * 32) >> 4);
-              tc::mma_bf16(d_tmem + hh * TN, ad, bd, idesc, (!first || j > 0 || kk > 0) ? 1u : 0u);
-            }
+        const uint32_t d_tmem = tmem + (uint32_t)(b * TN);
+        for (int s = c0; s < c1; ++s) {
+          if (!__all_sync(0xffffffffu, mbar_wait_bounded(&full[st], ph, T.status))) {
+            ok = false;
+            break;
           }
-          tc::mma_commit(&empty[sj]);               // stage free once these MMAs finish
+          tc::fence_after_sync();
+          if (elect_one()) {
+            const uint32_t sa = sbase + (uint32_t)st * kStageBytes;
+#pragma unroll
+            for (int kk = 0; kk < kTK / 16; ++kk) {
+              const uint64_t ad = a_desc0 | (uint64_t)((sa + kk * 32) >> 4);
+              const uint64_t bd = b_desc0 | (uint64_t)((sa + kABytes + kk * 16 * 128) >> 4);
+              tc::mma_bf16<CG>(d_tmem, ad, bd, idesc, (s > c0 || kk > 0) ? 1u : 0u);
+            }
+            tc::mma_commit<CG>(&empty[st]);                   // stage free once these finish
+            if (s + 1 == c1) tc::mma_commit<CG>(&acc_full[b]);   // accumulator complete
+          }
+          __syncwarp();
+          if (++st == S) {
+            st = 0;
+            ph ^= 1u;
+          }
         }
-        if (last) tc::mma_commit(&acc_full[bsel]);  // accumulator complete
+        c0 = c1;
       }
-      __syncwarp();
-      for (int j = 0; j < n; ++j) {
-        cursor_next<NP, MH>(T, c);
-        if (++st == S) {
-          st = 0;
-          ph ^= 1u;
-        }
-      }
-      u += n;
     }
     if (!ok && lane == 0) {
       // make the epilogue's waits end: release every accumulator it expects
-      for (int b = 0; b < NBUF; ++b) tc::mma_commit(&acc_full[b]);
+      for (int j = 0; j < NBUF; ++j) tc::mma_commit<CG>(&acc_full[j]);
     }
-    // every MMA is issued: the next launch in the stream may start its
-    // prologue during this CTA's epilogue
-    if (lane == 0) pdl_trigger();
+    __syncwarp();
   } else {
     // ---------------- epilogue: TMEM -> registers -> C -----------------------
     // C may still be being zero-filled by the kernel this launch depends on
@@ -419,55 +432,40 @@ __global__ void __launch_bounds__(kThreads, 1)
     // Without such a dependency the wait returns at once.
     pdl_wait();
     const int quarter = warp & 3;                  // TMEM lanes 32 quarter .. + 31
-    const int part = (warp - 2) >> 2;              // column part of this warp
-    constexpr int kParts = kEpiWarps / 4;
     uint8_t* my_stage = stage_c + (size_t)(warp - 2) * kStagePerWarp * kStageC;
+    const uint32_t drained = CG == 2 ? cluster_addr(acc_empty, 0) : 0u;
     int chunk = 0;   // staging tiles alternate per chunk
-    Cursor c = cursor_at<NP, MH>(T, u0);
     int b = NBUF - 1;
     uint32_t bph = 1;
-    // one iteration per segment: the slabs of one tile inside [u0, u1)
-    for (int64_t u = u0; u < u1;) {
-      const DenseProb& P = T.p[c.q];
-      const int q = c.q;
-      // the segment ends at the tile's end, the K chunk's end or the range's
-      const int seg_end = T.kchunk ? min(c.slabs, (c.slab / T.kchunk + 1) * T.kchunk) : c.slabs;
-      int64_t ue = u + (seg_end - c.slab);
-      if (ue > u1) ue = u1;
-      const bool whole = (c.slab == 0) && (ue - u == c.slabs);
-      const int mt = c.mt, nt = c.nt;
-      if (++b == NBUF) {
-        b = 0;
-        bph ^= 1u;
-      }
-      // the tiles' C rows, fetched while the MMAs run
-      int32_t trow[MH];
-#pragma unroll
-      for (int hh = 0; hh < MH; ++hh) {
-        const int copy = mt * MH + hh;
-        trow[hh] = copy < P.n_copy ? __ldg(&P.tile_order[copy]) : 0;
-      }
+    const int kc = T.kchunk, out_i32 = T.out_i32;
+    while (it.next(sg)) {
+      const DenseProb& P = T.p[sg.q];
+      const int q = sg.q;
+      const int copy = sg.mt * CG + rank;
+      // the tile's C rows, fetched while the MMAs run
+      const int trow = copy < P.n_copy ? __ldg(&P.tile_order[copy]) : 0;
       // the problem's scalars in registers for the chunk loop
       const int64_t PM = P.M, PN = P.N;
-      const int n_copy = P.n_copy, tma_c = P.tma_c, out_i32 = T.out_i32;
-      const bool add = !whole || P.accumulate;
-      const bool ok = __all_sync(0xffffffffu, mbar_wait_bounded(&acc_full[b], bph, T.status));
-      tc::fence_after_sync();
-      const int64_t n0 = (int64_t)nt * TN;
-#pragma unroll
-      for (int hh = 0; hh < MH; ++hh) {
-        const int copy = mt * MH + hh;
-        if (copy >= n_copy) break;   // warp-uniform
-        const int64_t row0 = (int64_t)trow[hh] * kTM + quarter * 32;
+      const int64_t row0 = (int64_t)trow * kTM + quarter * 32;
+      const bool rows_ok = copy < P.n_copy && row0 < PM;
+      const int tma_c = P.tma_c;
+      const bool add = !sg.whole || P.accumulate;
+      const int64_t n0 = (int64_t)sg.nt * TN;
+      for (int c0 = sg.s0; c0 < sg.s1; c0 = kc ? min(sg.s1, (c0 / kc + 1) * kc) : sg.s1) {
+        if (++b == NBUF) {
+          b = 0;
+          bph ^= 1u;
+        }
+        const bool ok = __all_sync(0xffffffffu, mbar_wait_bounded(&acc_full[b], bph, T.status));
+        tc::fence_after_sync();
 #pragma unroll 1
-        for (int cc = part * (TN / 32 / kParts); cc < (part + 1) * (TN / 32 / kParts); ++cc) {
-          uint32_t r[32];
-          tc::tmem_ld_32x32b_x32(tmem + ((uint32_t)(quarter * 32) << 16) +
-                                     (uint32_t)(b * MH * TN + hh * TN + cc * 32),
-                                 r);
-          tc::tmem_ld_wait();
+        for (int cc = 0; cc < TN / 32; ++cc) {
           const int64_t col0 = n0 + cc * 32;
-          if (!ok || row0 >= PM || col0 >= PN) continue;   // warp-uniform
+          if (!ok || !rows_ok || col0 >= PN) break;   // warp-uniform
+          uint32_t r[32];
+          tc::tmem_ld_32x32b_x32(
+              tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(b * TN + cc * 32), r);
+          tc::tmem_ld_wait();
           if (out_i32) {
             // an exact integer in FP32 (|partial| < 2^24): convert to INT32
 #pragma unroll
@@ -527,16 +525,16 @@ __global__ void __launch_bounds__(kThreads, 1)
               }
             }
           }
+          __syncwarp();
+        }
+        // accumulator drained: hand it back to the MMA issuer
+        tc::fence_before_sync();
+        __syncwarp();
+        if (lane == 0) {
+          if constexpr (CG == 2) mbar_arrive_cluster(drained + (uint32_t)b * 8u);
+          else mbar_arrive(&acc_empty[b]);
         }
       }
-      // accumulator drained: hand it back to the MMA issuer
-      tc::fence_before_sync();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&acc_empty[b]);
-      const int adv = (int)(ue - u);
-      u = ue;
-      if (c.slab + adv >= c.slabs) cursor_next_tile<NP, MH>(T, c);
-      else c.slab += adv;   // the next K chunk of the same tile
     }
     // the staging tiles must not be released (CTA exit) while TMA reads
     // them, and C must be complete when the kernel ends
@@ -544,57 +542,137 @@ __global__ void __launch_bounds__(kThreads, 1)
     __syncwarp();
   }
   tc::fence_before_sync();
-  __syncthreads();
-  tc::fence_after_sync();
-  if (warp == 1) tc::tmem_dealloc(tmem, NBUF * MH * TN);
+  // no CTA of a pair leaves (or frees TMEM) while the other may still signal
+  // its barriers or read its shared memory
+  if constexpr (CG == 2) cluster_sync_all();
+  else __syncthreads();
+  if (warp == 1) {
+    tc::fence_after_sync();
+    tc::tmem_dealloc<CG>(tmem, NBUF * TN);
+  }
 }
 
-template <int TN, int MH>
-size_t dense_smem_bytes(int stages) {
-  return 1024 + (size_t)stages * (MH * kABytes + (size_t)TN * kTK * 2) + kEpiBytes + 256;
+// Zero the C tiles that the split cuts (their pieces are added): block
+// (b - 1, part) looks at the start of worker b's share, and zeroes the tile
+// when that is the tile's first cut.  A programmatic dependent of the launch
+// before it that lets the tensor-core launch start once that one has
+// completed: its A and B are then final and only its writes of C wait.
+template <int NP>
+__global__ void __launch_bounds__(256)
+    dense_cut_fill_kernel(const __grid_constant__ DenseTable<NP> T, int CG, int TN) {
+  pdl_wait();
+  pdl_trigger();
+  const DensePos c = T.start[blockIdx.x + 1];
+  if (c.q >= T.split.count || c.slab == 0) return;
+  const DensePos prev = T.start[blockIdx.x];
+  if (prev.q == c.q && prev.tile == c.tile && prev.slab > 0) return;
+  const DenseProb& P = T.p[c.q];
+  if (P.accumulate) return;
+  int mt, nt;
+  dense_tile_at(P, c.tile, &mt, &nt);
+  const int64_t n0 = (int64_t)nt * TN;
+  const int64_t cols = P.N - n0 < TN ? P.N - n0 : TN;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const bool vec = P.tma_c && cols % 4 == 0;
+  for (int r = (int)blockIdx.y * 8 + warp; r < CG * kTM; r += (int)gridDim.y * 8) {
+    const int copy = mt * CG + r / kTM;
+    if (copy >= P.n_copy) continue;
+    const int64_t row = (int64_t)__ldg(&P.tile_order[copy]) * kTM + r % kTM;
+    if (row >= P.M) continue;
+    float* dst = P.C + row * P.ldc + n0;
+    if (vec) {
+      for (int64_t i = lane; i < cols / 4; i += 32)
+        reinterpret_cast<uint4*>(dst)[i] = make_uint4(0, 0, 0, 0);
+    } else {
+      for (int64_t i = lane; i < cols; i += 32) dst[i] = 0.0f;
+    }
+  }
 }
 
-template <int TN, int MH>
+template <int TN, int CG>
 constexpr int dense_stages() {
-  return (200 * 1024) / (MH * kABytes + TN * kTK * 2) > 6 ? 6
-                                                         : (200 * 1024) / (MH * kABytes + TN * kTK * 2);
+  constexpr int n = (200 * 1024) / ((int)kABytes + TN / CG * kTK * 2);
+  return n > 8 ? 8 : n;
+}
+
+template <int TN, int CG>
+size_t dense_smem_bytes() {
+  return 1024 + (size_t)dense_stages<TN, CG>() * (kABytes + (size_t)TN / CG * kTK * 2) + kEpiBytes +
+         256;
 }
 
 int64_t slabs_of(int64_t K) { return (K + kTK - 1) / kTK; }
 
-template <int TN, int NP, int MH>
-rosko_status launch_table(DenseTable<NP>& T, int64_t grid, bool pdl, cudaStream_t st) {
-  const size_t smem = dense_smem_bytes<TN, MH>(T.stages);
-  static size_t set = 0;
-  auto fn = dense_panel_kernel<TN, NP, MH>;
-  if (smem > set) {
+template <int TN, int NP, int CG>
+rosko_status launch_table(const DenseTable<NP>& T, cudaStream_t st) {
+  constexpr int stages = dense_stages<TN, CG>();
+  const size_t smem = dense_smem_bytes<TN, CG>();
+  static bool set = false;
+  auto fn = dense_panel_kernel<TN, NP, CG>;
+  if (!set) {
     if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
         cudaSuccess)
       return ROSKO_ERR_CUDA;
-    set = smem;
+    set = true;
   }
-  if (pdl) {
-    // starts while the preceding zero fill runs; its epilogue waits for it
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    if (cudaLaunchKernelEx(&cfg, fn, T) != cudaSuccess) return ROSKO_ERR_CUDA;
-  } else {
-    fn<<<(unsigned)grid, kThreads, smem, st>>>(T);
-  }
+  if (launch_dependent(fn, dim3((unsigned)(T.split.workers * CG)), dim3(kThreads), smem, st, T,
+                       stages) != cudaSuccess)
+    return ROSKO_ERR_CUDA;
   count_launches(1);
   return cudaGetLastError() == cudaSuccess ? ROSKO_OK : ROSKO_ERR_CUDA;
 }
 
-rosko_status encode_dense_maps(const DenseJob& j, int MH, CUtensorMap* mA, CUtensorMap* mB,
-                               CUtensorMap* mC, bool c_ok, int TN, bool* b3d) {
+// The scalars of the problems and the split over `ctas` CTAs in workers of
+// cg; false when the cost space does not fit 31 bits.
+bool plan_split(const DenseJob* jobs, int count, int TN, int ctas, int cg, DenseProb* p,
+                DenseSplit* S) {
+  int64_t units = 0, tiles = 0, slabs_all = 0;
+  int n = 0;
+  for (int i = 0; i < count; ++i) {
+    const DenseJob& j = jobs[i];
+    if (j.n_tiles <= 0 || j.N <= 0) continue;
+    DenseProb& P = p[n++];
+    P.n_copy = (int)j.n_tiles;
+    P.mtiles = (P.n_copy + cg - 1) / cg;
+    P.ntn = (int)((j.N + TN - 1) / TN);
+    P.slabs = (int)slabs_of(j.K);
+    P.cost = std::max(P.slabs, kEpiCost);
+    const int64_t t = (int64_t)P.mtiles * P.ntn;
+    if (units >= (int64_t(1) << 31) || t >= (int64_t(1) << 31)) return false;
+    P.tiles = (int)t;
+    P.cost0 = (int)units;
+    P.accumulate = j.accumulate;
+    units += t * P.cost;
+    tiles += t;
+    slabs_all += t * P.slabs;
+  }
+  if (units >= (int64_t(1) << 31)) return false;
+  S->count = n;
+  // persistent workers: one per SM (or pair of SMs) at most, and no share
+  // below kMinPiece slabs unless it is a tile of its own
+  int64_t G = std::max(1, std::min(std::min(ctas, num_sms()), kMaxWorkers) / cg);
+  G = std::min<int64_t>(G, std::max(tiles, slabs_all / kMinPiece));
+  G = std::max<int64_t>(G, 1);
+  S->workers = (int)G;
+  S->rounds = n == 1 ? (int)(tiles / G) : 0;
+  S->tile0 = (int)(S->rounds * G);
+  S->units = (int)(n == 1 ? (tiles - S->tile0) * p[0].cost : units);
+  S->cut = n == 1 || tiles < 2 * G ? 1 : 0;
+  return true;
+}
+
+// Which of the (active) problems has a tile cut by the split.
+void cut_problems(const DenseSplit& S, const DenseProb* p, std::vector<char>* cut) {
+  cut->assign((size_t)S.count, 0);
+  for (int b = 1; b < S.workers; ++b) {
+    const DensePos c = dense_pos(S, p, b);
+    if (c.q < S.count && c.slab > 0) (*cut)[(size_t)c.q] = 1;
+  }
+}
+
+// Tensor maps of one problem: A, B (bn = columns one CTA loads per slab), C.
+rosko_status encode_dense_maps(const DenseJob& j, CUtensorMap* mA, CUtensorMap* mB,
+                               CUtensorMap* mC, bool c_ok, int bn, bool* b3d) {
   if (c_ok) {
     const cuuint64_t dims[2] = {(cuuint64_t)j.N, (cuuint64_t)j.M};
     const cuuint64_t strides[1] = {(cuuint64_t)j.ldc * 4};
@@ -610,7 +688,7 @@ rosko_status encode_dense_maps(const DenseJob& j, int MH, CUtensorMap* mA, CUten
   {
     const cuuint64_t dims[2] = {(cuuint64_t)j.Kpad, (cuuint64_t)j.dense_rows};
     const cuuint64_t strides[1] = {(cuuint64_t)j.Kpad * 2};
-    const cuuint32_t box[2] = {(cuuint32_t)kTK, (cuuint32_t)(kTM * MH)};
+    const cuuint32_t box[2] = {(cuuint32_t)kTK, (cuuint32_t)kTM};
     const cuuint32_t es[2] = {1, 1};
     if (encode_tiled(mA, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(j.dense_A), dims,
                      strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
@@ -623,7 +701,7 @@ rosko_status encode_dense_maps(const DenseJob& j, int MH, CUtensorMap* mA, CUten
     // B viewed as [N / 64][K][64]: chunk z starts 128 bytes after chunk z-1
     const cuuint64_t dims[3] = {64, (cuuint64_t)j.K, (cuuint64_t)(j.N / 64)};
     const cuuint64_t strides[2] = {(cuuint64_t)j.ldb * 2, 128};
-    const cuuint32_t box[3] = {64, (cuuint32_t)kTK, (cuuint32_t)(TN / 64)};
+    const cuuint32_t box[3] = {64, (cuuint32_t)kTK, (cuuint32_t)(bn / 64)};
     const cuuint32_t es[3] = {1, 1, 1};
     *b3d = encode_tiled(mB, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(j.B), dims,
                         strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
@@ -644,37 +722,22 @@ rosko_status encode_dense_maps(const DenseJob& j, int MH, CUtensorMap* mA, CUten
   return ROSKO_OK;
 }
 
-// Tile-granular split when there are at least two tiles per CTA: the
-// stream-K balance is then not needed and uncut tiles need no zero fill of C
-// and no reductions.
-static bool use_aligned(int64_t tiles, int64_t G) { return tiles >= 2 * G; }
-
-// Stream-K pieces shorter than this many K slabs cost more in reductions
-// (every piece adds its partial tile into C) than they gain in balance.
-constexpr int64_t kMinUnitsPerCta = 8;
-
-// CTAs of a launch over `units` (tile, slab) units in `tiles` tiles: one per
-// SM at most, and no stream-K piece shorter than kMinUnitsPerCta slabs.
-static int64_t grid_for(int64_t units, int64_t tiles, int ctas) {
-  // (the kernel's 32-bit split arithmetic wants G < 2^16)
-  int64_t G = std::min<int64_t>(std::min(ctas, 65535), units);
-  if (!use_aligned(tiles, G)) G = std::min<int64_t>(G, std::max(tiles, units / kMinUnitsPerCta));
-  return std::max<int64_t>(1, G);
-}
-
-template <int TN, int NP, int MH>
-rosko_status run_jobs(const DenseJob* jobs, int count, int ctas, cudaStream_t st) {
+template <int TN, int NP, int CG>
+rosko_status run_jobs(const DenseJob* jobs, int count, int ctas, bool zero_cut, bool after_fill,
+                      cudaStream_t st) {
   static_assert(sizeof(DenseTable<NP>) <= 32 * 1024 - 256, "kernel parameter table too large");
   DenseTable<NP> T;
   std::memset(static_cast<void*>(&T), 0, sizeof(T));
-  int64_t units = 0;
+  if (!plan_split(jobs, count, TN, ctas, CG, T.p, &T.split)) return ROSKO_ERR_UNSUPPORTED;
+  if (T.split.count == 0) return ROSKO_OK;
   int n = 0;
   for (int i = 0; i < count; ++i) {
     const DenseJob& j = jobs[i];
     if (j.n_tiles <= 0 || j.N <= 0) continue;
     const bool c_ok = ((reinterpret_cast<uintptr_t>(j.C) % 16) == 0) && ((j.ldc * 4) % 16 == 0);
     bool b3d = false;
-    rosko_status s = encode_dense_maps(j, MH, &T.tmA[n], &T.tmB[n], &T.tmC[n], c_ok, TN, &b3d);
+    rosko_status s =
+        encode_dense_maps(j, &T.tmA[n], &T.tmB[n], &T.tmC[n], c_ok, TN / CG, &b3d);
     if (s != ROSKO_OK) return s;
     DenseProb& P = T.p[n];
     P.tma_c = c_ok ? 1 : 0;
@@ -682,114 +745,91 @@ rosko_status run_jobs(const DenseJob* jobs, int count, int ctas, cudaStream_t st
     P.tile_order = j.tile_order_dev;
     P.C = j.C;
     P.ldc = j.ldc;
-    P.M = j.M;
-    P.N = j.N;
-    P.unit0 = units;
-    P.n_copy = (int)j.n_tiles;
-    P.n_ntiles = (int)((j.N + TN - 1) / TN);
-    P.slabs = (int)slabs_of(j.K);
-    P.accumulate = j.accumulate;
-    P.vec_ok = ((reinterpret_cast<uintptr_t>(j.C) % 16) == 0) && ((j.ldc * 4) % 16 == 0);
-    units += (int64_t)((P.n_copy + MH - 1) / MH) * P.n_ntiles * P.slabs;
+    P.M = (int)j.M;
+    P.N = (int)j.N;
     ++n;
   }
-  if (n == 0) return ROSKO_OK;
-  // the kernel splits and walks units in 32-bit arithmetic
-  if (units >= (int64_t(1) << 31)) return ROSKO_ERR_UNSUPPORTED;
-  T.count = n;
-  T.units = units;
-  int64_t tiles = 0;
-  for (int i = 0; i < n; ++i) tiles += (int64_t)((T.p[i].n_copy + MH - 1) / MH) * T.p[i].n_ntiles;
-  const int64_t grid = grid_for(units, tiles, ctas);
-  T.aligned = use_aligned(tiles, grid) ? 1 : 0;
+  for (int b = 0; b <= T.split.workers; ++b) T.start[b] = dense_pos(T.split, T.p, b);
   T.kchunk = jobs[0].kchunk;
   T.out_i32 = jobs[0].out_i32;
-  T.stages = dense_stages<TN, MH>();
+  T.early_ab = zero_cut || after_fill ? 1 : 0;
   T.status = device_status_word();
   if (!T.status) return ROSKO_ERR_CUDA;
-  return launch_table<TN, NP, MH>(T, grid, jobs[0].pdl != 0, st);
+  if (zero_cut) {
+    const dim3 grid((unsigned)std::max(1, T.split.workers - 1), 8);
+    if (launch_dependent(dense_cut_fill_kernel<NP>, grid, dim3(256), 0, st, T, CG, TN) !=
+        cudaSuccess)
+      return ROSKO_ERR_CUDA;
+    count_launches(1);
+  }
+  return launch_table<TN, NP, CG>(T, st);
+}
+
+// CTAs per worker: pairs as soon as there are two row tiles to share and two
+// CTAs to run them (a pair over a single row tile would leave half of it idle).
+int group_of(int64_t n_tiles, int ctas) { return n_tiles >= 2 && ctas >= 2 ? 2 : 1; }
+
+template <int TN, int NP>
+rosko_status dispatch_group(const DenseJob* jobs, int count, int cg, int ctas, bool zero_cut,
+                            bool after_fill, cudaStream_t st) {
+  return cg == 2 ? run_jobs<TN, NP, 2>(jobs, count, ctas, zero_cut, after_fill, st)
+                 : run_jobs<TN, NP, 1>(jobs, count, ctas, zero_cut, after_fill, st);
+}
+
+rosko_status dispatch_jobs(const DenseJob* jobs, int count, int TN, int cg, int ctas,
+                           bool zero_cut, bool after_fill, cudaStream_t st) {
+  if (count <= 0) return ROSKO_OK;
+  if ((TN != 128 && TN != 256) || count > 64) return ROSKO_ERR_INVALID_ARG;
+  if (count == 1)
+    return TN == 256 ? dispatch_group<256, 1>(jobs, 1, cg, ctas, zero_cut, after_fill, st)
+                     : dispatch_group<128, 1>(jobs, 1, cg, ctas, zero_cut, after_fill, st);
+  return TN == 256 ? dispatch_group<256, 64>(jobs, count, cg, ctas, zero_cut, after_fill, st)
+                   : dispatch_group<128, 64>(jobs, count, cg, ctas, zero_cut, after_fill, st);
 }
 
 }  // namespace
 
-static int64_t job_units(int64_t n_tiles, int64_t N, int64_t K, int TN, int MH) {
-  return ((n_tiles + MH - 1) / MH) * ((N + TN - 1) / TN) * slabs_of(K);
-}
-
-int64_t dense_grid(int64_t n_tiles, int64_t N, int64_t K, int TN, int ctas, int MH) {
-  const int64_t units = job_units(n_tiles, N, K, TN, MH);
-  return grid_for(units, units / slabs_of(K), ctas);
-}
-
-// True when the stream-K split of `units` over `ctas` CTAs cuts some tile of
-// `slabs` units (those tiles are accumulated with atomics into a zeroed C).
-static bool split_cuts_tile(int64_t units_before, int64_t units, int64_t total, int64_t slabs,
-                            int64_t G) {
-  for (int64_t b = 0; b <= G; ++b) {
-    const int64_t u = total * b / G;
-    if (u <= units_before || u >= units_before + units) continue;
-    if ((u - units_before) % slabs != 0) return true;
-  }
-  return false;
-}
-
-bool dense_needs_zero(int64_t n_tiles, int64_t N, int64_t K, int TN, int ctas, int MH) {
-  const int64_t units = job_units(n_tiles, N, K, TN, MH);
-  const int64_t G = dense_grid(n_tiles, N, K, TN, ctas, MH);
-  if (use_aligned(units / slabs_of(K), G)) return false;
-  return split_cuts_tile(0, units, units, slabs_of(K), G);
-}
-
-// For a batch: which jobs have a tile cut between CTAs (job order as given).
-void dense_batch_needs_zero(const DenseJob* jobs, int count, int TN, int ctas, int MH,
-                            bool* out) {
-  int64_t total = 0;
-  for (int i = 0; i < count; ++i)
-    if (jobs[i].n_tiles > 0 && jobs[i].N > 0)
-      total += job_units(jobs[i].n_tiles, jobs[i].N, jobs[i].K, TN, MH);
-  int64_t tiles = 0;
-  for (int i = 0; i < count; ++i)
-    if (jobs[i].n_tiles > 0 && jobs[i].N > 0)
-      tiles += job_units(jobs[i].n_tiles, jobs[i].N, jobs[i].K, TN, MH) / slabs_of(jobs[i].K);
-  const int64_t G = grid_for(total, tiles, ctas);
-  const bool aligned = use_aligned(tiles, G);
-  int64_t before = 0;
-  for (int i = 0; i < count; ++i) {
-    out[i] = false;
-    if (aligned) continue;
-    if (jobs[i].n_tiles <= 0 || jobs[i].N <= 0) continue;
-    const int64_t units = job_units(jobs[i].n_tiles, jobs[i].N, jobs[i].K, TN, MH);
-    out[i] = split_cuts_tile(before, units, total, slabs_of(jobs[i].K), G);
-    before += units;
-  }
-}
-
-template <int NP>
-static rosko_status dispatch_jobs(const DenseJob* jobs, int count, int TN, int MH, int ctas,
-                                  cudaStream_t st) {
-  if (TN == 256 && MH == 2) return run_jobs<256, NP, 2>(jobs, count, ctas, st);
-  if (TN == 256) return run_jobs<256, NP, 1>(jobs, count, ctas, st);
-  if (MH == 2) return run_jobs<128, NP, 2>(jobs, count, ctas, st);
-  return run_jobs<128, NP, 1>(jobs, count, ctas, st);
-}
-
-rosko_status dense_batch_launch(const DenseJob* jobs, int count, int TN, int ctas, int MH,
-                                cudaStream_t st) {
-  if (count <= 0) return ROSKO_OK;
-  if ((TN != 128 && TN != 256) || (MH != 1 && MH != 2)) return ROSKO_ERR_INVALID_ARG;
+bool dense_needs_zero(int64_t n_tiles, int64_t N, int64_t K, int TN, int ctas) {
+  if (n_tiles <= 0 || N <= 0) return false;
   if (ctas <= 0) ctas = num_sms();
-  if (count == 1) return dispatch_jobs<1>(jobs, 1, TN, MH, ctas, st);
-  if (count <= 64) return dispatch_jobs<64>(jobs, count, TN, MH, ctas, st);
-  return ROSKO_ERR_INVALID_ARG;
+  DenseJob j{};
+  j.n_tiles = n_tiles;
+  j.N = N;
+  j.K = K;
+  DenseProb p{};
+  DenseSplit S{};
+  if (!plan_split(&j, 1, TN, ctas, group_of(n_tiles, ctas), &p, &S)) return false;
+  std::vector<char> cut;
+  cut_problems(S, &p, &cut);
+  return !cut.empty() && cut[0];
 }
+
+rosko_status dense_batch_launch(const DenseJob* jobs, int count, int TN, int cg, cudaStream_t st) {
+  return dispatch_jobs(jobs, count, TN, cg, num_sms(), false, false, st);
+}
+
+// Which jobs of a batch have a tile cut between workers (job order as given;
+// the caller zero-fills their C unless they accumulate).
+void dense_batch_needs_zero(const DenseJob* jobs, int count, int TN, int cg, bool* out) {
+  std::vector<DenseProb> p((size_t)std::max(count, 1));
+  DenseSplit S{};
+  for (int i = 0; i < count; ++i) out[i] = false;
+  if (!plan_split(jobs, count, TN, num_sms(), cg, p.data(), &S)) return;   // the launch refuses it
+  std::vector<char> cut;
+  cut_problems(S, p.data(), &cut);
+  for (int i = 0, n = 0; i < count; ++i)
+    if (jobs[i].n_tiles > 0 && jobs[i].N > 0) out[i] = cut[(size_t)n++] != 0;
+}
+
+int dense_group(int64_t n_tiles) { return group_of(n_tiles, num_sms()); }
 
 namespace {
 // Zero rows x row_bytes of C (pitch bytes apart), one CTA per row at a time.
-// Dependents may launch at once: they wait (griddepcontrol.wait) before
-// touching C.
+// As dense_cut_fill_kernel, a link of the programmatic chain.
 __global__ void zero_fill_kernel(char* __restrict__ C, int64_t pitch, int64_t row_bytes,
                                  int64_t rows, int vec16) {
-  pdl_trigger();   // the tensor-core launch after it starts at once
+  pdl_wait();
+  pdl_trigger();   // the tensor-core launch after it starts now
   for (int64_t r = blockIdx.x; r < rows; r += gridDim.x) {
     char* row = C + r * pitch;
     if (vec16) {
@@ -805,6 +845,8 @@ __global__ void zero_fill_kernel(char* __restrict__ C, int64_t pitch, int64_t ro
 // INT8 -> BF16 (exact: |code| <= 127), K rows of N, into rows of ldo.
 __global__ void i8_to_bf16_kernel(const int8_t* __restrict__ B, int64_t K, int64_t N, int64_t ldb,
                                   __nv_bfloat16* __restrict__ out, int64_t ldo) {
+  pdl_wait();
+  pdl_trigger();   // the launch after it waits in its own
   const int64_t cols = (ldo + 3) / 4;   // four values per thread
   const int64_t n = K * cols;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
@@ -833,11 +875,10 @@ rosko_status zero_fill_launch(const ZeroFill& z, cudaStream_t st) {
   // a grid that is resident at once, so that every CTA has signalled its
   // dependents before the tensor-core launch needs an SM
   const int64_t grid = std::min<int64_t>(z.rows, (int64_t)num_sms() * 4);
-  // an ordinary launch: when it starts, every launch before it has completed,
-  // so its programmatic dependent (the tensor-core kernel) may read A and B
-  // at once; only that kernel's writes of C wait for the fill
-  zero_fill_kernel<<<(unsigned)grid, 256, 0, st>>>(static_cast<char*>(z.C), z.pitch, z.row_bytes,
-                                                   z.rows, vec16);
+  if (launch_dependent(zero_fill_kernel, dim3((unsigned)grid), dim3(256), 0, st,
+                       static_cast<char*>(z.C), z.pitch, z.row_bytes, z.rows, vec16) !=
+      cudaSuccess)
+    return ROSKO_ERR_CUDA;
   count_launches(1);
   return cudaGetLastError() == cudaSuccess ? ROSKO_OK : ROSKO_ERR_CUDA;
 }
@@ -849,9 +890,8 @@ constexpr int kI8ChunkSlabs = 16;
 
 rosko_status dense_spmm_i8_launch(const rosko_packed_s* h, int64_t n_tiles, const int8_t* B,
                                   int64_t N, int64_t ldb, int32_t* C, int64_t ldc, int TN,
-                                  int ctas, int MH, const ZeroFill* zf, cudaStream_t st) {
+                                  int ctas, const ZeroFill* zf, cudaStream_t st) {
   if (n_tiles <= 0 || N <= 0) return ROSKO_OK;
-  if (TN != 128 && TN != 256) return ROSKO_ERR_INVALID_ARG;
   if (ctas <= 0) ctas = num_sms();
   const int64_t K = h->K;
   const int64_t ldo = (N + 7) / 8 * 8;   // 16-byte rows for the tensor map
@@ -862,10 +902,11 @@ rosko_status dense_spmm_i8_launch(const rosko_packed_s* h, int64_t n_tiles, cons
     return ROSKO_ERR_OOM;
   const int64_t work = K * ((ldo + 3) / 4);
   const unsigned blocks = (unsigned)std::max<int64_t>(1, std::min<int64_t>((work + 255) / 256, 4096));
-  i8_to_bf16_kernel<<<blocks, 256, 0, st>>>(B, K, N, ldb, static_cast<__nv_bfloat16*>(scratch),
-                                            ldo);
+  rosko_status s = launch_dependent(i8_to_bf16_kernel, dim3(blocks), dim3(256), 0, st, B, K, N, ldb,
+                                    static_cast<__nv_bfloat16*>(scratch), ldo) == cudaSuccess
+                       ? ROSKO_OK
+                       : ROSKO_ERR_CUDA;
   count_launches(1);
-  rosko_status s = cudaGetLastError() == cudaSuccess ? ROSKO_OK : ROSKO_ERR_CUDA;
   // the zero fill of C (after the conversion, so that B is complete when the
   // dependent tensor-core launch starts)
   if (s == ROSKO_OK && zf) s = zero_fill_launch(*zf, st);
@@ -886,59 +927,40 @@ rosko_status dense_spmm_i8_launch(const rosko_packed_s* h, int64_t n_tiles, cons
     j.accumulate = 1;   // every chunk adds into the zeroed (or accumulated) C
     j.kchunk = kI8ChunkSlabs;
     j.out_i32 = 1;
-    j.pdl = zf ? 1 : 0;
-    s = dense_batch_launch(&j, 1, TN, ctas, MH, st);
+    s = dispatch_jobs(&j, 1, TN, group_of(n_tiles, ctas), ctas, false, zf != nullptr, st);
   }
   pool_free(scratch, st);
   return s;
 }
 
-rosko_status dense_spmm_launch(const void* dense_A, int64_t dense_rows, int64_t Kpad,
-                               const int32_t* tile_order_dev, int64_t n_tiles, int64_t K,
-                               const void* B, int64_t N, int64_t ldb, float* C, int64_t ldc,
-                               int64_t M, int accumulate, int TN, int ctas, int MH,
-                               bool c_zeroed, const ZeroFill* zf, cudaStream_t st) {
+rosko_status dense_spmm_launch(const rosko_packed_s* h, int64_t n_tiles, const void* B, int64_t N,
+                               int64_t ldb, float* C, int64_t ldc, int accumulate, int TN,
+                               int ctas, bool zero_cut, const ZeroFill* zf, cudaStream_t st) {
   if (n_tiles <= 0 || N <= 0) return ROSKO_OK;
-  if (TN != 128 && TN != 256) return ROSKO_ERR_INVALID_ARG;
   if (ctas <= 0) ctas = num_sms();
+  // the whole of C (the sparse panels need it too), or only the cut tiles
   if (zf) {
     rosko_status s = zero_fill_launch(*zf, st);
     if (s != ROSKO_OK) return s;
-  } else if (!accumulate && !c_zeroed && dense_needs_zero(n_tiles, N, K, TN, ctas, MH)) {
-    // zero the C rows of every dense tile (tiles are disjoint row blocks)
-    std::vector<int32_t> order((size_t)n_tiles);
-    if (cudaMemcpyAsync(order.data(), tile_order_dev, order.size() * 4, cudaMemcpyDeviceToHost,
-                        st) != cudaSuccess ||
-        cudaStreamSynchronize(st) != cudaSuccess)
-      return ROSKO_ERR_CUDA;
-    for (int32_t t : order) {
-      const int64_t r0 = (int64_t)t * kTM;
-      const int64_t rows = std::min<int64_t>(kTM, M - r0);
-      if (rows > 0 &&
-          cudaMemset2DAsync(C + r0 * ldc, (size_t)ldc * 4, 0, (size_t)N * 4, (size_t)rows, st) !=
-              cudaSuccess)
-        return ROSKO_ERR_CUDA;
-    }
   }
   DenseJob j;
-  j.dense_A = dense_A;
-  j.dense_rows = dense_rows;
-  j.Kpad = Kpad;
-  j.tile_order_dev = tile_order_dev;
+  j.dense_A = h->dense_A;
+  j.dense_rows = h->n_copy * kTM;
+  j.Kpad = h->Kpad;
+  j.tile_order_dev = h->tile_order_dev;
   j.n_tiles = n_tiles;
-  j.K = K;
+  j.K = h->K;
   j.B = B;
   j.N = N;
   j.ldb = ldb;
   j.C = C;
   j.ldc = ldc;
-  j.M = M;
+  j.M = h->M;
   j.accumulate = accumulate;
   // a programmatic dependent of its zero fill only (it reads A and B before
   // any wait, which is safe only after a launch that started after every
   // earlier one had completed)
-  j.pdl = zf ? 1 : 0;
-  return dense_batch_launch(&j, 1, TN, ctas, MH, st);
+  return dispatch_jobs(&j, 1, TN, group_of(n_tiles, ctas), ctas, zero_cut, zf != nullptr, st);
 }
 
 }  // namespace rosko

@@ -1074,8 +1074,7 @@ static int64_t direct_prob(const DirectJob& j, int V, int64_t items0, DirectProb
   return n_segs * P->strips;
 }
 
-rosko_status direct_batch_launch(const DirectJob* jobs, int count, int V, cudaStream_t st,
-                                 bool pdl) {
+rosko_status direct_batch_launch(const DirectJob* jobs, int count, int V, cudaStream_t st) {
   if (count <= 0) return ROSKO_OK;
   if (count > 64) return ROSKO_ERR_INVALID_ARG;
   const rosko_dtype a = jobs[0].h->dt, b = jobs[0].b_dt, c = jobs[0].c_dt;
@@ -1114,29 +1113,18 @@ rosko_status direct_batch_launch(const DirectJob* jobs, int count, int V, cudaSt
     const int64_t items = fill(T);
     if (items < 0 || items > INT_MAX) return ROSKO_ERR_UNSUPPORTED;   // 31-bit item index
     if (items == 0) return ROSKO_OK;
-    if (pdl) {
-      // a programmatic dependent of the launch before it (waits in-kernel)
-      cudaLaunchConfig_t cfg = {};
-      cfg.gridDim = dim3((unsigned)((items + 7) / 8));
-      cfg.blockDim = dim3(256);
-      cfg.dynamicSmemBytes = e->smem;
-      cfg.stream = st;
-      cudaLaunchAttribute attr[1];
-      attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-      attr[0].val.programmaticStreamSerializationAllowed = 1;
-      cfg.attrs = attr;
-      cfg.numAttrs = 1;
-      if (cudaLaunchKernelEx(&cfg, e->one, T) != cudaSuccess) return ROSKO_ERR_CUDA;
-    } else {
-      e->one<<<(unsigned)((items + 7) / 8), 256, e->smem, st>>>(T);
-    }
+    if (launch_dependent(e->one, dim3((unsigned)((items + 7) / 8)), dim3(256), e->smem, st, T) !=
+        cudaSuccess)
+      return ROSKO_ERR_CUDA;
   } else {
     DirectTable<64> T;
     std::memset(static_cast<void*>(&T), 0, sizeof(T));
     const int64_t items = fill(T);
     if (items < 0 || items > INT_MAX) return ROSKO_ERR_UNSUPPORTED;   // 31-bit item index
     if (items == 0) return ROSKO_OK;
-    e->many<<<(unsigned)((items + 7) / 8), 256, e->smem, st>>>(T);
+    if (launch_dependent(e->many, dim3((unsigned)((items + 7) / 8)), dim3(256), e->smem, st, T) !=
+        cudaSuccess)
+      return ROSKO_ERR_CUDA;
   }
   count_launches(1);
   return cudaGetLastError() == cudaSuccess ? ROSKO_OK : ROSKO_ERR_CUDA;
@@ -1151,7 +1139,7 @@ rosko_status sparse_spmm_launch(rosko_packed_s* h, const void* B, rosko_dtype b_
   if (L.order == 4) {
     // one warp per C row, B from L2; no K split, C written (or added) directly
     DirectJob j{h, B, b_dt, N, ldb, col_scale, C, c_dt, ldc, accumulate, panel_list, n_panels};
-    return direct_batch_launch(&j, 1, L.V, st, true);
+    return direct_batch_launch(&j, 1, L.V, st);
   }
   if (L.order == 2 && !h->rnz) return ROSKO_ERR_UNSUPPORTED;
   if (L.order == 3 && (!h->gnz || L.R != 16 || L.W != 8)) return ROSKO_ERR_UNSUPPORTED;
