@@ -76,11 +76,11 @@ typedef enum {
  *   k_c   rows of B staged in shared memory per pipeline slab.
  *   m_c   C rows per CTA = warps per CTA x m_r.
  *   split_k  number of K ranges reduced into C with atomics (>= 1).
- *   dense_split_pm  BF16, and INT8 with an INT32 result: 128-row tiles of A
- *         whose density in per mille (nonzeros per 1000 entries) is >= this
- *         value run on the tensor-core dense-panel path, the others on the
- *         sparse path; >= 1001 = never.  At pack time the same field is the
- *         minimum density for which a dense copy is kept.
+ *   dense_split_pm  BF16 and INT8: 128-row tiles of A whose density in per
+ *         mille (nonzeros per 1000 entries) is >= this value run on the
+ *         tensor-core dense-panel path, the others on the sparse path;
+ *         >= 1001 = never.  At pack time the same field is the minimum
+ *         density for which a dense copy is kept.
  *   dense_n_r      C columns per tensor-core tile (128 or 256).
  *   dense_split_k  CTAs over which the tensor-core path divides its (tile, K
  *         slab) work, at most one per SM (default: one per SM); a tile whose
@@ -180,14 +180,14 @@ rosko_status rosko_pack_transposed(const void* A_dev, rosko_dtype a_dtype, int64
  * differ run to run in the last bits.  N may be 0 (no-op).
  * Dense-panel tiles (BF16) multiply their explicit zeros too, so there a
  * non-finite B value meets 0 * Inf = NaN, while skipped rows never see it.
- * INT8 packs with an INT32 result run their dense-enough tiles on the same
- * tensor-core path, exactly: the codes are integers exact in BF16, every K
- * chunk of at most 1024 sums below 2^24 in magnitude (exact in the FP32
- * accumulator) and is added into C as INT32, so the result is bit-identical
- * to the integer sum; the call converts B to BF16 in stream-ordered scratch
- * (K x N x 2 bytes from the library's device memory pool on `stream`,
- * released in stream order).  The FP32 (dequantised) INT8 result stays on
- * the CUDA-core path.
+ * INT8 packs run their dense-enough tiles on the same tensor-core path,
+ * exactly: the codes are integers exact in BF16, every K chunk of at most
+ * 1024 sums below 2^24 in magnitude (exact in the FP32 accumulator) and is
+ * added to an INT32 sum, so an INT32 result is bit-identical to the integer
+ * sum, and an FP32 (dequantised) result is that sum scaled (a tile whose K
+ * range is divided adds its scaled pieces).  The call converts B to BF16 in
+ * stream-ordered scratch (K x N x 2 bytes from the library's device memory
+ * pool on `stream`, released in stream order).
  * Stream order: when C must be zero-filled first (tiles or rows cut along K
  * and added), the fill is a small kernel ahead of a tensor-core launch (of
  * the cut tiles only, unless the sparse part adds too), else a memset.  Every

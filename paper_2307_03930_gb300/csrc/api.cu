@@ -206,10 +206,9 @@ void dense_config(int64_t n_tiles, int64_t N, int64_t K, int sms, int* TN_out, i
 // (the autotuner and the selector refine it per shape).
 constexpr int kDenseSplitPm = 15;
 constexpr int kDenseCopyPm = 1;
-// INT8 codes through the BF16 tensor pipe (exact, K chunks of 1024 added into
-// INT32 C): against ~15 TOPS of 2*nnz*N for the INT8 row-direct kernel
-// (c3 shapes) the break-even tile density is again near 1.5%; dense copies of
-// INT8 packs are kept from 1% (the copies are BF16: twice the INT8 bytes).
+// INT8 codes through the BF16 tensor pipe: per tile the break-even is near
+// the same 1.5%; dense copies of INT8 packs are kept from 1% (the copies are
+// BF16: twice the INT8 bytes).
 constexpr int kDenseSplitPmI8 = 15;
 constexpr int kDenseCopyPmI8 = 10;
 
@@ -283,6 +282,21 @@ rosko_status schedule_analytic(int64_t M, int64_t K, int64_t N, int64_t nnz, int
     // by these models costs 5% over the better of the two paths.
     const double t_dense = 10.8 + 2.0 * (double)M * (double)K * (double)N / 0.58e15 * 1e6;
     const double t_direct = 5.3 + (double)nnz * (double)N * 2.0 / 10.9e12 * 1e6;
+    if (t_direct < t_dense) t->dense_split_pm = 1001;
+  }
+  if (dt == ROSKO_I8 && order == 4) {
+    // The same choice for INT8 codes (either result type).  Row-direct: 2.5 us
+    // plus a byte of B per nonzero and column, whole 256-column strips, at
+    // ~8.5 TB/s.  Tensor cores: three launches' 8.5 us, the dense product at
+    // ~1.9 PFLOP/s, and the memory it moves: B converted to BF16 (3 bytes per
+    // value), C and the dense copies.  512x4608x3136 at 90 %: 27-30 us against
+    // 110-117 us; 512x1024x1000: 12-15 against 14.7; 200x1500x130 at 60 %: 11
+    // against 6.
+    const double t_dense = 8.5 + 2.0 * (double)M * (double)K * (double)N / 1.9e15 * 1e6 +
+                           3.0 * (double)K * (double)N / 5e12 * 1e6 +
+                           4.0 * (double)M * (double)N / 3e12 * 1e6 +
+                           2.0 * (double)M * (double)K / 7e12 * 1e6;
+    const double t_direct = 2.5 + (double)nnz * (double)((N + 255) / 256) * 256.0 / 8.5e12 * 1e6;
     if (t_direct < t_dense) t->dense_split_pm = 1001;
   }
   int TN = 256, ds = 1;
@@ -504,8 +518,8 @@ rosko_status spmm_run(rosko_packed_s* A, const void* B_dev, rosko_dtype b_dtype,
   }
   // ---- dense-panel split: a prefix of the density-sorted dense copies ----
   int64_t n_dense = 0, dense_panels = 0;
-  // tensor-core tiles: BF16, or INT8 codes with an INT32 result (exact)
-  const bool tc_ok = p == ROSKO_BF16 || (p == ROSKO_I8 && c_dtype == ROSKO_I32);
+  // tensor-core tiles: BF16, or INT8 codes (integer sums exact)
+  const bool tc_ok = p == ROSKO_BF16 || p == ROSKO_I8;
   if (tc_ok && A->n_copy > 0 && t.dense_split_pm <= 1000) {
     while (n_dense < A->n_copy &&
            A->tile_density[(size_t)n_dense] * 1000.0 >= (double)t.dense_split_pm) {
@@ -594,11 +608,10 @@ rosko_status spmm_run(rosko_packed_s* A, const void* B_dev, rosko_dtype b_dtype,
     if (!direct_segments(A, A->panel_order_dev, n_sparse, which, &ns, &direct_cut))
       return ROSKO_ERR_UNSUPPORTED;
   }
-  // (INT8 tensor-core tiles add every K chunk into C)
   const bool zero_sparse = !accumulate && n_sparse > 0 && (L.split > 1 || direct_cut);
   const bool zero_dense =
       !accumulate && !skip_dense && n_dense > 0 &&
-      (p == ROSKO_I8 || dense_needs_zero(n_dense, N, A->K, t.dense_n_r, t.dense_split_k));
+      dense_needs_zero(n_dense, N, A->K, t.dense_n_r, t.dense_split_k);
   const bool zero_c = zero_sparse || zero_dense;
   if (flags & kRunPlanOnly) {
     // report the split and the resolved schedule, launch nothing
@@ -625,14 +638,14 @@ rosko_status spmm_run(rosko_packed_s* A, const void* B_dev, rosko_dtype b_dtype,
           cudaSuccess)
     return ROSKO_ERR_CUDA;
   if (run_dense) {
-    // BF16 without a sparse part that adds: only the cut tiles are zeroed
-    const bool cut_only = fill && !zero_sparse && p == ROSKO_BF16;
+    // without a sparse part that adds, only the cut tiles are zeroed
+    const bool cut_only = fill && !zero_sparse;
     const ZeroFill* z = fill && !cut_only ? &zf : nullptr;
     rosko_status s =
         p == ROSKO_I8
             ? dense_spmm_i8_launch(A, n_dense, static_cast<const int8_t*>(B_dev), N, ldb,
-                                   static_cast<int32_t*>(C_dev), ldc, t.dense_n_r,
-                                   t.dense_split_k, z, st)
+                                   col_scale_dev, C_dev, ldc, accumulate, t.dense_n_r,
+                                   t.dense_split_k, cut_only, z, st)
             : dense_spmm_launch(A, n_dense, B_dev, N, ldb, static_cast<float*>(C_dev), ldc,
                                 accumulate, t.dense_n_r, t.dense_split_k, cut_only, z, st);
     if (s != ROSKO_OK) return s;

@@ -230,16 +230,23 @@ struct DenseJob {
   float* C;
   int64_t ldc, M;
   int accumulate;
-  int kchunk = 0;    // K slabs per exact-integer chunk (INT8 codes), 0: none
-  int out_i32 = 0;   // C is INT32 (INT8 codes through the BF16 pipe)
+  // INT8 codes through the BF16 pipe (C is INT32, or FP32 with both scales): B
+  // is scratch that the launch fills from src_i8 (leading dimension src_ld)
+  int i8 = 0;
+  const int8_t* src_i8 = nullptr;
+  int64_t src_ld = 0;
+  const float* row_scale = nullptr;
+  const float* col_scale = nullptr;
 };
-// INT8 x INT8 -> INT32 through the BF16 tensor pipe: B is converted to BF16
-// (exact) in stream-ordered scratch, the handle's dense copies hold the INT8
-// codes as BF16, and every K chunk of <= 1024 (exact in FP32) is converted
-// and added into C, which the caller has zeroed unless it accumulates.
+// INT8 x INT8 through the BF16 tensor pipe: B is converted to BF16 (exact) in
+// stream-ordered scratch and the handle's dense copies hold the INT8 codes as
+// BF16; the integer sums are exact.  C is INT32, or with col_scale FP32
+// (scaled by the handle's row scales and col_scale).  zf, zero_cut: as
+// dense_spmm_launch.
 rosko_status dense_spmm_i8_launch(const rosko_packed_s* h, int64_t n_tiles, const int8_t* B,
-                                  int64_t N, int64_t ldb, int32_t* C, int64_t ldc, int TN,
-                                  int ctas, const ZeroFill* zf, cudaStream_t st);
+                                  int64_t N, int64_t ldb, const float* col_scale, void* C,
+                                  int64_t ldc, int accumulate, int TN, int ctas, bool zero_cut,
+                                  const ZeroFill* zf, cudaStream_t st);
 // One persistent launch over all jobs' dense tiles (count <= 64) by workers of
 // cg CTAs; C of jobs whose tiles the split cuts must be zeroed by the caller
 // unless they accumulate (dense_batch_needs_zero).

@@ -52,6 +52,15 @@
 // hands the tile to TMA: a tensor store for a whole tile, a tensor
 // reduce-add (element-wise add in L2) for a cut tile or C += A.B.  Two
 // staging tiles per warp let the next chunk's TMEM load overlap the copy.
+//
+// INT8 packs run through the same BF16 pipe (GB300's INT8 tensor rate is far
+// below it): the codes are exact in BF16, and accumulators end every
+// kI8ChunkSlabs K slabs, where every FP32 partial sum is still an exact
+// integer.  The epilogue converts each chunk and sums it in INT32 registers
+// while the next chunk's MMAs run, and writes C once per range: INT32, or
+// FP32 times the row and column scales.  (Adding every chunk into INT32 C in
+// global memory instead cost an epilogue per 1,024 K: 162 against 115 us for
+// 4096x11008x2048, and kept the scaled result off the tensor cores.)
 // C whose rows are not 16-byte aligned falls back to direct stores and
 // 16-byte atomics.
 #include <algorithm>
@@ -71,10 +80,16 @@ constexpr uint32_t kStageC = 32 * 32 * 4;      // one 32 x 32 FP32 staging tile
 // Epilogue warps: 4 (one per TMEM lane quarter), two staging tiles each.
 // Eight warps ran the epilogue in the same time (it is bound by the TMA
 // stores and L2 reductions, ~28 bytes per cycle per SM, not by the warps).
-constexpr int kEpiWarps = 4;
-constexpr int kStagePerWarp = 2;
-constexpr uint32_t kEpiBytes = kEpiWarps * kStagePerWarp * kStageC;
-constexpr int kThreads = 64 + 32 * kEpiWarps;
+// INT8 packs (I8) take eight, two per quarter with half of the columns each:
+// their 128 columns of INT32 sums per lane live in registers.
+template <bool I8> constexpr int kEpiWarps = I8 ? 8 : 4;
+template <bool I8> constexpr int kThreads = 64 + 32 * kEpiWarps<I8>;
+constexpr int kStageTiles = 8;                 // staging tiles of all warps
+constexpr uint32_t kEpiBytes = kStageTiles * kStageC;
+// INT8 codes: K slabs of 64 per exact chunk.  16 slabs = 1024 products of
+// magnitude <= 127^2, so a partial sum stays below 1024 * 16129 < 2^24 and is
+// exact in the FP32 accumulator.
+constexpr int kI8ChunkSlabs = 16;
 // A tile's cost in K slabs is at least its epilogue's time (128 KB per
 // 128 x 256 accumulator at ~28 B/clk: about nine slabs of 512 cycles; the
 // same ratio for 128-column tiles).
@@ -130,11 +145,9 @@ struct DenseTable {
   // where each worker's share begins (computed on the host: the divisions
   // cost a worker about a microsecond at its start)
   DensePos start[kMaxWorkers + 1];
-  // INT8 codes through the BF16 pipe: accumulator segments end every
-  // `kchunk` K slabs (0: only at tile ends), so that every FP32 partial sum
-  // stays an exact integer, and C is INT32 (partials converted and added)
-  int kchunk;
-  int out_i32;
+  // INT8 packs: the scales of an FP32 result (NULL: C is INT32)
+  const float* row_scale;
+  const float* col_scale;
   // 1: the launch follows a zero fill of C that started after everything
   // before it had completed, so A and B may be read at once
   int early_ab;
@@ -229,8 +242,8 @@ struct SegIter {
   }
 };
 
-template <int TN, int NP, int CG>
-__global__ void __cluster_dims__(CG, 1, 1) __launch_bounds__(kThreads, 1)
+template <int TN, int NP, int CG, bool I8>
+__global__ void __cluster_dims__(CG, 1, 1) __launch_bounds__(kThreads<I8>, 1)
     dense_panel_kernel(const __grid_constant__ DenseTable<NP> T, int S) {
   constexpr int BN = TN / CG;                             // B columns this CTA loads
   constexpr uint32_t kBBytes = (uint32_t)BN * kTK * 2;
@@ -266,7 +279,7 @@ __global__ void __cluster_dims__(CG, 1, 1) __launch_bounds__(kThreads, 1)
       }
       for (int b = 0; b < 2; ++b) {
         mbar_init(&acc_full[b], 1);
-        mbar_init(&acc_empty[b], CG * kEpiWarps);
+        mbar_init(&acc_empty[b], CG * kEpiWarps<I8>);
       }
       fence_barrier_init();
     }
@@ -286,7 +299,7 @@ __global__ void __cluster_dims__(CG, 1, 1) __launch_bounds__(kThreads, 1)
   if constexpr (CG == 2) cluster_wait();
   uint32_t tmem = 0;
   if (warp != 0) {
-    asm volatile("bar.sync 1, %0;" ::"n"(kThreads - 32) : "memory");
+    asm volatile("bar.sync 1, %0;" ::"n"(kThreads<I8> - 32) : "memory");
     tc::fence_after_sync();
     tmem = *tmem_slot;
   }
@@ -378,11 +391,10 @@ __global__ void __cluster_dims__(CG, 1, 1) __launch_bounds__(kThreads, 1)
     bool ok = true;
     int b = NBUF - 1;          // accumulator of the current segment
     uint32_t bph = 0;          // parity of its last release (fresh: passes)
-    const int kc = T.kchunk;
     while (rank == 0 && ok && it.next(sg)) {
       for (int c0 = sg.s0; ok && c0 < sg.s1;) {
         // slabs [c0, c1) sum in one accumulator
-        const int c1 = kc ? min(sg.s1, (c0 / kc + 1) * kc) : sg.s1;
+        const int c1 = I8 ? min(sg.s1, c0 + kI8ChunkSlabs) : sg.s1;
         if (++b == NBUF) {
           b = 0;
           bph ^= 1u;
@@ -432,12 +444,35 @@ __global__ void __cluster_dims__(CG, 1, 1) __launch_bounds__(kThreads, 1)
     // Without such a dependency the wait returns at once.
     pdl_wait();
     const int quarter = warp & 3;                  // TMEM lanes 32 quarter .. + 31
+    constexpr int kParts = kEpiWarps<I8> / 4;      // warps that share a quarter
+    constexpr int kChunks = TN / 32 / kParts;      // 32-column chunks of a warp
+    constexpr int kStagePerWarp = kStageTiles / kEpiWarps<I8>;
+    const int part = (warp - 2) >> 2;              // column part of this warp
     uint8_t* my_stage = stage_c + (size_t)(warp - 2) * kStagePerWarp * kStageC;
     const uint32_t drained = CG == 2 ? cluster_addr(acc_empty, 0) : 0u;
     int chunk = 0;   // staging tiles alternate per chunk
     int b = NBUF - 1;
     uint32_t bph = 1;
-    const int kc = T.kchunk, out_i32 = T.out_i32;
+    const bool i32 = I8 && !T.row_scale;
+    auto wait_acc = [&]() -> bool {
+      if (++b == NBUF) {
+        b = 0;
+        bph ^= 1u;
+      }
+      const bool ok = __all_sync(0xffffffffu, mbar_wait_bounded(&acc_full[b], bph, T.status));
+      tc::fence_after_sync();
+      return ok;
+    };
+    const uint32_t my_tmem = tmem + ((uint32_t)(quarter * 32) << 16);
+    auto release_acc = [&]() {
+      // accumulator drained: hand it back to the MMA issuer
+      tc::fence_before_sync();
+      __syncwarp();
+      if (lane == 0) {
+        if constexpr (CG == 2) mbar_arrive_cluster(drained + (uint32_t)b * 8u);
+        else mbar_arrive(&acc_empty[b]);
+      }
+    };
     while (it.next(sg)) {
       const DenseProb& P = T.p[sg.q];
       const int q = sg.q;
@@ -451,88 +486,120 @@ __global__ void __cluster_dims__(CG, 1, 1) __launch_bounds__(kThreads, 1)
       const int tma_c = P.tma_c;
       const bool add = !sg.whole || P.accumulate;
       const int64_t n0 = (int64_t)sg.nt * TN;
-      for (int c0 = sg.s0; c0 < sg.s1; c0 = kc ? min(sg.s1, (c0 / kc + 1) * kc) : sg.s1) {
-        if (++b == NBUF) {
-          b = 0;
-          bph ^= 1u;
+      const int64_t ldc = P.ldc;
+      float* c_row0 = P.C + row0 * ldc + lane;   // this lane's column of a chunk
+      // write (or add) the 32 x 32 chunk at column col0: r[j] of lane i is
+      // the value (FP32 or INT32 bits) of row row0 + i, column col0 + j
+      auto put_chunk = [&](const uint32_t (&r)[32], int64_t col0) {
+        if (tma_c) {
+          // staging tile (chunk % n) is free once the copy issued n chunks
+          // ago has read it
+          uint8_t* buf = my_stage + (size_t)(chunk % kStagePerWarp) * kStageC;
+          if (lane == 0) bulk_wait_read<kStagePerWarp - 1>();
+          __syncwarp();
+          // row `lane`, 16-byte chunk j at (j ^ (lane % 8)): the 128-byte swizzle
+#pragma unroll
+          for (int j = 0; j < 8; ++j)
+            *reinterpret_cast<uint4*>(buf + lane * 128 + ((j ^ (lane & 7)) << 4)) =
+                make_uint4(r[4 * j], r[4 * j + 1], r[4 * j + 2], r[4 * j + 3]);
+          fence_proxy_async_smem();
+          __syncwarp();
+          if (lane == 0) {
+            // rows past M and columns past N are clipped by the tensor map
+            if (add) tma_reduce_add_2d(&T.tmC[q], (int32_t)col0, (int32_t)row0, buf);
+            else tma_store_2d(&T.tmC[q], (int32_t)col0, (int32_t)row0, buf);
+            bulk_commit();
+          }
+          ++chunk;
+          return;
         }
-        const bool ok = __all_sync(0xffffffffu, mbar_wait_bounded(&acc_full[b], bph, T.status));
-        tc::fence_after_sync();
+        // C rows not 16-byte aligned (no tensor map): transpose the 32 x 32
+        // chunk through this warp's staging tile (rotated rows, no bank
+        // conflicts) so that each store instruction writes 32 consecutive
+        // columns of one row
+        uint32_t* tr = reinterpret_cast<uint32_t*>(my_stage);
+        // the staging tiles may still be read by this warp's TMA stores of
+        // an earlier problem of the batch (one with aligned C rows): wait
+        // until those reads are done before reusing the space
+        if (lane == 0) bulk_wait_read<0>();
+        __syncwarp();
+#pragma unroll
+        for (int j = 0; j < 32; ++j) tr[lane * 32 + ((j + lane) & 31)] = r[j];
+        __syncwarp();
+        const int rows = (int)(PM - row0 < 32 ? PM - row0 : 32);
+        if (col0 + lane < PN) {
+          // eight rows at a time: their shared-memory reads, then their stores
+          float* dst = c_row0 + col0;
 #pragma unroll 1
-        for (int cc = 0; cc < TN / 32; ++cc) {
-          const int64_t col0 = n0 + cc * 32;
-          if (!ok || !rows_ok || col0 >= PN) break;   // warp-uniform
-          uint32_t r[32];
-          tc::tmem_ld_32x32b_x32(
-              tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(b * TN + cc * 32), r);
-          tc::tmem_ld_wait();
-          if (out_i32) {
-            // an exact integer in FP32 (|partial| < 2^24): convert to INT32
+          for (int r0 = 0; r0 < rows; r0 += 8, dst += 8 * ldc) {
+            uint32_t v[8];
 #pragma unroll
-            for (int j = 0; j < 32; ++j) r[j] = (uint32_t)__float2int_rn(__uint_as_float(r[j]));
-          }
-          if (tma_c) {
-            // staging tile (chunk & 1) is free once the copy issued two
-            // chunks ago has read it
-            uint8_t* buf = my_stage + (size_t)(chunk % kStagePerWarp) * kStageC;
-            if (lane == 0) bulk_wait_read<kStagePerWarp - 1>();
-            __syncwarp();
-            // row `lane`, 16-byte chunk j at (j ^ (lane % 8)): the 128-byte swizzle
+            for (int i = 0; i < 8; ++i) v[i] = tr[(r0 + i) * 32 + ((lane + r0 + i) & 31)];
 #pragma unroll
-            for (int j = 0; j < 8; ++j)
-              *reinterpret_cast<uint4*>(buf + lane * 128 + ((j ^ (lane & 7)) << 4)) =
-                  make_uint4(r[4 * j], r[4 * j + 1], r[4 * j + 2], r[4 * j + 3]);
-            fence_proxy_async_smem();
-            __syncwarp();
-            if (lane == 0) {
-              // rows past M and columns past N are clipped by the tensor map
-              if (add) tma_reduce_add_2d(&T.tmC[q], (int32_t)col0, (int32_t)row0, buf);
-              else tma_store_2d(&T.tmC[q], (int32_t)col0, (int32_t)row0, buf);
-              bulk_commit();
-            }
-            ++chunk;
-            continue;
-          }
-          // C rows not 16-byte aligned (no tensor map): transpose the 32 x 32
-          // chunk through this warp's staging tile (rotated rows, no bank
-          // conflicts) so that each store instruction writes 32 consecutive
-          // columns of one row
-          float* tr = reinterpret_cast<float*>(my_stage);
-          // the staging tiles may still be read by this warp's TMA stores of
-          // an earlier problem of the batch (one with aligned C rows): wait
-          // until those reads are done before reusing the space
-          if (lane == 0) bulk_wait_read<0>();
-          __syncwarp();
-#pragma unroll
-          for (int j = 0; j < 32; ++j) tr[lane * 32 + ((j + lane) & 31)] = __uint_as_float(r[j]);
-          __syncwarp();
-          const int64_t col = col0 + lane;
-          const int rows = (int)(PM - row0 < 32 ? PM - row0 : 32);
-          if (col < PN) {
-#pragma unroll 4
-            for (int rr = 0; rr < rows; ++rr) {
-              const float v = tr[rr * 32 + ((lane + rr) & 31)];
-              float* dst = P.C + (row0 + rr) * P.ldc + col;
-              if (out_i32) {
-                int* di = reinterpret_cast<int*>(dst);
-                const int iv = (int)__float_as_uint(v);   // already converted
-                if (add) atomicAdd(di, iv);
-                else *di = iv;
-              } else if (add) {
-                atomicAdd(dst, v);   // a cut tile, or C += A.B
+            for (int i = 0; i < 8; ++i) {
+              if (r0 + i >= rows) break;
+              float* d = dst + i * ldc;
+              if (!add) {
+                *reinterpret_cast<uint32_t*>(d) = v[i];
+              } else if (i32) {
+                atomicAdd(reinterpret_cast<int*>(d), (int)v[i]);
               } else {
-                *dst = v;
+                atomicAdd(d, __uint_as_float(v[i]));   // a cut tile, or C += A.B
               }
             }
           }
-          __syncwarp();
         }
-        // accumulator drained: hand it back to the MMA issuer
-        tc::fence_before_sync();
         __syncwarp();
-        if (lane == 0) {
-          if constexpr (CG == 2) mbar_arrive_cluster(drained + (uint32_t)b * 8u);
-          else mbar_arrive(&acc_empty[b]);
+      };
+      if constexpr (!I8) {
+        const bool ok = wait_acc();
+#pragma unroll 1
+        for (int cc = 0; cc < kChunks; ++cc) {
+          const int64_t col0 = n0 + cc * 32;
+          if (!ok || !rows_ok || col0 >= PN) break;   // warp-uniform
+          uint32_t r[32];
+          tc::tmem_ld_32x32b_x32(my_tmem + (uint32_t)(b * TN + cc * 32), r);
+          tc::tmem_ld_wait();
+          put_chunk(r, col0);
+        }
+        release_acc();
+      } else {
+        // INT32 sums; at the end, in place, the bits that go to C
+        uint32_t sum[kChunks][32];
+#pragma unroll
+        for (int cc = 0; cc < kChunks; ++cc)
+#pragma unroll
+          for (int j = 0; j < 32; ++j) sum[cc][j] = 0;
+        bool ok = true;
+        for (int c0 = sg.s0; c0 < sg.s1; c0 += kI8ChunkSlabs) {
+          ok = wait_acc() && ok;
+#pragma unroll
+          for (int h = 0; h < 2 * kChunks; ++h) {
+            uint32_t r[16];
+            tc::tmem_ld_32x32b_x16(
+                my_tmem + (uint32_t)(b * TN + part * kChunks * 32 + h * 16), r);
+            tc::tmem_ld_wait();
+            // an exact integer in FP32 (|partial| < 2^24)
+#pragma unroll
+            for (int j = 0; j < 16; ++j)
+              sum[h / 2][(h & 1) * 16 + j] += (uint32_t)__float2int_rn(__uint_as_float(r[j]));
+          }
+          release_acc();
+        }
+        const float rs = !i32 && rows_ok && row0 + lane < PM ? __ldg(&T.row_scale[row0 + lane]) : 0.0f;
+#pragma unroll
+        for (int cc = 0; cc < kChunks; ++cc) {
+          const int64_t col0 = n0 + (part * kChunks + cc) * 32;
+          if (ok && rows_ok && col0 < PN) {   // warp-uniform
+            if (!i32) {
+              const float cs = col0 + lane < PN ? __ldg(&T.col_scale[col0 + lane]) : 0.0f;
+#pragma unroll
+              for (int j = 0; j < 32; ++j)
+                sum[cc][j] = __float_as_uint(((float)(int32_t)sum[cc][j] * rs) *
+                                             __shfl_sync(0xffffffffu, cs, j));
+            }
+            put_chunk(sum[cc], col0);
+          }
         }
       }
     }
@@ -553,18 +620,15 @@ __global__ void __cluster_dims__(CG, 1, 1) __launch_bounds__(kThreads, 1)
 }
 
 // Zero the C tiles that the split cuts (their pieces are added): block
-// (b - 1, part) looks at the start of worker b's share, and zeroes the tile
-// when that is the tile's first cut.  A programmatic dependent of the launch
-// before it that lets the tensor-core launch start once that one has
-// completed: its A and B are then final and only its writes of C wait.
+// (b - 1, part of kFillParts) looks at the start of worker b's share, and
+// zeroes its part of the tile when that is the tile's first cut.
+constexpr int kFillParts = 8;
 template <int NP>
-__global__ void __launch_bounds__(256)
-    dense_cut_fill_kernel(const __grid_constant__ DenseTable<NP> T, int CG, int TN) {
-  pdl_wait();
-  pdl_trigger();
-  const DensePos c = T.start[blockIdx.x + 1];
+__device__ __forceinline__ void fill_cut_tile(const DenseTable<NP>& T, int CG, int TN, int b,
+                                              int part) {
+  const DensePos c = T.start[b + 1];
   if (c.q >= T.split.count || c.slab == 0) return;
-  const DensePos prev = T.start[blockIdx.x];
+  const DensePos prev = T.start[b];
   if (prev.q == c.q && prev.tile == c.tile && prev.slab > 0) return;
   const DenseProb& P = T.p[c.q];
   if (P.accumulate) return;
@@ -574,7 +638,7 @@ __global__ void __launch_bounds__(256)
   const int64_t cols = P.N - n0 < TN ? P.N - n0 : TN;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const bool vec = P.tma_c && cols % 4 == 0;
-  for (int r = (int)blockIdx.y * 8 + warp; r < CG * kTM; r += (int)gridDim.y * 8) {
+  for (int r = part * 8 + warp; r < CG * kTM; r += kFillParts * 8) {
     const int copy = mt * CG + r / kTM;
     if (copy >= P.n_copy) continue;
     const int64_t row = (int64_t)__ldg(&P.tile_order[copy]) * kTM + r % kTM;
@@ -585,6 +649,78 @@ __global__ void __launch_bounds__(256)
         reinterpret_cast<uint4*>(dst)[i] = make_uint4(0, 0, 0, 0);
     } else {
       for (int64_t i = lane; i < cols; i += 32) dst[i] = 0.0f;
+    }
+  }
+}
+
+// A programmatic dependent of the launch before it that lets the tensor-core
+// launch start once that one has completed: its A and B are then final and
+// only its writes of C wait for this fill.
+template <int NP>
+__global__ void __launch_bounds__(256)
+    dense_cut_fill_kernel(const __grid_constant__ DenseTable<NP> T, int CG, int TN) {
+  pdl_wait();
+  pdl_trigger();
+  fill_cut_tile(T, CG, TN, (int)blockIdx.x / kFillParts, (int)blockIdx.x % kFillParts);
+}
+
+// INT8 -> BF16 (exact: |code| <= 127), K rows of N, into rows of ldo (a
+// multiple of 8), by blocks [0, gx * gy); the blocks after them zero the cut
+// tiles of C, so that an INT8 product has one launch ahead of the tensor-core
+// one.  Bound by its 3 bytes per value of memory traffic: a lane takes 8
+// consecutive codes (one 8-byte load: rows of B are 16-byte aligned; the last
+// group of a row is read code by code, since nothing past N may be), writes
+// 16 bytes, and has four rows in flight.  Code-by-code loads took 23 us for
+// 11008 x 2048, this 9.5.
+constexpr int kCvtRows = 4;
+struct Convert {
+  const int8_t* B;
+  __nv_bfloat16* out;
+  int64_t K, N, ldb, ldo;
+  int gx, gy;
+};
+__global__ void __launch_bounds__(256)
+    i8_prepare_kernel(const Convert c, const __grid_constant__ DenseTable<1> T, int CG, int TN) {
+  pdl_wait();
+  pdl_trigger();   // the launch after it waits in its own
+  const int bid = (int)blockIdx.x - c.gx * c.gy;
+  if (bid >= 0) {
+    fill_cut_tile(T, CG, TN, bid / kFillParts, bid % kFillParts);
+    return;
+  }
+  const int by = (int)blockIdx.x / c.gx, bx = (int)blockIdx.x - by * c.gx;
+  const int64_t c0 = ((int64_t)bx * 32 + (threadIdx.x & 31)) * 8;
+  if (c0 >= c.ldo) return;
+  const bool whole = c0 + 8 <= c.N;
+  for (int64_t k0 = ((int64_t)by * 8 + (threadIdx.x >> 5)) * kCvtRows; k0 < c.K;
+       k0 += (int64_t)c.gy * 8 * kCvtRows) {
+    uint2 v[kCvtRows];
+#pragma unroll
+    for (int i = 0; i < kCvtRows; ++i) {
+      v[i] = make_uint2(0u, 0u);
+      if (k0 + i >= c.K) break;
+      const int8_t* src = c.B + (k0 + i) * c.ldb + c0;
+      if (whole) {
+        v[i] = __ldg(reinterpret_cast<const uint2*>(src));
+      } else {
+        for (int j = 0; c0 + j < c.N; ++j) {
+          const uint32_t byte = (uint32_t)(uint8_t)src[j] << (8 * (j & 3));
+          if (j < 4) v[i].x |= byte;
+          else v[i].y |= byte;
+        }
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < kCvtRows; ++i) {
+      if (k0 + i >= c.K) break;
+      __nv_bfloat162 o[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const uint32_t w = j < 2 ? v[i].x : v[i].y;
+        const int sh = 16 * (j & 1);
+        o[j] = __floats2bfloat162_rn((float)(int8_t)(w >> sh), (float)(int8_t)(w >> (sh + 8)));
+      }
+      *reinterpret_cast<uint4*>(c.out + (k0 + i) * c.ldo + c0) = *reinterpret_cast<const uint4*>(o);
     }
   }
 }
@@ -603,19 +739,19 @@ size_t dense_smem_bytes() {
 
 int64_t slabs_of(int64_t K) { return (K + kTK - 1) / kTK; }
 
-template <int TN, int NP, int CG>
+template <int TN, int NP, int CG, bool I8>
 rosko_status launch_table(const DenseTable<NP>& T, cudaStream_t st) {
   constexpr int stages = dense_stages<TN, CG>();
   const size_t smem = dense_smem_bytes<TN, CG>();
   static bool set = false;
-  auto fn = dense_panel_kernel<TN, NP, CG>;
+  auto fn = dense_panel_kernel<TN, NP, CG, I8>;
   if (!set) {
     if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
         cudaSuccess)
       return ROSKO_ERR_CUDA;
     set = true;
   }
-  if (launch_dependent(fn, dim3((unsigned)(T.split.workers * CG)), dim3(kThreads), smem, st, T,
+  if (launch_dependent(fn, dim3((unsigned)(T.split.workers * CG)), dim3(kThreads<I8>), smem, st, T,
                        stages) != cudaSuccess)
     return ROSKO_ERR_CUDA;
   count_launches(1);
@@ -678,7 +814,8 @@ rosko_status encode_dense_maps(const DenseJob& j, CUtensorMap* mA, CUtensorMap* 
     const cuuint64_t strides[1] = {(cuuint64_t)j.ldc * 4};
     const cuuint32_t box[2] = {32, 32};
     const cuuint32_t es[2] = {1, 1};
-    if (encode_tiled(mC, j.out_i32 ? CU_TENSOR_MAP_DATA_TYPE_INT32 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32,
+    const bool i32 = j.i8 && !j.row_scale;
+    if (encode_tiled(mC, i32 ? CU_TENSOR_MAP_DATA_TYPE_INT32 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32,
                      2, j.C, dims, strides, box, es,
                      CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                      CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) !=
@@ -722,7 +859,7 @@ rosko_status encode_dense_maps(const DenseJob& j, CUtensorMap* mA, CUtensorMap* 
   return ROSKO_OK;
 }
 
-template <int TN, int NP, int CG>
+template <int TN, int NP, int CG, bool I8>
 rosko_status run_jobs(const DenseJob* jobs, int count, int ctas, bool zero_cut, bool after_fill,
                       cudaStream_t st) {
   static_assert(sizeof(DenseTable<NP>) <= 32 * 1024 - 256, "kernel parameter table too large");
@@ -750,41 +887,63 @@ rosko_status run_jobs(const DenseJob* jobs, int count, int ctas, bool zero_cut, 
     ++n;
   }
   for (int b = 0; b <= T.split.workers; ++b) T.start[b] = dense_pos(T.split, T.p, b);
-  T.kchunk = jobs[0].kchunk;
-  T.out_i32 = jobs[0].out_i32;
-  T.early_ab = zero_cut || after_fill ? 1 : 0;
+  T.row_scale = jobs[0].row_scale;
+  T.col_scale = jobs[0].col_scale;
+  T.early_ab = !I8 && (zero_cut || after_fill) ? 1 : 0;
   T.status = device_status_word();
   if (!T.status) return ROSKO_ERR_CUDA;
-  if (zero_cut) {
-    const dim3 grid((unsigned)std::max(1, T.split.workers - 1), 8);
-    if (launch_dependent(dense_cut_fill_kernel<NP>, grid, dim3(256), 0, st, T, CG, TN) !=
-        cudaSuccess)
+  const int fill_blocks = zero_cut ? std::max(1, T.split.workers - 1) * kFillParts : 0;
+  if constexpr (I8) {
+    // B to BF16, and the fill
+    const DenseJob& j = jobs[0];
+    Convert c;
+    c.B = j.src_i8;
+    c.out = static_cast<__nv_bfloat16*>(const_cast<void*>(j.B));
+    c.K = j.K;
+    c.N = j.N;
+    c.ldb = j.src_ld;
+    c.ldo = j.ldb;
+    c.gx = (int)((c.ldo / 8 + 31) / 32);
+    c.gy = (int)std::min<int64_t>((c.K + 8 * kCvtRows - 1) / (8 * kCvtRows), 4096);
+    if (launch_dependent(i8_prepare_kernel, dim3((unsigned)(c.gx * c.gy + fill_blocks)), dim3(256),
+                         0, st, c, T, CG, TN) != cudaSuccess)
+      return ROSKO_ERR_CUDA;
+    count_launches(1);
+  } else if (fill_blocks > 0) {
+    if (launch_dependent(dense_cut_fill_kernel<NP>, dim3((unsigned)fill_blocks), dim3(256), 0, st,
+                         T, CG, TN) != cudaSuccess)
       return ROSKO_ERR_CUDA;
     count_launches(1);
   }
-  return launch_table<TN, NP, CG>(T, st);
+  return launch_table<TN, NP, CG, I8>(T, st);
 }
 
 // CTAs per worker: pairs as soon as there are two row tiles to share and two
 // CTAs to run them (a pair over a single row tile would leave half of it idle).
 int group_of(int64_t n_tiles, int ctas) { return n_tiles >= 2 && ctas >= 2 ? 2 : 1; }
 
-template <int TN, int NP>
+template <int TN, int NP, bool I8>
 rosko_status dispatch_group(const DenseJob* jobs, int count, int cg, int ctas, bool zero_cut,
                             bool after_fill, cudaStream_t st) {
-  return cg == 2 ? run_jobs<TN, NP, 2>(jobs, count, ctas, zero_cut, after_fill, st)
-                 : run_jobs<TN, NP, 1>(jobs, count, ctas, zero_cut, after_fill, st);
+  return cg == 2 ? run_jobs<TN, NP, 2, I8>(jobs, count, ctas, zero_cut, after_fill, st)
+                 : run_jobs<TN, NP, 1, I8>(jobs, count, ctas, zero_cut, after_fill, st);
 }
 
 rosko_status dispatch_jobs(const DenseJob* jobs, int count, int TN, int cg, int ctas,
                            bool zero_cut, bool after_fill, cudaStream_t st) {
   if (count <= 0) return ROSKO_OK;
   if ((TN != 128 && TN != 256) || count > 64) return ROSKO_ERR_INVALID_ARG;
+  if (count == 1 && jobs[0].i8)
+    return TN == 256
+               ? dispatch_group<256, 1, true>(jobs, 1, cg, ctas, zero_cut, after_fill, st)
+               : dispatch_group<128, 1, true>(jobs, 1, cg, ctas, zero_cut, after_fill, st);
   if (count == 1)
-    return TN == 256 ? dispatch_group<256, 1>(jobs, 1, cg, ctas, zero_cut, after_fill, st)
-                     : dispatch_group<128, 1>(jobs, 1, cg, ctas, zero_cut, after_fill, st);
-  return TN == 256 ? dispatch_group<256, 64>(jobs, count, cg, ctas, zero_cut, after_fill, st)
-                   : dispatch_group<128, 64>(jobs, count, cg, ctas, zero_cut, after_fill, st);
+    return TN == 256
+               ? dispatch_group<256, 1, false>(jobs, 1, cg, ctas, zero_cut, after_fill, st)
+               : dispatch_group<128, 1, false>(jobs, 1, cg, ctas, zero_cut, after_fill, st);
+  return TN == 256
+             ? dispatch_group<256, 64, false>(jobs, count, cg, ctas, zero_cut, after_fill, st)
+             : dispatch_group<128, 64, false>(jobs, count, cg, ctas, zero_cut, after_fill, st);
 }
 
 }  // namespace
@@ -842,25 +1001,6 @@ __global__ void zero_fill_kernel(char* __restrict__ C, int64_t pitch, int64_t ro
   }
 }
 
-// INT8 -> BF16 (exact: |code| <= 127), K rows of N, into rows of ldo.
-__global__ void i8_to_bf16_kernel(const int8_t* __restrict__ B, int64_t K, int64_t N, int64_t ldb,
-                                  __nv_bfloat16* __restrict__ out, int64_t ldo) {
-  pdl_wait();
-  pdl_trigger();   // the launch after it waits in its own
-  const int64_t cols = (ldo + 3) / 4;   // four values per thread
-  const int64_t n = K * cols;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t k = i / cols, c0 = (i - k * cols) * 4;
-    __nv_bfloat16 v[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int64_t c = c0 + j;
-      v[j] = __float2bfloat16_rn(c < N ? (float)B[k * ldb + c] : 0.0f);
-      if (c < ldo) out[k * ldo + c] = v[j];
-    }
-  }
-}
 }  // namespace
 
 rosko_status zero_fill_launch(const ZeroFill& z, cudaStream_t st) {
@@ -883,14 +1023,10 @@ rosko_status zero_fill_launch(const ZeroFill& z, cudaStream_t st) {
   return cudaGetLastError() == cudaSuccess ? ROSKO_OK : ROSKO_ERR_CUDA;
 }
 
-// K slabs of 64 per exact chunk: 16 slabs = 1024 products of magnitude
-// <= 127^2, so a partial sum stays below 1024 * 16129 < 2^24 and is exact in
-// the FP32 accumulator.
-constexpr int kI8ChunkSlabs = 16;
-
 rosko_status dense_spmm_i8_launch(const rosko_packed_s* h, int64_t n_tiles, const int8_t* B,
-                                  int64_t N, int64_t ldb, int32_t* C, int64_t ldc, int TN,
-                                  int ctas, const ZeroFill* zf, cudaStream_t st) {
+                                  int64_t N, int64_t ldb, const float* col_scale, void* C,
+                                  int64_t ldc, int accumulate, int TN, int ctas, bool zero_cut,
+                                  const ZeroFill* zf, cudaStream_t st) {
   if (n_tiles <= 0 || N <= 0) return ROSKO_OK;
   if (ctas <= 0) ctas = num_sms();
   const int64_t K = h->K;
@@ -900,16 +1036,8 @@ rosko_status dense_spmm_i8_launch(const rosko_packed_s* h, int64_t n_tiles, cons
   // freed memory mapped: released after the launch that reads it
   if (pool_malloc(&scratch, (size_t)std::max<int64_t>(K * ldo, 1) * 2, st) != cudaSuccess)
     return ROSKO_ERR_OOM;
-  const int64_t work = K * ((ldo + 3) / 4);
-  const unsigned blocks = (unsigned)std::max<int64_t>(1, std::min<int64_t>((work + 255) / 256, 4096));
-  rosko_status s = launch_dependent(i8_to_bf16_kernel, dim3(blocks), dim3(256), 0, st, B, K, N, ldb,
-                                    static_cast<__nv_bfloat16*>(scratch), ldo) == cudaSuccess
-                       ? ROSKO_OK
-                       : ROSKO_ERR_CUDA;
-  count_launches(1);
-  // the zero fill of C (after the conversion, so that B is complete when the
-  // dependent tensor-core launch starts)
-  if (s == ROSKO_OK && zf) s = zero_fill_launch(*zf, st);
+  // the zero fill of all of C when the sparse panels need it too
+  rosko_status s = zf ? zero_fill_launch(*zf, st) : ROSKO_OK;
   if (s == ROSKO_OK) {
     DenseJob j;
     j.dense_A = h->dense_A;
@@ -921,13 +1049,16 @@ rosko_status dense_spmm_i8_launch(const rosko_packed_s* h, int64_t n_tiles, cons
     j.B = scratch;
     j.N = N;
     j.ldb = ldo;
-    j.C = reinterpret_cast<float*>(C);
+    j.C = static_cast<float*>(C);
     j.ldc = ldc;
     j.M = h->M;
-    j.accumulate = 1;   // every chunk adds into the zeroed (or accumulated) C
-    j.kchunk = kI8ChunkSlabs;
-    j.out_i32 = 1;
-    s = dispatch_jobs(&j, 1, TN, group_of(n_tiles, ctas), ctas, false, zf != nullptr, st);
+    j.accumulate = accumulate;
+    j.i8 = 1;
+    j.src_i8 = B;
+    j.src_ld = ldb;
+    j.row_scale = col_scale ? h->row_scale : nullptr;
+    j.col_scale = col_scale;
+    s = dispatch_jobs(&j, 1, TN, group_of(n_tiles, ctas), ctas, zero_cut, zf != nullptr, st);
   }
   pool_free(scratch, st);
   return s;
