@@ -49,9 +49,10 @@ struct SegEntry {
   uint32_t rec[12];
 };
 static_assert(sizeof(SegEntry) == 64, "a segment entry is 64 bytes");
-inline int64_t seg_records_for(int64_t nnz, int64_t M) {
+__host__ __device__ inline int64_t seg_records_for(int64_t nnz, int64_t M) {
   const int64_t twice_mean = M > 0 ? (2 * nnz + M - 1) / M : 0;
-  return std::max<int64_t>(kSegRecords, (twice_mean + 31) / 32 * 32);
+  const int64_t len = (twice_mean + 31) / 32 * 32;
+  return len > kSegRecords ? len : kSegRecords;
 }
 
 struct rosko_packed_s {
@@ -80,19 +81,20 @@ struct rosko_packed_s {
   // Row-direct work segments (row stream only), at two granularities: list
   // 0 cuts every row into pieces of at most kSegRecords nonzeros (many
   // warps for few or long rows), list 1 only rows longer than
-  // seg_records_for (twice the mean; few atomics for even matrices).  Per
-  // list: one SegEntry per segment (head = the record range of the piece in
-  // the row stream, sentinel excluded, and cut = 1 when the row has several
-  // pieces; then the piece's first records) in row order (nat) and in
-  // panel_order order (ord, packs with dense copies); prefix[i] / split[i]
-  // count the segments / the panels with a cut row among the first i panels
-  // of panel_order (or of the natural order without one).
-  // lpt: every segment of the list, longest piece first (ties in row
-  // order) - the order of a launch that runs all panels sparse, so that the
-  // longest pieces start first and the 8 items of a block have similar
-  // lengths (an inspector-executor ordering of the work, fixed at pack time).
+  // seg_records_for (twice the mean; few atomics for even matrices); where
+  // both lengths are the same the two share their arrays.  Per list: one
+  // SegEntry per segment (head = the record range of the piece in the row
+  // stream, sentinel excluded, and cut = 1 when the row has several pieces;
+  // then the piece's first records) in panel_order order (ord, packs with
+  // dense copies); prefix[i] / split[i] count the segments / the panels with
+  // a cut row among the first i panels of panel_order (or of the natural
+  // order without one).
+  // lpt: every segment of the list, longest pieces first (by length class,
+  // ties in row order) - the order of a launch that runs all panels sparse,
+  // so that the longest pieces start first and the 8 items of a block have
+  // similar lengths (an inspector-executor ordering of the work, fixed at
+  // pack time).
   struct SegList {
-    SegEntry* nat = nullptr;
     SegEntry* ord = nullptr;
     SegEntry* lpt = nullptr;
     std::vector<int64_t> prefix;

@@ -568,25 +568,215 @@ __global__ void fill_kernel(float* __restrict__ out, int64_t n, float v) {
     out[i] = v;
 }
 
+// ---- work segments of the row-direct traversal (see rosko_packed_s) --------
+// Planned on the device: the host only learns how many pieces each panel has.
+// (Planned on the host, the piece lists and their sorting took 266 us of the
+// 388 us pack of a 4608 x 512 matrix, and 1.9 of 2.7 ms for 11008 x 4096.)
+//
+// lpt order: pieces by length class, longest first, ties in row order.  A
+// class is a range of lengths (kSegClasses of them between the list's piece
+// length and 0), so the order is a stable counting sort: the summary kernel
+// counts each block's pieces per class, its last block turns the counts into
+// offsets, and the writing kernel ranks the pieces inside a block.
+constexpr int kSegRows = 256;      // rows per block of both kernels
+constexpr int kSegClasses = 64;
+
+__host__ __device__ inline int seg_class_shift(int seg) {
+  int s = 0;
+  while ((seg >> s) >= kSegClasses) ++s;
+  return s;
+}
+// Pieces of a row of nr nonzeros: the first ns - 1 hold seg records each, the
+// last one rem.
+struct RowPieces {
+  int ns, rem, cls;
+};
+__device__ __forceinline__ RowPieces row_pieces(int nr, int seg, int shift) {
+  RowPieces p;
+  p.ns = nr > seg ? (nr + seg - 1) / seg : 1;
+  p.rem = nr - (p.ns - 1) * seg;
+  p.cls = (seg - p.rem) >> shift;
+  return p;
+}
+
+// The counting half of the plan, run by pack_summary_kernel.
+struct SegCount {
+  const int2* rcnt;      // scanned row offsets; NULL: no row stream
+  int32_t* panel_segs;   // [2][P]: pieces of a panel, bit 31: a row of it is cut
+  int32_t* hist;         // [2][kSegClasses][nblk] counts, then exclusive offsets
+  int* ticket;           // blocks done (starts at 0)
+  int m_r, nblk;
+};
+
 // What the host needs to lay out the handle, gathered from the scans into one
 // array so that a single copy brings it back:
 //   sum64[0..3]    nonzeros, packed columns, touched columns, gather-union total
 //   sum64[4..4+P]  nonzero offset of every panel, then the total
-//   rowptr[0..M]   row-stream offsets (row stream only)
-__global__ void pack_summary_kernel(const int2* __restrict__ cnt, int64_t n, int64_t P, int64_t K,
-                                    const int* __restrict__ touched_total,
-                                    const int2* __restrict__ rcnt, int64_t M,
-                                    const int2* __restrict__ flag, int64_t nf,
-                                    int64_t* __restrict__ sum64, int32_t* __restrict__ rowptr) {
+//   panel_segs     per list and panel the work segments (row stream only)
+__global__ void __launch_bounds__(kSegRows)
+    pack_summary_kernel(const int2* __restrict__ cnt, int64_t n, int64_t P, int64_t K,
+                        const int* __restrict__ touched_total, int64_t M,
+                        const int2* __restrict__ flag, int64_t nf, int64_t* __restrict__ sum64,
+                        SegCount sc) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int nnz = cnt[n].x;
   if (i == 0) {
-    sum64[0] = cnt[n].x;
+    sum64[0] = nnz;
     sum64[1] = cnt[n].y;
     sum64[2] = *touched_total;
     sum64[3] = flag ? flag[nf].x : 0;
   }
-  if (i <= P) sum64[4 + i] = i < P ? cnt[i * K].x : cnt[n].x;
-  if (rcnt && i <= M) rowptr[i] = rcnt[i].x;
+  if (i <= P) sum64[4 + i] = i < P ? cnt[i * K].x : nnz;
+  if (!sc.rcnt || (int)blockIdx.x >= sc.nblk) return;   // uniform over the block
+  __shared__ int h[2 * kSegClasses];
+  __shared__ bool last;
+  if (threadIdx.x < 2 * kSegClasses) h[threadIdx.x] = 0;
+  __syncthreads();
+  const bool in = i < M;
+  const int nr = in ? sc.rcnt[i + 1].x - sc.rcnt[i].x - 1 : 0;
+#pragma unroll
+  for (int g = 0; g < 2; ++g) {
+    const int seg = g ? (int)seg_records_for(nnz, M) : kSegRecords;
+    RowPieces p = row_pieces(nr, seg, seg_class_shift(seg));
+    if (!in) p.ns = 0;
+    if (in) {
+      atomicAdd(&h[g * kSegClasses + p.cls], 1);
+      if (p.ns > 1) atomicAdd(&h[g * kSegClasses], p.ns - 1);
+    }
+    // the rows of a panel are m_r (8, 16 or 32) neighbouring lanes
+    int sum = p.ns, cut = p.ns > 1 ? 1 : 0;
+    for (int o = 1; o < sc.m_r; o <<= 1) {
+      sum += __shfl_xor_sync(0xffffffffu, sum, o);
+      cut |= __shfl_xor_sync(0xffffffffu, cut, o);
+    }
+    if (in && i % sc.m_r == 0)
+      sc.panel_segs[(int64_t)g * P + i / sc.m_r] = (int)((uint32_t)sum | ((uint32_t)cut << 31));
+  }
+  __syncthreads();
+  if (threadIdx.x < 2 * kSegClasses)
+    sc.hist[(int64_t)threadIdx.x * sc.nblk + blockIdx.x] = h[threadIdx.x];
+  // the last block turns each list's counts into offsets
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(sc.ticket, 1) == sc.nblk - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  const int64_t len = (int64_t)kSegClasses * sc.nblk;
+  const int64_t per = (len + kSegRows - 1) / kSegRows;
+  const int64_t j0 = min((int64_t)threadIdx.x * per, len), j1 = min(j0 + per, len);
+  int2 v = make_int2(0, 0);
+  for (int64_t j = j0; j < j1; ++j) {
+    v.x += __ldcg(&sc.hist[j]);
+    v.y += __ldcg(&sc.hist[len + j]);
+  }
+  int2 total;
+  int2 off = block_excl_scan(v, &total);
+  for (int64_t j = j0; j < j1; ++j) {
+    const int a = __ldcg(&sc.hist[j]), b = __ldcg(&sc.hist[len + j]);
+    sc.hist[j] = off.x;
+    sc.hist[len + j] = off.y;
+    off.x += a;
+    off.y += b;
+  }
+}
+
+// The writing half: the entries of every list (one when both piece lengths
+// are the same) from the row stream.  A block plans its 256 rows (a thread
+// per row and list), then each half-warp writes the entries of a row at a
+// time, one 4-byte word per lane: {row, first record, end record, cut} and
+// the piece's first 48 bytes of records (zero past its end).
+struct SegWrite {
+  const int2* rcnt;
+  const uint32_t* rnz;
+  const int32_t* hist;        // offsets of (class, block), per list
+  const int32_t* ord_base;    // [2][P]: first piece of a panel in panel order
+  SegEntry* ord[2];           // NULL: no panel order
+  SegEntry* lpt[2];
+  int64_t M, P;
+  int seg[2];
+  int rec_words, m_r, nblk, lists;
+};
+__global__ void __launch_bounds__(2 * kSegRows) seg_write_kernel(const SegWrite w) {
+  __shared__ int first[kSegRows], len[kSegRows];
+  __shared__ int at_full[2][kSegRows], at_rem[2][kSegRows], at_ord[2][kSegRows];
+  __shared__ int base[2][kSegRows / 32][kSegClasses];   // per warp and class
+  const int g = threadIdx.x >> 8, r = threadIdx.x & (kSegRows - 1);
+  const int wr = r >> 5, lane = threadIdx.x & 31;
+  const int64_t row = (int64_t)blockIdx.x * kSegRows + r;
+  const bool in = row < w.M && g < w.lists;
+  for (int i = threadIdx.x; i < 2 * (kSegRows / 32) * kSegClasses; i += 2 * kSegRows)
+    (&base[0][0][0])[i] = 0;
+  const int e0 = in ? w.rcnt[row].x : 0;
+  const int nr = in ? w.rcnt[row + 1].x - e0 - 1 : 0;
+  if (g == 0) {
+    first[r] = e0;
+    len[r] = in ? nr : -1;
+  }
+  __syncthreads();
+  const int seg = w.seg[g];
+  RowPieces p = row_pieces(nr, seg, seg_class_shift(seg));
+  if (!in) p.ns = 0;
+  // class 0 takes the row's full pieces (and its last one when that is in
+  // class 0 too); the other classes at most the last piece
+  const int n0 = in ? p.ns - 1 + (p.cls == 0 ? 1 : 0) : 0;
+  int incl = n0;
+  for (int o = 1; o < 32; o <<= 1) {
+    const int t = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += t;
+  }
+  const int key = in && p.cls > 0 ? p.cls : 0;
+  const unsigned same = __match_any_sync(0xffffffffu, key);
+  const int rank = __popc(same & ((1u << lane) - 1u));
+  if (key > 0 && rank == 0) base[g][wr][key] = __popc(same);
+  if (lane == 31) base[g][wr][0] = incl;
+  // this panel's pieces before this row
+  int before = p.ns;
+  for (int o = 1; o < w.m_r; o <<= 1) {
+    const int t = __shfl_up_sync(0xffffffffu, before, o);
+    if ((lane & (w.m_r - 1)) >= o) before += t;
+  }
+  before -= p.ns;
+  __syncthreads();
+  if (r < kSegClasses && g < w.lists) {
+    int at = w.hist[((int64_t)g * kSegClasses + r) * w.nblk + blockIdx.x];
+    for (int i = 0; i < kSegRows / 32; ++i) {
+      const int c = base[g][i][r];
+      base[g][i][r] = at;
+      at += c;
+    }
+  }
+  __syncthreads();
+  if (in) {
+    const int full0 = base[g][wr][0] + incl - n0;
+    at_full[g][r] = full0;
+    at_rem[g][r] = p.cls == 0 ? full0 + p.ns - 1 : base[g][wr][p.cls] + rank;
+    at_ord[g][r] = w.ord[g] ? w.ord_base[(int64_t)g * w.P + row / w.m_r] + before : 0;
+  }
+  __syncthreads();
+  const int l16 = threadIdx.x & 15;
+  const int words = 12 / w.rec_words * w.rec_words;   // inline words of whole records
+  for (int it = threadIdx.x >> 4; it < w.lists * kSegRows; it += 2 * kSegRows / 16) {
+    const int gg = it >> 8, rr = it & (kSegRows - 1);
+    const int n = len[rr];
+    if (n < 0) continue;
+    const int sg = w.seg[gg];
+    const int ns = n > sg ? (n + sg - 1) / sg : 1;
+    for (int k = 0; k < ns; ++k) {
+      const int a = first[rr] + k * sg;
+      const int e = k + 1 < ns ? a + sg : first[rr] + n;
+      uint32_t v = 0;
+      if (l16 == 0) v = (uint32_t)(blockIdx.x * kSegRows + rr);
+      else if (l16 == 1) v = (uint32_t)a;
+      else if (l16 == 2) v = (uint32_t)e;
+      else if (l16 == 3) v = ns > 1 ? 1u : 0u;
+      else if (l16 - 4 < words && l16 - 4 < (e - a) * w.rec_words)
+        v = w.rnz[(int64_t)a * w.rec_words + l16 - 4];
+      const int to = k + 1 < ns ? at_full[gg][rr] + k : at_rem[gg][rr];
+      reinterpret_cast<uint32_t*>(&w.lpt[gg][to])[l16] = v;
+      if (w.ord[gg]) reinterpret_cast<uint32_t*>(&w.ord[gg][at_ord[gg][rr] + k])[l16] = v;
+    }
+  }
 }
 
 // Dense-panel split bookkeeping (BF16 packs): 128-row tiles sorted by density,
@@ -628,80 +818,26 @@ void plan_dense_tiles(rosko_packed_s* h, int32_t dense_min_pm) {
   h->Kpad = (K + 7) / 8 * 8;
 }
 
-// Row-direct work segments (see rosko_packed_s) from the row-stream offsets,
-// at both granularities: {row, first record, end record, cut} in row order
-// (nat) and, with a panel order, in that order (ord).
-void plan_segments(rosko_packed_s* h, const int32_t* rp, const std::vector<int32_t>* panel_order,
-                   std::vector<int4> nat[2], std::vector<int4> ord[2], std::vector<int4> lpt[2]) {
-  const int64_t M = h->M, P = h->P;
-  const int64_t lens[2] = {kSegRecords, seg_records_for(h->nnz, M)};
+// The host's part of the work segments: per list the pieces and cut panels
+// among the first i panels of panel_order (or of the natural order), and each
+// panel's first piece in that order.
+void plan_segments(rosko_packed_s* h, const int32_t* panel_segs, bool panel_order,
+                   std::vector<int32_t>* ord_base) {
+  const int64_t P = h->P;
+  ord_base->assign((size_t)(2 * P), 0);
   for (int g = 0; g < 2; ++g) {
-    const int64_t seg = lens[g];
     rosko_packed_s::SegList& L = h->segs[g];
-    L.records = (int32_t)seg;
-    nat[g].reserve((size_t)M + (size_t)(h->nnz / seg) + 1);
-    std::vector<int64_t> panel_seg((size_t)P + 1, 0);
-    std::vector<char> panel_split((size_t)P, 0);
-    for (int64_t p = 0; p < P; ++p) {
-      panel_seg[(size_t)p] = (int64_t)nat[g].size();
-      for (int64_t r = p * h->m_r; r < std::min<int64_t>(M, (p + 1) * h->m_r); ++r) {
-        const int64_t nr = (int64_t)rp[r + 1] - rp[r] - 1;   // minus the sentinel
-        const int64_t ns = std::max<int64_t>(1, (nr + seg - 1) / seg);
-        if (ns > 1) panel_split[(size_t)p] = 1;
-        const int64_t row_end = (int64_t)rp[r + 1] - 1;
-        for (int64_t k = 0; k < ns; ++k) {
-          const int64_t e0 = (int64_t)rp[r] + k * seg;
-          // the entry's head; its inline records are written on the device
-          nat[g].push_back(make_int4((int)r, (int)e0, (int)std::min<int64_t>(e0 + seg, row_end),
-                                     ns > 1 ? 1 : 0));
-        }
-      }
-    }
-    panel_seg[(size_t)P] = (int64_t)nat[g].size();
+    L.records = g ? (int32_t)seg_records_for(h->nnz, h->M) : kSegRecords;
     L.prefix.assign((size_t)P + 1, 0);
     L.split.assign((size_t)P + 1, 0);
     for (int64_t i = 0; i < P; ++i) {
-      const int64_t p = panel_order ? (*panel_order)[(size_t)i] : i;
-      if (panel_order)
-        ord[g].insert(ord[g].end(), nat[g].begin() + panel_seg[(size_t)p],
-                      nat[g].begin() + panel_seg[(size_t)p + 1]);
-      L.prefix[(size_t)i + 1] = L.prefix[(size_t)i] + (panel_seg[(size_t)p + 1] - panel_seg[(size_t)p]);
-      L.split[(size_t)i + 1] = L.split[(size_t)i] + panel_split[(size_t)p];
+      const int64_t p = panel_order ? h->panel_order_host[(size_t)i] : i;
+      const uint32_t v = (uint32_t)panel_segs[(size_t)(g * P + p)];
+      (*ord_base)[(size_t)(g * P + p)] = (int32_t)L.prefix[(size_t)i];
+      L.prefix[(size_t)i + 1] = L.prefix[(size_t)i] + (int64_t)(v & 0x7FFFFFFFu);
+      L.split[(size_t)i + 1] = L.split[(size_t)i] + (int32_t)(v >> 31);
     }
-    lpt[g] = nat[g];
-    std::stable_sort(lpt[g].begin(), lpt[g].end(), [](const int4& a, const int4& b) {
-      return a.z - a.y > b.z - b.y;
-    });
   }
-}
-
-// The work segments' entries: each head (staged from the host, 16 bytes)
-// and the first 48 bytes of the piece's records in the row stream (written
-// by the phase-2 launch); one thread per (segment, 4-byte word: 4 of head,
-// 12 of records), over up to six lists.
-struct InlineLists {
-  SegEntry* list[6];
-  const int4* heads[6];
-  int64_t n[6];
-  int64_t first[7];   // first thread of each list
-};
-__global__ void seg_inline_kernel(InlineLists L, const uint32_t* __restrict__ rnz, int rec_words) {
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  int l = 0;
-  while (l < 5 && t >= L.first[l + 1]) ++l;
-  if (t >= L.first[6]) return;
-  const int64_t local = t - L.first[l];
-  const int64_t s = local / 16;
-  const int w = (int)(local - s * 16);
-  const int4 hd = L.heads[l][s];
-  SegEntry& e = L.list[l][s];
-  if (w < 4) {
-    reinterpret_cast<int*>(&e.head)[w] = w == 0 ? hd.x : (w == 1 ? hd.y : (w == 2 ? hd.z : hd.w));
-    return;
-  }
-  const int rw = w - 4;
-  const int64_t words = (int64_t)(hd.z - hd.y) * rec_words;
-  if (rw < words && rw / rec_words < 12 / rec_words) e.rec[rw] = rnz[(int64_t)hd.y * rec_words + rw];
 }
 
 // Bump allocator over byte offsets, each region 256-byte aligned.
@@ -747,11 +883,18 @@ rosko_status pack_typed(const S* A, int64_t lda, const float* scale_in, bool qua
   const size_t o_fsums = s.take((size_t)blocks_for(nf) * sizeof(int2));
   const size_t o_scale = s.take(quantize_rows ? (size_t)M * 4 : 0);
   const size_t o_sum64 = s.take((size_t)(P + 5) * 8);
-  const size_t o_rp = s.take(rows ? (size_t)(M + 1) * 4 : 0);
+  const size_t o_psegs = s.take(rows ? (size_t)(2 * P) * 4 : 0);
   const size_t summary_bytes = s.top - o_sum64;
+  const int64_t nblk = (M + kSegRows - 1) / kSegRows;
   PoolScratch scr;
   scr.st = st;
   if (pool_malloc(&scr.p, s.top + 256, st) != cudaSuccess) return ROSKO_ERR_OOM;
+  // the segment plan's class counts (packs with a row stream)
+  PoolScratch seg_scr;
+  seg_scr.st = st;
+  if (rows && pool_malloc(&seg_scr.p, (size_t)(2 * kSegClasses * nblk) * 4, st) != cudaSuccess)
+    return ROSKO_ERR_OOM;
+  int32_t* seg_hist = static_cast<int32_t*>(seg_scr.p);
   char* sb = static_cast<char*>(scr.p);
   int2* cnt = reinterpret_cast<int2*>(sb + o_cnt);
   int* touched = reinterpret_cast<int*>(sb + o_touch);
@@ -820,9 +963,18 @@ rosko_status pack_typed(const S* A, int64_t lda, const float* scale_in, bool qua
   }
   {
     const int64_t span = std::max<int64_t>(P, M) + 1;
-    pack_summary_kernel<<<(unsigned)((span + 255) / 256), 256, 0, st>>>(
-        cnt, n, P, K, tot + 2, rcnt, M, flag, nf, reinterpret_cast<int64_t*>(sb + o_sum64),
-        rows ? reinterpret_cast<int32_t*>(sb + o_rp) : nullptr);
+    SegCount sc;
+    std::memset(&sc, 0, sizeof(sc));
+    if (rows) {
+      sc.rcnt = rcnt;
+      sc.panel_segs = reinterpret_cast<int32_t*>(sb + o_psegs);
+      sc.hist = seg_hist;
+      sc.ticket = tot + 3;
+      sc.m_r = h->m_r;
+      sc.nblk = (int)nblk;
+    }
+    pack_summary_kernel<<<(unsigned)((span + kSegRows - 1) / kSegRows), kSegRows, 0, st>>>(
+        cnt, n, P, K, tot + 2, M, flag, nf, reinterpret_cast<int64_t*>(sb + o_sum64), sc);
     count_launches(1);
   }
   std::vector<int64_t> summary((summary_bytes + 7) / 8);
@@ -838,13 +990,15 @@ rosko_status pack_typed(const S* A, int64_t lda, const float* scale_in, bool qua
   h->touched_k = summary[2];
   h->gu_total = gather ? summary[3] : 0;
   h->panel_nnz.assign(summary.begin() + 4, summary.begin() + 5 + P);
-  const int32_t* rp =
-      rows ? reinterpret_cast<const int32_t*>(reinterpret_cast<const char*>(summary.data()) +
-                                              (o_rp - o_sum64))
-           : nullptr;
   if (dense) plan_dense_tiles(h, dense_min_pm);
-  std::vector<int4> nat[2], ord[2], lpt[2];
-  if (rows) plan_segments(h, rp, dense ? &h->panel_order_host : nullptr, nat, ord, lpt);
+  std::vector<int32_t> ord_base;
+  if (rows)
+    plan_segments(h,
+                  reinterpret_cast<const int32_t*>(reinterpret_cast<const char*>(summary.data()) +
+                                                   (o_psegs - o_sum64)),
+                  dense, &ord_base);
+  // both piece lengths the same: one list serves as both
+  const int lists = !rows ? 0 : (h->segs[0].records == h->segs[1].records ? 1 : 2);
 
   const size_t rsz = rec_size(h->dt);
   const int64_t nnz = h->nnz, n_cols = h->n_cols;
@@ -852,13 +1006,13 @@ rosko_status pack_typed(const S* A, int64_t lda, const float* scale_in, bool qua
   // staged from the host in one copy
   const size_t o_to = L.take(dense ? (size_t)T * 4 : 0);
   const size_t o_po = L.take(dense ? (size_t)P * 4 : 0);
+  const size_t o_ob = L.take(dense && rows ? ord_base.size() * 4 : 0);
   const size_t staged = L.top;
-  // written on the device (the segment entries: heads staged apart, below)
-  size_t o_seg[6];
-  for (int g = 0; g < 2; ++g) {
-    o_seg[3 * g] = L.take(nat[g].size() * sizeof(SegEntry));
-    o_seg[3 * g + 1] = L.take(ord[g].size() * sizeof(SegEntry));
-    o_seg[3 * g + 2] = L.take(lpt[g].size() * sizeof(SegEntry));
+  size_t o_ord[2] = {0, 0}, o_lpt[2] = {0, 0};
+  for (int g = 0; g < lists; ++g) {
+    const size_t bytes = (size_t)h->segs[g].prefix[(size_t)P] * sizeof(SegEntry);
+    o_ord[g] = L.take(dense ? bytes : 0);
+    o_lpt[g] = L.take(bytes);
   }
   // written on the device
   const size_t o_pc = L.take((size_t)(P + 1) * 4);
@@ -887,9 +1041,9 @@ rosko_status pack_typed(const S* A, int64_t lda, const float* scale_in, bool qua
     h->rowptr = reinterpret_cast<int32_t*>(b + o_rowptr);
     h->rnz = b + o_rnz;
     for (int g = 0; g < 2; ++g) {
-      h->segs[g].nat = reinterpret_cast<SegEntry*>(b + o_seg[3 * g]);
-      h->segs[g].ord = dense ? reinterpret_cast<SegEntry*>(b + o_seg[3 * g + 1]) : nullptr;
-      h->segs[g].lpt = reinterpret_cast<SegEntry*>(b + o_seg[3 * g + 2]);
+      const int l = g < lists ? g : 0;
+      h->segs[g].ord = dense ? reinterpret_cast<SegEntry*>(b + o_ord[l]) : nullptr;
+      h->segs[g].lpt = reinterpret_cast<SegEntry*>(b + o_lpt[l]);
     }
   }
   if (gather) {
@@ -907,35 +1061,10 @@ rosko_status pack_typed(const S* A, int64_t lda, const float* scale_in, bool qua
     if (dense) {
       std::memcpy(stage.data() + o_to, h->tile_order.data(), (size_t)T * 4);
       std::memcpy(stage.data() + o_po, h->panel_order_host.data(), (size_t)P * 4);
+      if (rows) std::memcpy(stage.data() + o_ob, ord_base.data(), ord_base.size() * 4);
     }
     // a pageable source is staged before the call returns
     if (cudaMemcpyAsync(b, stage.data(), staged, cudaMemcpyHostToDevice, st) != cudaSuccess)
-      return ROSKO_ERR_CUDA;
-  }
-  // the segment heads (16 bytes each; the entries' inline records are
-  // filled on the device) go to stream-ordered scratch from the library's
-  // pool (it keeps freed memory mapped: the default pool would map it anew
-  // on every pack), released after the launch that expands them
-  size_t n_heads = 0;
-  for (int g = 0; g < 2; ++g) n_heads += nat[g].size() + ord[g].size() + lpt[g].size();
-  std::vector<int4> heads;
-  heads.reserve(n_heads);
-  for (int g = 0; g < 2; ++g)
-    for (const std::vector<int4>* v : {&nat[g], &ord[g], &lpt[g]}) heads.insert(heads.end(), v->begin(), v->end());
-  struct Scratch {
-    void* p = nullptr;
-    cudaStream_t st;
-    ~Scratch() {
-      if (p) pool_free(p, st);
-    }
-  } heads_dev{nullptr, st};
-  if (n_heads > 0) {
-    if (pool_malloc(&heads_dev.p, n_heads * sizeof(int4), st) != cudaSuccess) {
-      heads_dev.p = nullptr;
-      return ROSKO_ERR_OOM;
-    }
-    if (cudaMemcpyAsync(heads_dev.p, heads.data(), n_heads * sizeof(int4), cudaMemcpyHostToDevice,
-                        st) != cudaSuccess)
       return ROSKO_ERR_CUDA;
   }
 
@@ -990,31 +1119,26 @@ rosko_status pack_typed(const S* A, int64_t lda, const float* scale_in, bool qua
           A, geo, scale, w);
   count_launches(1);
   if (rows) {
-    // the segments' inline records, once the row stream is written
-    InlineLists il;
-    std::memset(&il, 0, sizeof(il));
-    int nl = 0;
-    // heads are staged in the order nat, ord, lpt of list 0, then of list 1
-    const int4* hp = static_cast<const int4*>(heads_dev.p);
+    // the work segments, once the row stream is written
+    SegWrite sw;
+    std::memset(&sw, 0, sizeof(sw));
+    sw.rcnt = rcnt;
+    sw.rnz = static_cast<const uint32_t*>(h->rnz);
+    sw.hist = seg_hist;
+    sw.ord_base = dense ? reinterpret_cast<const int32_t*>(b + o_ob) : nullptr;
     for (int g = 0; g < 2; ++g) {
-      SegEntry* dst[3] = {h->segs[g].nat, h->segs[g].ord, h->segs[g].lpt};
-      const std::vector<int4>* src[3] = {&nat[g], &ord[g], &lpt[g]};
-      for (int k = 0; k < 3; ++k) {
-        if (dst[k] && !src[k]->empty()) {
-          il.list[nl] = dst[k];
-          il.heads[nl] = hp;
-          il.n[nl++] = (int64_t)src[k]->size();
-        }
-        hp += src[k]->size();
-      }
+      sw.ord[g] = h->segs[g].ord;
+      sw.lpt[g] = h->segs[g].lpt;
+      sw.seg[g] = h->segs[g].records;
     }
-    il.first[0] = 0;
-    for (int l = 0; l < 6; ++l) il.first[l + 1] = il.first[l] + (l < nl ? il.n[l] * 16 : 0);
-    if (il.first[6] > 0) {
-      seg_inline_kernel<<<(unsigned)((il.first[6] + 255) / 256), 256, 0, st>>>(
-          il, static_cast<const uint32_t*>(h->rnz), (int)(rsz / 4));
-      count_launches(1);
-    }
+    sw.M = M;
+    sw.P = P;
+    sw.rec_words = (int)(rsz / 4);
+    sw.m_r = h->m_r;
+    sw.nblk = (int)nblk;
+    sw.lists = lists;
+    seg_write_kernel<<<(unsigned)nblk, 2 * kSegRows, 0, st>>>(sw);
+    count_launches(1);
   }
   // the scratch is released on return: wait for the writes that read it
   if (cudaStreamSynchronize(st) != cudaSuccess || cudaGetLastError() != cudaSuccess)

@@ -44,8 +44,10 @@ uint64_t fnv1a(const unsigned char* p, size_t n, uint64_t h = 146959810393466560
   return h;
 }
 
-// The device pointers of a handle, in image order.
-void** ptr_slots(rosko_packed_s* h, void** slots[kNumPtrs]) {
+// The device pointers of a handle, in image order.  Slots 14 and 16 of the
+// format once held the segments in row order, which no launch reads: an image
+// may give them, this library writes them empty.
+void** ptr_slots(rosko_packed_s* h, void** slots[kNumPtrs], void** unused) {
   int i = 0;
   slots[i++] = reinterpret_cast<void**>(&h->panel_col);
   slots[i++] = reinterpret_cast<void**>(&h->colrec);
@@ -61,9 +63,9 @@ void** ptr_slots(rosko_packed_s* h, void** slots[kNumPtrs]) {
   slots[i++] = &h->dense_A;
   slots[i++] = reinterpret_cast<void**>(&h->tile_order_dev);
   slots[i++] = reinterpret_cast<void**>(&h->panel_order_dev);
-  slots[i++] = reinterpret_cast<void**>(&h->segs[0].nat);
+  slots[i++] = unused;
   slots[i++] = reinterpret_cast<void**>(&h->segs[0].ord);
-  slots[i++] = reinterpret_cast<void**>(&h->segs[1].nat);
+  slots[i++] = unused;
   slots[i++] = reinterpret_cast<void**>(&h->segs[1].ord);
   slots[i++] = reinterpret_cast<void**>(&h->segs[0].lpt);
   slots[i++] = reinterpret_cast<void**>(&h->segs[1].lpt);
@@ -109,7 +111,8 @@ rosko_status packed_serialize(const rosko_packed_s* hc, void* buf, int64_t cap, 
   H.Kpad = h->Kpad;
   H.base_bytes = h->base_bytes;
   void** slots[kNumPtrs];
-  ptr_slots(h, slots);
+  void* unused = nullptr;
+  ptr_slots(h, slots, &unused);
   for (int i = 0; i < kNumPtrs; ++i) {
     const char* p = static_cast<const char*>(*slots[i]);
     H.ptr_off[i] = p ? (int64_t)(p - static_cast<const char*>(h->base)) : -1;
@@ -211,7 +214,8 @@ rosko_status packed_deserialize(const void* vbuf, int64_t size, cudaStream_t st,
   }
   h->base_bytes = H.base_bytes;
   void** slots[kNumPtrs];
-  ptr_slots(h, slots);
+  void* unused = nullptr;
+  ptr_slots(h, slots, &unused);
   for (int i = 0; i < kNumPtrs; ++i)
     *slots[i] = H.ptr_off[i] < 0 ? nullptr : static_cast<char*>(h->base) + H.ptr_off[i];
   // a pageable source: the copy is complete when the call returns

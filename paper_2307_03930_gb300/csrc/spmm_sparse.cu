@@ -1004,18 +1004,13 @@ const SegEntry* direct_segments(const rosko_packed_s* h, const int32_t* panel_li
   if (cut) *cut = false;
   *n_segs = -1;
   const rosko_packed_s::SegList& L = h->segs[which & 1];
-  if (!L.nat || n_panels < 0 || n_panels > h->P) return nullptr;
+  if (!L.lpt || n_panels < 0 || n_panels > h->P) return nullptr;
   const SegEntry* base;
-  if (n_panels == h->P && L.lpt && (!panel_list || panel_list == h->panel_order_dev)) {
+  if (n_panels == h->P && (!panel_list || panel_list == h->panel_order_dev)) {
     // every panel runs sparse: any order of all segments covers them, and
     // the longest-first order balances the launch
     base = L.lpt;
-  } else if (!panel_list) {
-    // all panels in order (the prefix sums' last entry is the total in
-    // either order)
-    if (n_panels != h->P) return nullptr;
-    base = L.nat;
-  } else if (panel_list == h->panel_order_dev && L.ord) {
+  } else if (panel_list && panel_list == h->panel_order_dev && L.ord) {
     base = L.ord;
   } else {
     return nullptr;
