@@ -21,7 +21,7 @@
 // L2 -> SM traffic falls by the same third.  The smaller stages also make the
 // ring six slabs deep instead of four.
 //
-// Warp roles: 0 = TMA producer, 1 = MMA issuer (and TMEM owner), 2.. =
+// Warp roles: 0 = TMA producer, 1 = MMA issuer (and TMEM owner), 4-11 =
 // epilogue (warp w reads TMEM lanes 32 (w % 4) .. 32 (w % 4) + 31).  The
 // producer and MMA warps wait as whole warps and one elected lane issues
 // (elect.sync, see elect_one: with a plain `lane == 0` branch a slab's four
@@ -50,15 +50,14 @@
 // at a time into a 32 x 32 FP32 staging tile in shared memory (128-byte
 // swizzle, so the row-per-lane writes are bank-conflict free) and one lane
 // hands the tile to TMA: a tensor store for a whole tile, a tensor
-// reduce-add (element-wise add in L2) for a cut tile or C += A.B.  Two
-// staging tiles per warp let the next chunk's TMEM load overlap the copy.
+// reduce-add (element-wise add in L2) for a cut tile or C += A.B.
 //
-// INT8 packs run through the same BF16 pipe (GB300's INT8 tensor rate is far
-// below it): the codes are exact in BF16, and accumulators end every
-// kI8ChunkSlabs K slabs, where every FP32 partial sum is still an exact
-// integer.  The epilogue converts each chunk and sums it in INT32 registers
-// while the next chunk's MMAs run, and writes C once per range: INT32, or
-// FP32 times the row and column scales.  (Adding every chunk into INT32 C in
+// Accumulators end every kChunkSlabs K slabs; the epilogue adds each chunk to
+// its sums in registers while the next chunk's MMAs run, and writes C once
+// per range.  INT8 packs run through the same BF16 pipe (GB300's INT8 tensor
+// rate is far below it): the codes are exact in BF16, every chunk's FP32 sum
+// is still an exact integer and is converted and summed in INT32; C is INT32,
+// or FP32 times the row and column scales.  (Adding every chunk into INT32 C in
 // global memory instead cost an epilogue per 1,024 K: 162 against 115 us for
 // 4096x11008x2048, and kept the scaled result off the tensor cores.)
 // C whose rows are not 16-byte aligned falls back to direct stores and
@@ -77,19 +76,30 @@ constexpr int kTM = 128;             // rows of a dense tile
 constexpr int kTK = 64;              // K per stage: 64 BF16 = one 128-byte swizzle row
 constexpr uint32_t kABytes = kTM * kTK * 2;   // 16 KB
 constexpr uint32_t kStageC = 32 * 32 * 4;      // one 32 x 32 FP32 staging tile
-// Epilogue warps: 4 (one per TMEM lane quarter), two staging tiles each.
-// Eight warps ran the epilogue in the same time (it is bound by the TMA
-// stores and L2 reductions, ~28 bytes per cycle per SM, not by the warps).
-// INT8 packs (I8) take eight, two per quarter with half of the columns each:
-// their 128 columns of INT32 sums per lane live in registers.
-template <bool I8> constexpr int kEpiWarps = I8 ? 8 : 4;
-template <bool I8> constexpr int kThreads = 64 + 32 * kEpiWarps<I8>;
-constexpr int kStageTiles = 8;                 // staging tiles of all warps
-constexpr uint32_t kEpiBytes = kStageTiles * kStageC;
-// INT8 codes: K slabs of 64 per exact chunk.  16 slabs = 1024 products of
-// magnitude <= 127^2, so a partial sum stays below 1024 * 16129 < 2^24 and is
-// exact in the FP32 accumulator.
-constexpr int kI8ChunkSlabs = 16;
+// Epilogue warps: two per TMEM lane quarter, each with half of the columns:
+// the 128 columns of sums per lane of a 256-column tile live in registers.
+constexpr int kEpiWarps = 8;
+constexpr uint32_t kEpiBytes = kEpiWarps * kStageC;   // a staging tile each
+// Warps 0-3 (producer, MMA issuer, two idle) give registers to the epilogue's
+// two warpgroups: 128 sums and what the stores need do not fit the 168 that
+// 384 threads can get at launch (they spilled: 108 against 98 us for
+// 11008x4096x2048).  152 at launch leave room on an SM for a block of the next
+// call's zero fill, which so starts before this grid has ended (1 us of a
+// 512x4608x3136 call).  The shares add up to no more than the launch's total.
+constexpr int kFirstEpi = 4;
+constexpr int kThreads = 32 * (kFirstEpi + kEpiWarps);
+constexpr int kRegsLaunch = 152, kRegsRest = 56, kRegsEpi = 200;
+static_assert(128 * kRegsRest + 32 * kEpiWarps * kRegsEpi <= kThreads * kRegsLaunch,
+              "setmaxnreg would wait for registers that the block does not have");
+// K slabs of 64 that one accumulator sums before the epilogue takes it over
+// into registers.  INT8 codes: 16 slabs = 1024 products of magnitude <= 127^2,
+// so a partial sum stays below 1024 * 16129 < 2^24 and is exact in the FP32
+// accumulator.  BF16: the tensor core truncates each addition, an error that
+// grows with the length of the chain (2048x4096x2048 at 50 %, against 64
+// bits: 2.1e-6 in chains of 54 slabs, 1.0e-6 of 27); chunks of 16 slabs added
+// with round-to-nearest keep it below 1e-6 whatever K and the split are, and
+// draining them costs nothing (the MMAs of the next chunk run meanwhile).
+constexpr int kChunkSlabs = 16;
 // A tile's cost in K slabs is at least its epilogue's time (128 KB per
 // 128 x 256 accumulator at ~28 B/clk: about nine slabs of 512 cycles; the
 // same ratio for 128-column tiles).
@@ -243,7 +253,7 @@ struct SegIter {
 };
 
 template <int TN, int NP, int CG, bool I8>
-__global__ void __cluster_dims__(CG, 1, 1) __launch_bounds__(kThreads<I8>, 1)
+__global__ void __cluster_dims__(CG, 1, 1) __maxnreg__(kRegsLaunch)
     dense_panel_kernel(const __grid_constant__ DenseTable<NP> T, int S) {
   constexpr int BN = TN / CG;                             // B columns this CTA loads
   constexpr uint32_t kBBytes = (uint32_t)BN * kTK * 2;
@@ -279,7 +289,7 @@ __global__ void __cluster_dims__(CG, 1, 1) __launch_bounds__(kThreads<I8>, 1)
       }
       for (int b = 0; b < 2; ++b) {
         mbar_init(&acc_full[b], 1);
-        mbar_init(&acc_empty[b], CG * kEpiWarps<I8>);
+        mbar_init(&acc_empty[b], CG * kEpiWarps);
       }
       fence_barrier_init();
     }
@@ -298,12 +308,14 @@ __global__ void __cluster_dims__(CG, 1, 1) __launch_bounds__(kThreads<I8>, 1)
   DenseSeg sg;
   if constexpr (CG == 2) cluster_wait();
   uint32_t tmem = 0;
-  if (warp != 0) {
-    asm volatile("bar.sync 1, %0;" ::"n"(kThreads<I8> - 32) : "memory");
+  if (warp == 1 || warp >= kFirstEpi) {
+    asm volatile("bar.sync 1, %0;" ::"n"(32 * (1 + kEpiWarps)) : "memory");
     tc::fence_after_sync();
     tmem = *tmem_slot;
   }
 
+  if (warp < kFirstEpi) {
+  asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsRest));
   if (warp == 0) {
     // ---------------- TMA producer -----------------------------------------
     if (!T.early_ab) pdl_wait();   // A and B may be the previous launch's output
@@ -394,7 +406,7 @@ __global__ void __cluster_dims__(CG, 1, 1) __launch_bounds__(kThreads<I8>, 1)
     while (rank == 0 && ok && it.next(sg)) {
       for (int c0 = sg.s0; ok && c0 < sg.s1;) {
         // slabs [c0, c1) sum in one accumulator
-        const int c1 = I8 ? min(sg.s1, c0 + kI8ChunkSlabs) : sg.s1;
+        const int c1 = min(sg.s1, c0 + kChunkSlabs);
         if (++b == NBUF) {
           b = 0;
           bph ^= 1u;
@@ -437,20 +449,20 @@ __global__ void __cluster_dims__(CG, 1, 1) __launch_bounds__(kThreads<I8>, 1)
       for (int j = 0; j < NBUF; ++j) tc::mma_commit<CG>(&acc_full[j]);
     }
     __syncwarp();
+  }
   } else {
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsEpi));
     // ---------------- epilogue: TMEM -> registers -> C -----------------------
     // C may still be being zero-filled by the kernel this launch depends on
     // (programmatic dependent launch): wait for it before any write to C.
     // Without such a dependency the wait returns at once.
     pdl_wait();
     const int quarter = warp & 3;                  // TMEM lanes 32 quarter .. + 31
-    constexpr int kParts = kEpiWarps<I8> / 4;      // warps that share a quarter
+    constexpr int kParts = kEpiWarps / 4;      // warps that share a quarter
     constexpr int kChunks = TN / 32 / kParts;      // 32-column chunks of a warp
-    constexpr int kStagePerWarp = kStageTiles / kEpiWarps<I8>;
-    const int part = (warp - 2) >> 2;              // column part of this warp
-    uint8_t* my_stage = stage_c + (size_t)(warp - 2) * kStagePerWarp * kStageC;
+    const int part = (warp - kFirstEpi) >> 2;              // column part of this warp
+    uint8_t* my_stage = stage_c + (size_t)(warp - kFirstEpi) * kStageC;
     const uint32_t drained = CG == 2 ? cluster_addr(acc_empty, 0) : 0u;
-    int chunk = 0;   // staging tiles alternate per chunk
     int b = NBUF - 1;
     uint32_t bph = 1;
     const bool i32 = I8 && !T.row_scale;
@@ -474,28 +486,52 @@ __global__ void __cluster_dims__(CG, 1, 1) __launch_bounds__(kThreads<I8>, 1)
       }
     };
     while (it.next(sg)) {
+      const int copy = sg.mt * CG + rank;
+      // the tile's C rows, fetched while the MMAs run (what else the stores
+      // need is read after the sums: registers are short until then)
+      const int trow = copy < T.p[sg.q].n_copy ? __ldg(&T.p[sg.q].tile_order[copy]) : -1;
+      // the range's sums (FP32 or INT32 bits); at the end, in place, the bits
+      // that go to C
+      uint32_t sum[kChunks][32];
+#pragma unroll
+      for (int cc = 0; cc < kChunks; ++cc)
+#pragma unroll
+        for (int j = 0; j < 32; ++j) sum[cc][j] = 0;
+      bool ok = true;
+      for (int c0 = sg.s0; c0 < sg.s1; c0 += kChunkSlabs) {
+        ok = wait_acc() && ok;
+#pragma unroll
+        for (int h = 0; h < 2 * kChunks; ++h) {
+          uint32_t r[16];
+          tc::tmem_ld_32x32b_x16(my_tmem + (uint32_t)(b * TN + part * kChunks * 32 + h * 16), r);
+          tc::tmem_ld_wait();
+#pragma unroll
+          for (int j = 0; j < 16; ++j) {
+            uint32_t& t = sum[h / 2][(h & 1) * 16 + j];
+            // (INT8: an exact integer in FP32, |partial| < 2^24)
+            if constexpr (I8) t += (uint32_t)__float2int_rn(__uint_as_float(r[j]));
+            else t = __float_as_uint(__uint_as_float(t) + __uint_as_float(r[j]));
+          }
+        }
+        release_acc();
+      }
       const DenseProb& P = T.p[sg.q];
       const int q = sg.q;
-      const int copy = sg.mt * CG + rank;
-      // the tile's C rows, fetched while the MMAs run
-      const int trow = copy < P.n_copy ? __ldg(&P.tile_order[copy]) : 0;
-      // the problem's scalars in registers for the chunk loop
-      const int64_t PM = P.M, PN = P.N;
-      const int64_t row0 = (int64_t)trow * kTM + quarter * 32;
-      const bool rows_ok = copy < P.n_copy && row0 < PM;
+      const int PM = P.M, PN = P.N;
+      const int row0 = trow * kTM + quarter * 32;
+      const bool rows_ok = trow >= 0 && row0 < PM;
       const int tma_c = P.tma_c;
       const bool add = !sg.whole || P.accumulate;
-      const int64_t n0 = (int64_t)sg.nt * TN;
+      const int n0 = sg.nt * TN;
       const int64_t ldc = P.ldc;
-      float* c_row0 = P.C + row0 * ldc + lane;   // this lane's column of a chunk
+      float* c_row0 = P.C + (int64_t)row0 * ldc + lane;   // this lane's column of a chunk
       // write (or add) the 32 x 32 chunk at column col0: r[j] of lane i is
       // the value (FP32 or INT32 bits) of row row0 + i, column col0 + j
-      auto put_chunk = [&](const uint32_t (&r)[32], int64_t col0) {
+      auto put_chunk = [&](const uint32_t (&r)[32], int col0) {
         if (tma_c) {
-          // staging tile (chunk % n) is free once the copy issued n chunks
-          // ago has read it
-          uint8_t* buf = my_stage + (size_t)(chunk % kStagePerWarp) * kStageC;
-          if (lane == 0) bulk_wait_read<kStagePerWarp - 1>();
+          // the staging tile is free once the last copy has read it
+          uint8_t* buf = my_stage;
+          if (lane == 0) bulk_wait_read<0>();
           __syncwarp();
           // row `lane`, 16-byte chunk j at (j ^ (lane % 8)): the 128-byte swizzle
 #pragma unroll
@@ -506,11 +542,10 @@ __global__ void __cluster_dims__(CG, 1, 1) __launch_bounds__(kThreads<I8>, 1)
           __syncwarp();
           if (lane == 0) {
             // rows past M and columns past N are clipped by the tensor map
-            if (add) tma_reduce_add_2d(&T.tmC[q], (int32_t)col0, (int32_t)row0, buf);
-            else tma_store_2d(&T.tmC[q], (int32_t)col0, (int32_t)row0, buf);
+            if (add) tma_reduce_add_2d(&T.tmC[q], col0, row0, buf);
+            else tma_store_2d(&T.tmC[q], col0, row0, buf);
             bulk_commit();
           }
-          ++chunk;
           return;
         }
         // C rows not 16-byte aligned (no tensor map): transpose the 32 x 32
@@ -526,7 +561,7 @@ __global__ void __cluster_dims__(CG, 1, 1) __launch_bounds__(kThreads<I8>, 1)
 #pragma unroll
         for (int j = 0; j < 32; ++j) tr[lane * 32 + ((j + lane) & 31)] = r[j];
         __syncwarp();
-        const int rows = (int)(PM - row0 < 32 ? PM - row0 : 32);
+        const int rows = PM - row0 < 32 ? PM - row0 : 32;
         if (col0 + lane < PN) {
           // eight rows at a time: their shared-memory reads, then their stores
           float* dst = c_row0 + col0;
@@ -551,55 +586,20 @@ __global__ void __cluster_dims__(CG, 1, 1) __launch_bounds__(kThreads<I8>, 1)
         }
         __syncwarp();
       };
-      if constexpr (!I8) {
-        const bool ok = wait_acc();
-#pragma unroll 1
-        for (int cc = 0; cc < kChunks; ++cc) {
-          const int64_t col0 = n0 + cc * 32;
-          if (!ok || !rows_ok || col0 >= PN) break;   // warp-uniform
-          uint32_t r[32];
-          tc::tmem_ld_32x32b_x32(my_tmem + (uint32_t)(b * TN + cc * 32), r);
-          tc::tmem_ld_wait();
-          put_chunk(r, col0);
-        }
-        release_acc();
-      } else {
-        // INT32 sums; at the end, in place, the bits that go to C
-        uint32_t sum[kChunks][32];
+      float rs = 0.0f;
+      if (I8 && !i32 && rows_ok && row0 + lane < PM) rs = __ldg(&T.row_scale[row0 + lane]);
 #pragma unroll
-        for (int cc = 0; cc < kChunks; ++cc)
+      for (int cc = 0; cc < kChunks; ++cc) {
+        const int col0 = n0 + (part * kChunks + cc) * 32;
+        if (ok && rows_ok && col0 < PN) {   // warp-uniform
+          if (I8 && !i32) {
+            const float cs = col0 + lane < PN ? __ldg(&T.col_scale[col0 + lane]) : 0.0f;
 #pragma unroll
-          for (int j = 0; j < 32; ++j) sum[cc][j] = 0;
-        bool ok = true;
-        for (int c0 = sg.s0; c0 < sg.s1; c0 += kI8ChunkSlabs) {
-          ok = wait_acc() && ok;
-#pragma unroll
-          for (int h = 0; h < 2 * kChunks; ++h) {
-            uint32_t r[16];
-            tc::tmem_ld_32x32b_x16(
-                my_tmem + (uint32_t)(b * TN + part * kChunks * 32 + h * 16), r);
-            tc::tmem_ld_wait();
-            // an exact integer in FP32 (|partial| < 2^24)
-#pragma unroll
-            for (int j = 0; j < 16; ++j)
-              sum[h / 2][(h & 1) * 16 + j] += (uint32_t)__float2int_rn(__uint_as_float(r[j]));
+            for (int j = 0; j < 32; ++j)
+              sum[cc][j] = __float_as_uint(((float)(int32_t)sum[cc][j] * rs) *
+                                           __shfl_sync(0xffffffffu, cs, j));
           }
-          release_acc();
-        }
-        const float rs = !i32 && rows_ok && row0 + lane < PM ? __ldg(&T.row_scale[row0 + lane]) : 0.0f;
-#pragma unroll
-        for (int cc = 0; cc < kChunks; ++cc) {
-          const int64_t col0 = n0 + (part * kChunks + cc) * 32;
-          if (ok && rows_ok && col0 < PN) {   // warp-uniform
-            if (!i32) {
-              const float cs = col0 + lane < PN ? __ldg(&T.col_scale[col0 + lane]) : 0.0f;
-#pragma unroll
-              for (int j = 0; j < 32; ++j)
-                sum[cc][j] = __float_as_uint(((float)(int32_t)sum[cc][j] * rs) *
-                                             __shfl_sync(0xffffffffu, cs, j));
-            }
-            put_chunk(sum[cc], col0);
-          }
+          put_chunk(sum[cc], col0);
         }
       }
     }
@@ -623,6 +623,7 @@ __global__ void __cluster_dims__(CG, 1, 1) __launch_bounds__(kThreads<I8>, 1)
 // (b - 1, part of kFillParts) looks at the start of worker b's share, and
 // zeroes its part of the tile when that is the tile's first cut.
 constexpr int kFillParts = 8;
+constexpr int kFillThreads = 128;   // few registers a block: see kRegsLaunch
 template <int NP>
 __device__ __forceinline__ void fill_cut_tile(const DenseTable<NP>& T, int CG, int TN, int b,
                                               int part) {
@@ -636,9 +637,9 @@ __device__ __forceinline__ void fill_cut_tile(const DenseTable<NP>& T, int CG, i
   dense_tile_at(P, c.tile, &mt, &nt);
   const int64_t n0 = (int64_t)nt * TN;
   const int64_t cols = P.N - n0 < TN ? P.N - n0 : TN;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = (int)blockDim.x >> 5;
   const bool vec = P.tma_c && cols % 4 == 0;
-  for (int r = part * 8 + warp; r < CG * kTM; r += kFillParts * 8) {
+  for (int r = part * nw + warp; r < CG * kTM; r += kFillParts * nw) {
     const int copy = mt * CG + r / kTM;
     if (copy >= P.n_copy) continue;
     const int64_t row = (int64_t)__ldg(&P.tile_order[copy]) * kTM + r % kTM;
@@ -657,7 +658,7 @@ __device__ __forceinline__ void fill_cut_tile(const DenseTable<NP>& T, int CG, i
 // launch start once that one has completed: its A and B are then final and
 // only its writes of C wait for this fill.
 template <int NP>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(kFillThreads)
     dense_cut_fill_kernel(const __grid_constant__ DenseTable<NP> T, int CG, int TN) {
   pdl_wait();
   pdl_trigger();
@@ -751,7 +752,7 @@ rosko_status launch_table(const DenseTable<NP>& T, cudaStream_t st) {
       return ROSKO_ERR_CUDA;
     set = true;
   }
-  if (launch_dependent(fn, dim3((unsigned)(T.split.workers * CG)), dim3(kThreads<I8>), smem, st, T,
+  if (launch_dependent(fn, dim3((unsigned)(T.split.workers * CG)), dim3(kThreads), smem, st, T,
                        stages) != cudaSuccess)
     return ROSKO_ERR_CUDA;
   count_launches(1);
@@ -910,8 +911,8 @@ rosko_status run_jobs(const DenseJob* jobs, int count, int ctas, bool zero_cut, 
       return ROSKO_ERR_CUDA;
     count_launches(1);
   } else if (fill_blocks > 0) {
-    if (launch_dependent(dense_cut_fill_kernel<NP>, dim3((unsigned)fill_blocks), dim3(256), 0, st,
-                         T, CG, TN) != cudaSuccess)
+    if (launch_dependent(dense_cut_fill_kernel<NP>, dim3((unsigned)fill_blocks),
+                         dim3(kFillThreads), 0, st, T, CG, TN) != cudaSuccess)
       return ROSKO_ERR_CUDA;
     count_launches(1);
   }
