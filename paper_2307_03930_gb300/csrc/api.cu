@@ -268,40 +268,22 @@ rosko_status schedule_analytic(int64_t M, int64_t K, int64_t N, int64_t nnz, int
   t->split_k = (int32_t)split;
   t->dense_split_pm =
       (dt == ROSKO_BF16) ? kDenseSplitPm : (dt == ROSKO_I8 ? kDenseSplitPmI8 : 1001);
-  if (dt == ROSKO_BF16 && order == 4) {
-    // Small or very sparse layers: the tensor-core launch has a fixed cost
-    // (set-up, the first cold loads, the epilogue) that row-direct does not.
-    // Model both paths on the uniform-density assumption (every tile on one
-    // side of the threshold) and keep the layer sparse when row-direct is
-    // predicted faster.  Both models are least-squares fits (relative error)
-    // to the 5,000 training layers of the selector's measurement sweep
-    // (M, K in [64, 4096] and convolution shapes, N in [196, 12544], 50-99.9%
-    // sparse, every schedule timed): dense ~10.8 us + 2 M K N at
-    // ~0.58 PFLOP/s, row-direct ~5.3 us + the nnz * N BF16 values it moves
-    // at ~10.9 TB/s.  On the 2,000 held-out layers picking the faster path
-    // by these models costs 5% over the better of the two paths.
-    const double t_dense = 10.8 + 2.0 * (double)M * (double)K * (double)N / 0.58e15 * 1e6;
-    const double t_direct = 5.3 + (double)nnz * (double)N * 2.0 / 10.9e12 * 1e6;
-    if (t_direct < t_dense) t->dense_split_pm = 1001;
-  }
-  if (dt == ROSKO_I8 && order == 4) {
-    // The same choice for INT8 codes (either result type).  Row-direct: 2.5 us
-    // plus a byte of B per nonzero and column, whole 256-column strips, at
-    // ~8.5 TB/s.  Tensor cores: three launches' 8.5 us, the dense product at
-    // ~1.9 PFLOP/s, and the memory it moves: B converted to BF16 (3 bytes per
-    // value), C and the dense copies.  512x4608x3136 at 90 %: 27-30 us against
-    // 110-117 us; 512x1024x1000: 12-15 against 14.7; 200x1500x130 at 60 %: 11
-    // against 6.
-    const double t_dense = 8.5 + 2.0 * (double)M * (double)K * (double)N / 1.9e15 * 1e6 +
-                           3.0 * (double)K * (double)N / 5e12 * 1e6 +
-                           4.0 * (double)M * (double)N / 3e12 * 1e6 +
-                           2.0 * (double)M * (double)K / 7e12 * 1e6;
-    const double t_direct = 2.5 + (double)nnz * (double)((N + 255) / 256) * 256.0 / 8.5e12 * 1e6;
-    if (t_direct < t_dense) t->dense_split_pm = 1001;
-  }
   int TN = 256, ds = 1;
   int mc = 128;
   dense_config((M + 127) / 128, N, K, sms, &TN, &ds, &mc, dt == ROSKO_I8);
+  if ((dt == ROSKO_BF16 || dt == ROSKO_I8) && order == 4 && M > 0 && K > 0 && N > 0) {
+    // Small or very sparse layers: the tensor-core launch has a fixed cost
+    // (set-up, the first cold loads, the epilogue) that row-direct does not.
+    // Estimate both on the uniform-density assumption (every tile on one side
+    // of the threshold) and keep the layer sparse when row-direct is
+    // predicted faster.  INT8 pays the conversion of B besides.
+    double t_dense = dense_time_us((M + 127) / 128, N, K, TN, ds);
+    if (dt == ROSKO_I8) t_dense += 3.5 + 3.0 * (double)K * (double)N / 5e6;
+    double t_direct = direct_time_us(M, N, nnz, dt, sms);
+    const int lpr = narrow_pick(M, K, N, nnz, dt, sms);
+    if (lpr > 0) t_direct = std::min(t_direct, narrow_time_us(M, K, N, nnz, dt, lpr, sms));
+    if (t_direct < t_dense) t->dense_split_pm = 1001;
+  }
   t->dense_n_r = TN;
   t->dense_split_k = ds;
   t->dense_m_c = mc;
@@ -563,6 +545,11 @@ rosko_status spmm_run(rosko_packed_s* A, const void* B_dev, rosko_dtype b_dtype,
     if (t.k_c < 8) t.k_c = 32;
     L.KC = t.k_c;
   }
+  if (L.order == 4 && !(tile && tile->n_r > 0)) {
+    // few columns: the kernel that keeps a strip of B in shared memory, where
+    // it is predicted faster (a width that the caller gives is kept)
+    L.narrow = narrow_pick(A->M, A->K, N, A->nnz, p, sms);
+  }
   if (L.order == 4) {
     // one warp per C row, B from L2: no slabs, no K split
     L.W = 1;
@@ -604,7 +591,7 @@ rosko_status spmm_run(rosko_packed_s* A, const void* B_dev, rosko_dtype b_dtype,
   bool direct_cut = false;
   if (L.order == 4 && n_sparse > 0) {
     int64_t ns = 0;
-    const int which = direct_pick(A, A->panel_order_dev, n_sparse, N, L.V);
+    const int which = direct_pick(A, A->panel_order_dev, n_sparse, N, L.V, L.narrow);
     if (!direct_segments(A, A->panel_order_dev, n_sparse, which, &ns, &direct_cut))
       return ROSKO_ERR_UNSUPPORTED;
   }

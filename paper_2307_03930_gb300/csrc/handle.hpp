@@ -173,8 +173,16 @@ rosko_status zero_fill_launch(const ZeroFill& z, cudaStream_t st);
 // spmm_sparse.cu
 struct SparseLaunch {
   int R, V, W, KC, stages, split;
-  int order;  // 1 = column order (Alg. 2), 2 = row-slot, 3 = row-slot + gather
+  int order;  // 1 = column order (Alg. 2), 2 = row-slot, 3 = row-slot + gather, 4 = row-direct
+  int narrow = 0;  // order 4: chunks per strip of the few-column kernel, 0 = the general one
 };
+int narrow_chunks(rosko_dtype p_dt, int64_t K, int64_t N);
+double narrow_time_us(int64_t M, int64_t K, int64_t N, int64_t nnz, rosko_dtype dt, int lpr,
+                      int sms);
+double direct_time_us(int64_t M, int64_t N, int64_t nnz, rosko_dtype dt, int sms);
+// The narrow kernel's chunks per strip where it is predicted faster than the
+// general row-direct kernel, else 0.
+int narrow_pick(int64_t M, int64_t K, int64_t N, int64_t nnz, rosko_dtype dt, int sms);
 rosko_status sparse_spmm_launch(rosko_packed_s* h, const void* B, rosko_dtype b_dt, int64_t N,
                                 int64_t ldb, const float* col_scale, void* C, rosko_dtype c_dt,
                                 int64_t ldc, int accumulate, const SparseLaunch& L,
@@ -216,7 +224,7 @@ const SegEntry* direct_segments(const rosko_packed_s* h, const int32_t* panel_li
 // The list a launch over these panels with width N and V columns per lane
 // uses (0 fine, 1 coarse); decided the same way for zero-fill and launch.
 int direct_pick(const rosko_packed_s* h, const int32_t* panel_list, int64_t n_panels, int64_t N,
-                int V);
+                int V, int narrow = 0);
 // One launch over all jobs (count <= 64, same handle / B / C types, V
 // columns per lane); C of jobs with cut rows must be zeroed by the caller
 // unless they accumulate.
@@ -257,6 +265,8 @@ void dense_batch_needs_zero(const DenseJob* jobs, int count, int TN, int cg, boo
 // CTAs per worker (1 or 2) of a launch over n_tiles row tiles, and whether its
 // split over `ctas` CTAs cuts a tile
 int dense_group(int64_t n_tiles);
+// Estimated time (us) of a single problem's launches on the tensor cores.
+double dense_time_us(int64_t n_tiles, int64_t N, int64_t K, int TN, int ctas);
 bool dense_needs_zero(int64_t n_tiles, int64_t N, int64_t K, int TN, int ctas);
 
 // api.cu

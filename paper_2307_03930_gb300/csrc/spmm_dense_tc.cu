@@ -759,6 +759,13 @@ rosko_status launch_table(const DenseTable<NP>& T, cudaStream_t st) {
   return cudaGetLastError() == cudaSuccess ? ROSKO_OK : ROSKO_ERR_CUDA;
 }
 
+// Persistent workers: one per SM (or pair of SMs) at most, and no share below
+// kMinPiece slabs unless it is a tile of its own.
+int64_t split_workers(int64_t tiles, int64_t slabs, int ctas, int cg) {
+  const int64_t G = std::max(1, std::min(std::min(ctas, num_sms()), kMaxWorkers) / cg);
+  return std::max<int64_t>(1, std::min<int64_t>(G, std::max(tiles, slabs / kMinPiece)));
+}
+
 // The scalars of the problems and the split over `ctas` CTAs in workers of
 // cg; false when the cost space does not fit 31 bits.
 bool plan_split(const DenseJob* jobs, int count, int TN, int ctas, int cg, DenseProb* p,
@@ -785,11 +792,7 @@ bool plan_split(const DenseJob* jobs, int count, int TN, int ctas, int cg, Dense
   }
   if (units >= (int64_t(1) << 31)) return false;
   S->count = n;
-  // persistent workers: one per SM (or pair of SMs) at most, and no share
-  // below kMinPiece slabs unless it is a tile of its own
-  int64_t G = std::max(1, std::min(std::min(ctas, num_sms()), kMaxWorkers) / cg);
-  G = std::min<int64_t>(G, std::max(tiles, slabs_all / kMinPiece));
-  G = std::max<int64_t>(G, 1);
+  const int64_t G = split_workers(tiles, slabs_all, ctas, cg);
   S->workers = (int)G;
   S->rounds = n == 1 ? (int)(tiles / G) : 0;
   S->tile0 = (int)(S->rounds * G);
@@ -962,6 +965,29 @@ bool dense_needs_zero(int64_t n_tiles, int64_t N, int64_t K, int TN, int ctas) {
   std::vector<char> cut;
   cut_problems(S, &p, &cut);
   return !cut.empty() && cut[0];
+}
+
+// ~4.6 us around the first and last slabs, the longest share at the measured
+// rate per slab (a 256-column slab runs at ~530 cycles of the 512 that the
+// pipe needs, a 128-column one at ~350: it moves 96 bytes per pipe cycle into
+// each SM), the last tile's epilogue, the zero fill of cut tiles (a launch),
+// and no less than the memory needs.  Called on every product: the split's
+// sizes without its positions.
+double dense_time_us(int64_t n_tiles, int64_t N, int64_t K, int TN, int ctas) {
+  if (n_tiles <= 0 || N <= 0 || K <= 0) return 0.0;
+  if (ctas <= 0) ctas = num_sms();
+  const int cg = group_of(n_tiles, ctas);
+  const int64_t slabs = slabs_of(K), cost = std::max<int64_t>(slabs, kEpiCost);
+  const int64_t tiles = (n_tiles + cg - 1) / cg * ((N + TN - 1) / TN);
+  const int64_t G = split_workers(tiles, tiles * slabs, ctas, cg);
+  const int64_t rounds = tiles / G, rest = tiles - rounds * G;
+  const bool cut = rest > 0 && slabs >= 2 * kMinPiece;
+  const double share = (double)rounds * cost +
+                       (cut ? (double)rest * cost / G : (rest > 0 ? (double)cost : 0.0));
+  const double mem = (2.0 * (double)n_tiles * kTM * K + 2.0 * (double)K * N +
+                      4.0 * (double)n_tiles * kTM * N) / 6.5e6;
+  return 4.6 + std::max(share * (TN == 256 ? 0.275 : 0.185), mem) + (TN == 256 ? 3.7 : 1.9) +
+         (cut ? 4.0 : 0.0);
 }
 
 rosko_status dense_batch_launch(const DenseJob* jobs, int count, int TN, int cg, cudaStream_t st) {

@@ -20,6 +20,7 @@
 //     contiguous 512-byte run (conflict free);
 //   * C is written once at the end (or added with atomics when K is split
 //     across CTAs).
+#include <atomic>
 #include <type_traits>
 #include <algorithm>
 #include <climits>
@@ -638,8 +639,22 @@ constexpr int async_batch() {
   return ((V * (int)sizeof(TB)) >= 32 || std::is_same<TA, double>::value) ? 4 : 8;
 }
 template <class TA, class TB, class TC, int V, int NP>
-constexpr size_t async_smem_bytes() {
+constexpr size_t async_ring_bytes() {
   return (size_t)8 * 2 * async_batch<TA, TB, TC, V, NP>() * 32 * V * sizeof(TB);
+}
+// FP32 sums of long rows: every 64 records a warp adds its sums to a second set
+// behind the rings, so that the rounding error grows with the number of a
+// row's pieces and not with its length.  (In registers that set cost the FP32
+// kernel 25 -> 27 us on 1024x1024x1024 at 90 %; strips of 512 columns serve
+// short rows and have none.)
+template <class TACC, int V>
+constexpr bool two_level() {
+  return std::is_same<TACC, float>::value && V <= 8;
+}
+template <class TA, class TB, class TC, int V, int NP>
+constexpr size_t async_smem_bytes() {
+  return async_ring_bytes<TA, TB, TC, V, NP>() +
+         (two_level<typename AccOf<TA>::type, V>() ? (size_t)8 * 32 * V * 4 : 0);
 }
 
 template <class TA, class TB, class TC, int V, int NP>
@@ -703,6 +718,11 @@ __global__ void __launch_bounds__(256, 3)
   TACC acc[V];
 #pragma unroll
   for (int v = 0; v < V; ++v) acc[v] = TACC(0);
+  constexpr bool kTwoLevel = two_level<TACC, V>();
+  // this lane's second set: chunk i of 4 sums at [i][lane]
+  float4* tot = reinterpret_cast<float4*>(ring_smem + async_ring_bytes<TA, TB, TC, V, NP>()) +
+                warp * (V / 4) * 32 + lane;
+  bool folded = false;
   TC* crow = reinterpret_cast<TC*>(P.C) + row * P.ldc;
   const WT* __restrict__ rnz = reinterpret_cast<const WT*>(P.rnz);
   // per lane chunk: the bytes inside N (0: past the end) and the chunk's
@@ -836,6 +856,33 @@ __global__ void __launch_bounds__(256, 3)
       consume(cnt, t + U, 1, wbb);
     }
     mine = nmine;
+    if constexpr (kTwoLevel) {
+      if (((base - e0) & 32) && base + 32 < e_end) {   // warp-uniform
+#pragma unroll
+        for (int i = 0; i < V / 4; ++i) {
+          float4 t = folded ? tot[i * 32] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+          t.x += acc[4 * i];
+          t.y += acc[4 * i + 1];
+          t.z += acc[4 * i + 2];
+          t.w += acc[4 * i + 3];
+          tot[i * 32] = t;
+          acc[4 * i] = acc[4 * i + 1] = acc[4 * i + 2] = acc[4 * i + 3] = TACC(0);
+        }
+        folded = true;
+      }
+    }
+  }
+  if constexpr (kTwoLevel) {
+    if (folded) {
+#pragma unroll
+      for (int i = 0; i < V / 4; ++i) {
+        const float4 t = tot[i * 32];
+        acc[4 * i] += t.x;
+        acc[4 * i + 1] += t.y;
+        acc[4 * i + 2] += t.z;
+        acc[4 * i + 3] += t.w;
+      }
+    }
   }
   // the next launch in the stream may be scheduled as this CTA finishes
   pdl_trigger();
@@ -867,6 +914,143 @@ __global__ void __launch_bounds__(256, 3)
       for (int v = 0; v < CE; ++v)
         if (col0 + v < N) crow[col0 + v] = o[v];
     }
+  }
+}
+
+// ---------------------------------------------------------------------------
+// Row-direct for few columns of C (a decoding step, a feature vector).  The
+// strips of the kernel above are 128 columns or more, so with N = 16 most of
+// its lanes copy nothing.  Here a whole strip of B (all K rows, LPR 16-byte
+// chunks wide, at most kNarrowSmem) sits in the shared memory of every block,
+// loaded once; a warp takes a work segment, its lanes 32 / LPR records at a
+// time (LPR lanes share a record, each multiplying its own 16 bytes of the B
+// row), and the partial sums meet in a shuffle tree at the segment's end.
+// The bound is shared memory: four records with 32-byte rows meet in a
+// 128-byte phase, whose bank conflicts double it (measured: 8.1 wavefronts per
+// 512-byte request), i.e. about half a cycle per record and SM.  11008 x 4096 at 90 %, N = 16, BF16: 18.5 us on the tensor
+// cores (90 MB of dense copies), 155 row-direct, 14.4 here.
+constexpr int kNarrowSmem = 200 * 1024;
+constexpr int kNarrowWarps = 32;
+
+struct NarrowParams {
+  const void* rnz;
+  const SegEntry* segs;
+  const void* B;
+  float* C;
+  int64_t n_segs, ldb, ldc;
+  int K, N, strips, load_c;
+};
+
+template <class TA, class TB, int LPR>
+__global__ void __launch_bounds__(32 * kNarrowWarps, 1) narrow_kernel(const NarrowParams p) {
+  using WT = typename RowRec<TA>::T;
+  constexpr int CE = 16 / (int)sizeof(TB);   // columns of a lane
+  constexpr int RPS = 32 / LPR;              // records of a warp step
+  // steps whose records are fetched together: a batch is in flight while the
+  // one before it is multiplied, across the ends of segments too
+  constexpr int UN = 4 * (LPR < 2 ? 1 : 2);
+  constexpr int BATCH = UN * RPS;
+  extern __shared__ __align__(16) unsigned char bs[];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int strip = (int)blockIdx.x % p.strips, part = (int)blockIdx.x / p.strips;
+  const int parts = (int)gridDim.x / p.strips;
+  pdl_wait();
+  pdl_trigger();
+  // the strip of B: chunk c of row k at (k LPR + c) 16 bytes, zero past N
+  {
+    const char* src = static_cast<const char*>(p.B);
+    const int64_t row_bytes = p.ldb * (int64_t)sizeof(TB);
+    const uint32_t dst = smem_u32(bs);
+    for (int i = threadIdx.x; i < p.K * LPR; i += 32 * kNarrowWarps) {
+      const int k = i / LPR, c = i % LPR;
+      const int col = (strip * LPR + c) * CE;
+      const int left = p.N - col;
+      const int bytes = left <= 0 ? 0 : (left >= CE ? 16 : left * (int)sizeof(TB));
+      cp_async<16>(dst + (uint32_t)i * 16u, src + (bytes ? k * row_bytes + col * (int)sizeof(TB) : 0),
+                   bytes);
+    }
+    cp_async_commit();
+  }
+  const int sub = lane % LPR, rl = lane / LPR;
+  const unsigned char* my_b = bs + sub * 16;
+  const int col0 = (strip * LPR + sub) * CE;
+  const WT* __restrict__ rnz = static_cast<const WT*>(p.rnz);
+  // neighbouring segments (of similar length, longest first) go to different
+  // blocks
+  const int64_t step = (int64_t)parts * kNarrowWarps;
+  int64_t si = (int64_t)warp * parts + part;
+  const int4 none = make_int4(0, 0, 0, 0);
+  int4 seg = si < p.n_segs ? __ldg(&p.segs[si].head) : none;
+  int4 nxt = si + step < p.n_segs ? __ldg(&p.segs[si + step].head) : none;
+  WT w[UN], wn[UN];
+  auto fetch = [&](WT (&r)[UN], int eb, int end) {
+#pragma unroll
+    for (int u = 0; u < UN; ++u) {
+      const int e = eb + u * RPS + rl;
+      r[u] = e < end ? __ldg(&rnz[e]) : WT{};
+    }
+  };
+  fetch(w, seg.y, seg.z);
+  cp_async_wait<0>();
+  __syncthreads();
+  float acc[CE];
+#pragma unroll
+  for (int v = 0; v < CE; ++v) acc[v] = 0.0f;
+  auto madd = [&](WT r) {
+    const uint4 b = *reinterpret_cast<const uint4*>(
+        my_b + (uint32_t)RowRec<TA>::k(r) * (uint32_t)(LPR * 16));
+    if constexpr (std::is_same<TB, __nv_bfloat16>::value) {
+      fma_bf16x2(acc[0], acc[1], r, b.x);
+      fma_bf16x2(acc[2], acc[3], r, b.y);
+      fma_bf16x2(acc[4], acc[5], r, b.z);
+      fma_bf16x2(acc[6], acc[7], r, b.w);
+    } else {
+      const float a = RowRec<TA>::a(r);
+      acc[0] = mac(a, __uint_as_float(b.x), acc[0]);
+      acc[1] = mac(a, __uint_as_float(b.y), acc[1]);
+      acc[2] = mac(a, __uint_as_float(b.z), acc[2]);
+      acc[3] = mac(a, __uint_as_float(b.w), acc[3]);
+    }
+  };
+  int eb = seg.y;
+  while (si < p.n_segs) {
+    const bool ends = eb + BATCH >= seg.z;   // this batch is the segment's last
+    if (ends) fetch(wn, nxt.y, nxt.z);
+    else fetch(wn, eb + BATCH, seg.z);
+    if (eb + BATCH <= seg.z) {
+#pragma unroll
+      for (int u = 0; u < UN; ++u) madd(w[u]);
+    } else {
+      // nothing is multiplied past the piece (0 times a non-finite B is not 0)
+#pragma unroll
+      for (int u = 0; u < UN; ++u)
+        if (eb + u * RPS + rl < seg.z) madd(w[u]);
+    }
+    if (ends) {
+#pragma unroll
+      for (int o = 16; o >= LPR; o >>= 1)
+#pragma unroll
+        for (int v = 0; v < CE; ++v) acc[v] += __shfl_xor_sync(0xffffffffu, acc[v], o);
+      if (rl == 0) {
+        float* c = p.C + (int64_t)seg.x * p.ldc + col0;
+#pragma unroll
+        for (int v = 0; v < CE; ++v) {
+          if (col0 + v >= p.N) break;
+          if (seg.w) atomicAdd(c + v, acc[v]);   // a piece of a cut row
+          else c[v] = p.load_c ? c[v] + acc[v] : acc[v];
+        }
+      }
+#pragma unroll
+      for (int v = 0; v < CE; ++v) acc[v] = 0.0f;
+      si += step;
+      seg = nxt;
+      eb = seg.y;
+      nxt = si + step < p.n_segs ? __ldg(&p.segs[si + step].head) : none;
+    } else {
+      eb += BATCH;
+    }
+#pragma unroll
+    for (int u = 0; u < UN; ++u) w[u] = wn[u];
   }
 }
 
@@ -1020,21 +1204,115 @@ const SegEntry* direct_segments(const rosko_packed_s* h, const int32_t* panel_li
   return base;
 }
 
-// Granularity for a launch: the coarse list when it still gives every SM
-// four waves of resident warps (24 per SM) over the column strips, else the
-// fine list (more, shorter pieces; the cut rows are added atomically).
+// Granularity for a launch.  The fine list adds warps for long rows, but a cut
+// row costs a zero fill of C (a memset between two launches, ~3 us) and atomic
+// adds, so rows stay whole (the coarse list) unless there is less than one
+// wave of resident warps (24 per SM) over the column strips and the mean row
+// is long (160 records; the coarse piece is twice the mean), where the longest
+// row alone would set the time.  Measured, fine against coarse (us):
+// 1024x1024x1024 at 90 % 28.8 / 25.0 (FP32), 24.8 / 17.0 (BF16), 512x4608x3136
+// at 90 % 127 / 94 (BF16), 117 / 91 (INT8); 128x4000x300 at 90 % (400 per row)
+// 14.5 / 35.8 (FP32), 300x4000x500 at 95 % 12.5 / 15.4 (BF16).
+// narrow: the few-column kernel, whose pieces each end in a shuffle tree: rows
+// stay whole (11008x4096x16 at 90 %: 31 us in pieces of 64, 14.4 whole).
+constexpr int kCutRecords = 320;
 int direct_pick(const rosko_packed_s* h, const int32_t* panel_list, int64_t n_panels, int64_t N,
-                int V) {
+                int V, int narrow) {
   int64_t ns = 0, ns_fine = 0;
   if (!direct_segments(h, panel_list, n_panels, 1, &ns, nullptr)) return 0;
+  if (narrow || h->segs[1].records < kCutRecords) return 1;
   const int64_t strips = (N + 32 * V - 1) / (32 * V);
-  if (ns * strips >= 4LL * 24 * num_sms()) return 1;
-  // few work items: the fine list adds warps for long rows, but a cut row
-  // costs a zero fill of C and atomic adds; when cutting adds under a
-  // quarter more pieces (an even matrix with a few rows just past 64
-  // records: 512x4608 at 99 %) the rows stay whole
+  if (ns * strips >= 24LL * num_sms()) return 1;
   if (!direct_segments(h, panel_list, n_panels, 0, &ns_fine, nullptr)) return 1;
   return 4 * ns_fine >= 5 * ns ? 0 : 1;
+}
+
+namespace {
+template <class TA, class TB>
+rosko_status narrow_launch(const NarrowParams& p, int lpr, int grid, size_t smem, cudaStream_t st) {
+  static std::atomic<bool> set[4];
+  auto go = [&](auto fn, int i) -> rosko_status {
+    if (!set[i].load(std::memory_order_acquire)) {
+      if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kNarrowSmem) !=
+          cudaSuccess)
+        return ROSKO_ERR_CUDA;
+      set[i].store(true, std::memory_order_release);
+    }
+    if (launch_dependent(fn, dim3((unsigned)grid), dim3(32 * kNarrowWarps), smem, st, p) !=
+        cudaSuccess)
+      return ROSKO_ERR_CUDA;
+    count_launches(1);
+    return cudaGetLastError() == cudaSuccess ? ROSKO_OK : ROSKO_ERR_CUDA;
+  };
+  switch (lpr) {
+    case 1: return go(narrow_kernel<TA, TB, 1>, 0);
+    case 2: return go(narrow_kernel<TA, TB, 2>, 1);
+    case 4: return go(narrow_kernel<TA, TB, 4>, 2);
+    default: return go(narrow_kernel<TA, TB, 8>, 3);
+  }
+}
+}  // namespace
+
+// Blocks per strip: one block per SM in all at most, and none without a
+// segment per warp or so.
+static int64_t narrow_parts(int64_t n_segs, int64_t strips, int sms) {
+  return std::max<int64_t>(
+      1, std::min<int64_t>(sms / strips, (n_segs + kNarrowWarps - 1) / kNarrowWarps));
+}
+
+// 16-byte chunks per strip of the narrow kernel (1, 2, 4 or 8), 0 when B does
+// not suit it: the strip of all K rows must fit in shared memory.
+int narrow_chunks(rosko_dtype p_dt, int64_t K, int64_t N) {
+  if (p_dt != ROSKO_F32 && p_dt != ROSKO_BF16) return 0;
+  const int64_t need = (N * (int64_t)dtype_size(p_dt) + 15) / 16;
+  int lpr = 1;
+  while (lpr < 8 && lpr < need && K * (2 * lpr) * 16 <= kNarrowSmem) lpr *= 2;
+  return K > 0 && K * lpr * 16 <= kNarrowSmem ? lpr : 0;
+}
+
+// Estimated times (us) of the row-direct kernels on GB300 for nnz nonzeros
+// spread evenly, from timed layers (M, K in [64, 11008], N in [8, 3136], 1 to
+// 10 % dense, FP32 and BF16; within ~25 %).
+// General: a record of a 256-column strip costs an SM ~9 cycles (BF16, INT8;
+// 14.5 for FP32's two chunks per lane), whatever of the strip lies inside N; a
+// row's records are one chain of L2 latencies, or (long rows of few items, see
+// direct_pick) cut into short ones after a memset; and every wave of resident
+// warps costs ~1.4 us however short its rows are.
+double direct_time_us(int64_t M, int64_t N, int64_t nnz, rosko_dtype dt, int sms) {
+  const double mean = (double)nnz / (double)std::max<int64_t>(M, 1);
+  const double strips = (double)((N + 255) / 256);
+  const double work = (double)nnz * strips / sms * (dt == ROSKO_F32 ? 14.5 : 9.3) / 1.93e3;
+  const double waves = (double)M * strips / (24.0 * sms);
+  const bool cut = 2.0 * mean >= kCutRecords && waves < 1.0;
+  const double per_record = dt == ROSKO_F32 ? 0.075 : (dt == ROSKO_BF16 ? 0.05 : 0.03);
+  const double chain = (cut ? kSegRecords : mean) * per_record;
+  return 3.0 + std::max(std::max(work, chain), waves * 1.4) + (cut ? 5.0 : 0.0);
+}
+
+// Narrow: per block the load of its strip (~60 KB a microsecond), the records
+// of its rows (shared-memory wavefronts per record: bank conflicts of the
+// strip's rows plus the record fetch) and per row of a warp the latency of its
+// first records and a shuffle tree (8194x108x488 with 3 records a row: 31.7
+// us, 7.3 in the general kernel).
+double narrow_time_us(int64_t M, int64_t K, int64_t N, int64_t nnz, rosko_dtype dt, int lpr,
+                      int sms) {
+  const int64_t cols = (int64_t)lpr * 16 / (int64_t)dtype_size(dt);
+  const int64_t strips = (N + cols - 1) / cols;
+  const int64_t parts = narrow_parts(M, strips, sms);
+  const double waves = (double)((strips * parts + sms - 1) / sms);
+  const double wf = lpr == 1 ? 0.36 : (lpr == 2 ? 0.57 : (lpr == 4 ? 0.9 : 1.3));
+  const double rows = (double)((M + parts * kNarrowWarps - 1) / (parts * kNarrowWarps));
+  const double block = (double)(K * lpr) * 16.0 / 60e3 +
+                       (double)nnz / (double)parts * wf / 1.93e3 + rows * 0.9;
+  return 3.0 + waves * block;
+}
+
+int narrow_pick(int64_t M, int64_t K, int64_t N, int64_t nnz, rosko_dtype dt, int sms) {
+  const int lpr = narrow_chunks(dt, K, N);
+  if (lpr == 0) return 0;
+  return narrow_time_us(M, K, N, nnz, dt, lpr, sms) < 0.95 * direct_time_us(M, N, nnz, dt, sms)
+             ? lpr
+             : 0;
 }
 
 // Fill one problem of a row-direct table; returns the problem's block count
@@ -1131,6 +1409,34 @@ rosko_status sparse_spmm_launch(rosko_packed_s* h, const void* B, rosko_dtype b_
                                 const int32_t* panel_list, int64_t n_panels, bool c_zeroed,
                                 cudaStream_t st) {
   if (n_panels <= 0) return ROSKO_OK;
+  if (L.order == 4 && L.narrow > 0) {
+    int64_t n_segs = 0;
+    const int which = direct_pick(h, panel_list, n_panels, N, L.V, L.narrow);
+    NarrowParams p{};
+    p.segs = direct_segments(h, panel_list, n_panels, which, &n_segs, nullptr);
+    if (!p.segs || !h->rnz) return ROSKO_ERR_UNSUPPORTED;
+    if (reinterpret_cast<uintptr_t>(B) % 16 != 0 ||
+        (ldb * (int64_t)dtype_size(b_dt)) % 16 != 0)
+      return ROSKO_ERR_INVALID_ARG;   // 16-byte chunks of B
+    p.rnz = h->rnz;
+    p.B = B;
+    p.C = static_cast<float*>(C);
+    p.n_segs = n_segs;
+    p.ldb = ldb;
+    p.ldc = ldc;
+    p.K = (int)h->K;
+    p.N = (int)N;
+    const int64_t cols = (int64_t)L.narrow * 16 / (int64_t)dtype_size(b_dt);
+    p.strips = (int)((N + cols - 1) / cols);
+    p.load_c = accumulate;
+    const int64_t parts = narrow_parts(n_segs, p.strips, num_sms());
+    const size_t smem = (size_t)h->K * L.narrow * 16;
+    const int64_t grid = parts * p.strips;
+    if (grid > INT_MAX) return ROSKO_ERR_UNSUPPORTED;
+    return h->dt == ROSKO_BF16
+               ? narrow_launch<__nv_bfloat16, __nv_bfloat16>(p, L.narrow, (int)grid, smem, st)
+               : narrow_launch<float, float>(p, L.narrow, (int)grid, smem, st);
+  }
   if (L.order == 4) {
     // one warp per C row, B from L2; no K split, C written (or added) directly
     DirectJob j{h, B, b_dt, N, ldb, col_scale, C, c_dt, ldc, accumulate, panel_list, n_panels};
