@@ -277,7 +277,7 @@ rosko_status schedule_analytic(int64_t M, int64_t K, int64_t N, int64_t nnz, int
     // Estimate both on the uniform-density assumption (every tile on one side
     // of the threshold) and keep the layer sparse when row-direct is
     // predicted faster.  INT8 pays the conversion of B besides.
-    double t_dense = dense_time_us((M + 127) / 128, N, K, TN, ds);
+    double t_dense = dense_time_us((M + 127) / 128, N, K, TN, ds, dt == ROSKO_I8);
     if (dt == ROSKO_I8) t_dense += 3.5 + 3.0 * (double)K * (double)N / 5e6;
     double t_direct = direct_time_us(M, N, nnz, dt, sms);
     const int lpr = narrow_pick(M, K, N, nnz, dt, sms);
@@ -598,7 +598,7 @@ rosko_status spmm_run(rosko_packed_s* A, const void* B_dev, rosko_dtype b_dtype,
   const bool zero_sparse = !accumulate && n_sparse > 0 && (L.split > 1 || direct_cut);
   const bool zero_dense =
       !accumulate && !skip_dense && n_dense > 0 &&
-      dense_needs_zero(n_dense, N, A->K, t.dense_n_r, t.dense_split_k);
+      dense_needs_zero(n_dense, N, A->K, t.dense_n_r, t.dense_split_k, p == ROSKO_I8);
   const bool zero_c = zero_sparse || zero_dense;
   if (flags & kRunPlanOnly) {
     // report the split and the resolved schedule, launch nothing

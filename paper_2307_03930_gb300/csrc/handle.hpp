@@ -266,8 +266,8 @@ void dense_batch_needs_zero(const DenseJob* jobs, int count, int TN, int cg, boo
 // split over `ctas` CTAs cuts a tile
 int dense_group(int64_t n_tiles);
 // Estimated time (us) of a single problem's launches on the tensor cores.
-double dense_time_us(int64_t n_tiles, int64_t N, int64_t K, int TN, int ctas);
-bool dense_needs_zero(int64_t n_tiles, int64_t N, int64_t K, int TN, int ctas);
+double dense_time_us(int64_t n_tiles, int64_t N, int64_t K, int TN, int ctas, bool i8);
+bool dense_needs_zero(int64_t n_tiles, int64_t N, int64_t K, int TN, int ctas, bool i8);
 
 // api.cu
 rosko_status spmm_validate(rosko_packed_s* A, const void* B_dev, rosko_dtype b_dtype, int64_t N,

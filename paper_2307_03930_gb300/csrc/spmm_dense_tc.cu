@@ -138,8 +138,9 @@ struct DenseProb {
 // The split of the work between the workers.  Rounds of whole tiles (one
 // problem only): tile r * workers + w for r < rounds; then the tiles from
 // tile0 on, cut along the cost space [0, units).
-// cut = 0: every share ends on a tile boundary (a batch with at least two
-// tiles per worker: its problems would otherwise be zero-filled whole).
+// cut = 0: every share ends on a tile boundary (see cut_rest; a batch with at
+// least two tiles per worker: its problems would otherwise be zero-filled
+// whole).
 struct DenseSplit {
   int count, workers, rounds, tile0, units, cut;
 };
@@ -267,6 +268,11 @@ __global__ void __cluster_dims__(CG, 1, 1) __maxnreg__(kRegsLaunch)
   constexpr uint32_t kStageBytes = kABytes + kBBytes;
   constexpr int NBUF = 512 / TN;                          // TMEM accumulators
   constexpr int kParts = TN / 128;                        // epilogue warps that share a tile's rows
+  // 256-column tiles: both accumulators serve every tile in turn.  128-column
+  // ones: two for each warpgroup's tiles, so that a group only ever waits on
+  // barriers whose every phase is its own (a parity says nothing about a
+  // phase further ahead).
+  static_assert(NBUF == 4 / kParts, "two accumulators per group of epilogue warps");
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -409,18 +415,19 @@ __global__ void __cluster_dims__(CG, 1, 1) __maxnreg__(kRegsLaunch)
     int st = 0;
     uint32_t ph = 0;
     bool ok = true;
-    int b = NBUF - 1;          // accumulator of the current segment
-    uint32_t bph = 0;          // parity of its last release (fresh: passes)
+    int grp = kParts - 1 ? 0 : 1;        // whose tile the current segment is
+    uint32_t used0 = 0, used1 = 0;       // chunks given to each group so far
     while (rank == 0 && ok && it.next(sg)) {
+      if (kParts == 1) grp ^= 1;
       for (int c0 = sg.s0; ok && c0 < sg.s1;) {
         // slabs [c0, c1) sum in one accumulator
         const int c1 = min(sg.s1, c0 + kChunkSlabs);
-        if (++b == NBUF) {
-          b = 0;
-          bph ^= 1u;
-        }
+        const uint32_t u = grp ? used1++ : used0++;
+        const int b = 2 * grp + (int)(u & 1u);
         // the epilogue (of both CTAs) must have drained this accumulator
-        if (!__all_sync(0xffffffffu, mbar_wait_bounded<CG == 2>(&acc_empty[b], bph, T.status))) {
+        // (parity of its last release; fresh: passes)
+        if (!__all_sync(0xffffffffu, mbar_wait_bounded<CG == 2>(&acc_empty[b], ((u >> 1) & 1u) ^ 1u,
+                                                                T.status))) {
           ok = false;
           break;
         }
@@ -474,18 +481,14 @@ __global__ void __cluster_dims__(CG, 1, 1) __maxnreg__(kRegsLaunch)
     uint8_t* my_stage = stage_c + (size_t)(warp - kFirstEpi) * NS * kStageC;
     int chunk = 0;   // staging tiles alternate per chunk
     const uint32_t drained = CG == 2 ? cluster_addr(acc_empty, 0) : 0u;
-    int b = NBUF - 1;
-    uint32_t bph = 1;
+    uint32_t used = 0;             // chunks of this group so far
+    int b = 0;                     // accumulator of the current one
     const bool i32 = I8 && !T.row_scale;
-    auto next_acc = [&]() {
-      if (++b == NBUF) {
-        b = 0;
-        bph ^= 1u;
-      }
-    };
     auto wait_acc = [&]() -> bool {
-      next_acc();
-      const bool ok = __all_sync(0xffffffffu, mbar_wait_bounded(&acc_full[b], bph, T.status));
+      b = (kParts == 1 ? 2 * group : 0) + (int)(used & 1u);
+      const bool ok = __all_sync(0xffffffffu,
+                                 mbar_wait_bounded(&acc_full[b], (used >> 1) & 1u, T.status));
+      ++used;
       tc::fence_after_sync();
       return ok;
     };
@@ -500,11 +503,7 @@ __global__ void __cluster_dims__(CG, 1, 1) __maxnreg__(kRegsLaunch)
       }
     };
     while (it.next(sg)) {
-      if (kParts == 1 && (turn++ & 1) != group) {
-        // the other warpgroup's tile: step over its accumulators
-        for (int c0 = sg.s0; c0 < sg.s1; c0 += kChunkSlabs) next_acc();
-        continue;
-      }
+      if (kParts == 1 && (turn++ & 1) != group) continue;   // the other group's tile
       const int copy = sg.mt * CG + rank;
       // the tile's C rows, fetched while the MMAs run (what else the stores
       // need is read after the sums: registers are short until then)
@@ -547,16 +546,17 @@ __global__ void __cluster_dims__(CG, 1, 1) __maxnreg__(kRegsLaunch)
       // write (or add) the 32 x 32 chunk at column col0: r[j] of lane i is
       // the value (FP32 or INT32 bits) of row row0 + i, column col0 + j
       auto put_chunk = [&](const uint32_t (&r)[32], int col0) {
-        if (tma_c) {
-          // the staging tile is free once the copy issued NS chunks ago has read it
-          uint8_t* buf = my_stage + (size_t)(chunk % NS) * kStageC;
-          if (lane == 0) bulk_wait_read<NS - 1>();
-          __syncwarp();
-          // row `lane`, 16-byte chunk j at (j ^ (lane % 8)): the 128-byte swizzle
+        // row `lane` of the 32 x 32 chunk into a staging tile, 16-byte chunk j at
+        // (j ^ (lane % 8)): the 128-byte swizzle.  The tile is free once the
+        // copy issued NS chunks ago has read it.
+        uint8_t* buf = my_stage + (size_t)(chunk % NS) * kStageC;
+        if (lane == 0) bulk_wait_read<NS - 1>();
+        __syncwarp();
 #pragma unroll
-          for (int j = 0; j < 8; ++j)
-            *reinterpret_cast<uint4*>(buf + lane * 128 + ((j ^ (lane & 7)) << 4)) =
-                make_uint4(r[4 * j], r[4 * j + 1], r[4 * j + 2], r[4 * j + 3]);
+        for (int j = 0; j < 8; ++j)
+          *reinterpret_cast<uint4*>(buf + lane * 128 + ((j ^ (lane & 7)) << 4)) =
+              make_uint4(r[4 * j], r[4 * j + 1], r[4 * j + 2], r[4 * j + 3]);
+        if (tma_c) {
           fence_proxy_async_smem();
           __syncwarp();
           if (lane == 0) {
@@ -568,32 +568,26 @@ __global__ void __cluster_dims__(CG, 1, 1) __maxnreg__(kRegsLaunch)
           ++chunk;
           return;
         }
-        // C rows not 16-byte aligned (no tensor map): transpose the 32 x 32
-        // chunk through this warp's staging tile (rotated rows, no bank
-        // conflicts) so that each store instruction writes 32 consecutive
-        // columns of one row
-        uint32_t* tr = reinterpret_cast<uint32_t*>(my_stage);
-        // the staging tiles may still be read by this warp's TMA stores of
-        // an earlier problem of the batch (one with aligned C rows): wait
-        // until those reads are done before reusing the space
-        if (lane == 0) bulk_wait_read<0>();
-        __syncwarp();
-#pragma unroll
-        for (int j = 0; j < 32; ++j) tr[lane * 32 + ((j + lane) & 31)] = r[j];
+        // C rows not 16-byte aligned (no tensor map): read back row by row, so
+        // that each store instruction writes 32 consecutive columns of one row
         __syncwarp();
         const int rows = PM - row0 < 32 ? PM - row0 : 32;
         if (col0 + lane < PN) {
-          // eight rows at a time: their shared-memory reads, then their stores
+          // some rows at a time: their shared-memory reads, then their stores
+          constexpr int RB = I8 ? 8 : 16;
           float* dst = c_row0 + col0;
+          const uint8_t* src = buf + (lane & 3) * 4;
+          const int ch = lane >> 2;
 #pragma unroll 1
-          for (int r0 = 0; r0 < rows; r0 += 8, dst += 8 * ldc) {
-            uint32_t v[8];
+          for (int r0 = 0; r0 < rows; r0 += RB, dst += RB * ldc) {
+            uint32_t v[RB];
 #pragma unroll
-            for (int i = 0; i < 8; ++i) v[i] = tr[(r0 + i) * 32 + ((lane + r0 + i) & 31)];
+            for (int i = 0; i < RB; ++i)
+              v[i] = *reinterpret_cast<const uint32_t*>(src + (r0 + i) * 128 + ((ch ^ (i & 7)) << 4));
+            float* d = dst;
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
+            for (int i = 0; i < RB; ++i, d += ldc) {
               if (r0 + i >= rows) break;
-              float* d = dst + i * ldc;
               if (!add) {
                 *reinterpret_cast<uint32_t*>(d) = v[i];
               } else if (i32) {
@@ -786,6 +780,19 @@ int64_t split_workers(int64_t tiles, int64_t slabs, int ctas, int cg) {
   return std::max<int64_t>(1, std::min<int64_t>(G, std::max(tiles, slabs / kMinPiece)));
 }
 
+// What cutting tiles costs a single product, in K slabs: the zero fill of the
+// cut tiles is a launch of its own (~4 us; fused with INT8's conversion; none
+// when C is accumulated into).
+int cut_cost(int TN, bool i8, bool accumulate) {
+  return accumulate ? 0 : (i8 ? 2 : (TN == 256 ? 14 : 20));
+}
+// Whether to cut the `rest` tiles that do not fill a round of G workers along
+// K, or deal them whole (2019x986x3352: 21.4 us cut, 18.5 whole;
+// 1024x4096x4096: 32 cut, 26 whole; 512x4608x3136: 22 cut, 28 whole).
+bool cut_rest(int64_t rest, int64_t cost, int64_t G, int extra) {
+  return rest > 0 && rest * cost / G + extra < cost;
+}
+
 // The scalars of the problems and the split over `ctas` CTAs in workers of
 // cg; false when the cost space does not fit 31 bits.
 bool plan_split(const DenseJob* jobs, int count, int TN, int ctas, int cg, DenseProb* p,
@@ -817,7 +824,12 @@ bool plan_split(const DenseJob* jobs, int count, int TN, int ctas, int cg, Dense
   S->rounds = n == 1 ? (int)(tiles / G) : 0;
   S->tile0 = (int)(S->rounds * G);
   S->units = (int)(n == 1 ? (tiles - S->tile0) * p[0].cost : units);
-  S->cut = n == 1 || tiles < 2 * G ? 1 : 0;
+  S->cut = tiles < 2 * G ? 1 : 0;
+  if (n == 1)
+    S->cut = cut_rest(tiles - S->tile0, p[0].cost, G,
+                      cut_cost(TN, jobs[0].i8 != 0, p[0].accumulate != 0))
+                 ? 1
+                 : 0;
   return true;
 }
 
@@ -972,13 +984,14 @@ rosko_status dispatch_jobs(const DenseJob* jobs, int count, int TN, int cg, int 
 
 }  // namespace
 
-bool dense_needs_zero(int64_t n_tiles, int64_t N, int64_t K, int TN, int ctas) {
+bool dense_needs_zero(int64_t n_tiles, int64_t N, int64_t K, int TN, int ctas, bool i8) {
   if (n_tiles <= 0 || N <= 0) return false;
   if (ctas <= 0) ctas = num_sms();
   DenseJob j{};
   j.n_tiles = n_tiles;
   j.N = N;
   j.K = K;
+  j.i8 = i8;
   DenseProb p{};
   DenseSplit S{};
   if (!plan_split(&j, 1, TN, ctas, group_of(n_tiles, ctas), &p, &S)) return false;
@@ -993,7 +1006,7 @@ bool dense_needs_zero(int64_t n_tiles, int64_t N, int64_t K, int TN, int ctas) {
 // each SM), the last tile's epilogue, the zero fill of cut tiles (a launch),
 // and no less than the memory needs.  Called on every product: the split's
 // sizes without its positions.
-double dense_time_us(int64_t n_tiles, int64_t N, int64_t K, int TN, int ctas) {
+double dense_time_us(int64_t n_tiles, int64_t N, int64_t K, int TN, int ctas, bool i8) {
   if (n_tiles <= 0 || N <= 0 || K <= 0) return 0.0;
   if (ctas <= 0) ctas = num_sms();
   const int cg = group_of(n_tiles, ctas);
@@ -1001,13 +1014,13 @@ double dense_time_us(int64_t n_tiles, int64_t N, int64_t K, int TN, int ctas) {
   const int64_t tiles = (n_tiles + cg - 1) / cg * ((N + TN - 1) / TN);
   const int64_t G = split_workers(tiles, tiles * slabs, ctas, cg);
   const int64_t rounds = tiles / G, rest = tiles - rounds * G;
-  const bool cut = rest > 0 && slabs >= 2 * kMinPiece;
+  const bool cut = slabs >= 2 * kMinPiece && cut_rest(rest, cost, G, cut_cost(TN, i8, false));
   const double share = (double)rounds * cost +
                        (cut ? (double)rest * cost / G : (rest > 0 ? (double)cost : 0.0));
   const double mem = (2.0 * (double)n_tiles * kTM * K + 2.0 * (double)K * N +
                       4.0 * (double)n_tiles * kTM * N) / 6.5e6;
   return 4.6 + std::max(share * (TN == 256 ? 0.275 : 0.185), mem) + (TN == 256 ? 3.7 : 1.9) +
-         (cut ? 4.0 : 0.0);
+         (cut && !i8 ? 4.0 : 0.0);
 }
 
 rosko_status dense_batch_launch(const DenseJob* jobs, int count, int TN, int cg, cudaStream_t st) {

@@ -23,6 +23,8 @@ pytestmark = pytest.mark.gpu
     (257, 4200, 70, 128, 0),       # 2 tiles cut over every pair
     (129, 1024, 2305, 128, 6),     # 19 tiles, K of exactly two minimum pieces
     (300, 960, 2000, 256, 10),     # K below two minimum pieces: never cut
+    (256, 5100, 700, 128, 2),      # one pair, 6 tiles of 80 slabs (5 chunks) each
+    (200, 9000, 900, 128, 4),      # 8 tiles of 9 chunks on two pairs, taken in turn
 ])
 @pytest.mark.parametrize("accumulate", [False, True])
 def test_pair_split(M, K, N, TN, ctas, accumulate):
