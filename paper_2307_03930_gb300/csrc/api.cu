@@ -19,9 +19,9 @@ namespace rosko {
 
 namespace {
 std::mutex g_mu;
-int* g_status[64] = {nullptr};
-int g_sms[64] = {0};
-PFN_cuTensorMapEncodeTiled_v12000 g_encode = nullptr;
+std::atomic<int*> g_status[64];
+std::atomic<int> g_sms[64];
+std::atomic<PFN_cuTensorMapEncodeTiled_v12000> g_encode{nullptr};
 }  // namespace
 
 namespace {
@@ -112,49 +112,48 @@ __global__ void probe_wait_kernel(int* status) {
 }
 void count_launches(int n) { g_launches.fetch_add(n, std::memory_order_relaxed); }
 
+// Both are asked for several times per product: no lock once they are known.
 int* device_status_word() {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
+  if (int* w = g_status[dev].load(std::memory_order_acquire)) return w;
   std::lock_guard<std::mutex> lk(g_mu);
-  if (!g_status[dev]) {
+  if (!g_status[dev].load(std::memory_order_relaxed)) {
     void* p = nullptr;
     if (cudaMalloc(&p, 256) != cudaSuccess) return nullptr;
     if (cudaMemset(p, 0, 256) != cudaSuccess) return nullptr;
-    g_status[dev] = static_cast<int*>(p);
+    g_status[dev].store(static_cast<int*>(p), std::memory_order_release);
   }
-  return g_status[dev];
+  return g_status[dev].load(std::memory_order_relaxed);
 }
 
 int num_sms() {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 152;
-  std::lock_guard<std::mutex> lk(g_mu);
-  if (!g_sms[dev]) {
-    int n = 0;
-    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0)
-      n = 152;
-    g_sms[dev] = n;
-  }
-  return g_sms[dev];
+  if (const int n = g_sms[dev].load(std::memory_order_relaxed)) return n;
+  int n = 0;
+  if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0)
+    n = 152;
+  g_sms[dev].store(n, std::memory_order_relaxed);
+  return n;
 }
 
 CUresult encode_tiled(CUtensorMap* map, CUtensorMapDataType dt, cuuint32_t rank, void* gaddr,
                       const cuuint64_t* dims, const cuuint64_t* strides, const cuuint32_t* box,
                       const cuuint32_t* estrides, CUtensorMapInterleave il, CUtensorMapSwizzle sw,
                       CUtensorMapL2promotion l2, CUtensorMapFloatOOBfill oob) {
-  {
-    std::lock_guard<std::mutex> lk(g_mu);
-    if (!g_encode) {
-      void* fn = nullptr;
-      cudaDriverEntryPointQueryResult q;
-      if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault,
-                                           &q) != cudaSuccess ||
-          q != cudaDriverEntryPointSuccess || !fn)
-        return CUDA_ERROR_NOT_FOUND;
-      g_encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
-    }
+  PFN_cuTensorMapEncodeTiled_v12000 enc = g_encode.load(std::memory_order_acquire);
+  if (!enc) {
+    void* fn = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault,
+                                         &q) != cudaSuccess ||
+        q != cudaDriverEntryPointSuccess || !fn)
+      return CUDA_ERROR_NOT_FOUND;
+    enc = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
+    g_encode.store(enc, std::memory_order_release);
   }
-  return g_encode(map, dt, rank, gaddr, dims, strides, box, estrides, il, sw, l2, oob);
+  return enc(map, dt, rank, gaddr, dims, strides, box, estrides, il, sw, l2, oob);
 }
 
 // Tensor-core dense-panel tiles (the kernel runs them on CTA pairs, 256 rows
