@@ -174,6 +174,8 @@ __device__ __forceinline__ int scan_job_of(const ScanSet& s, int64_t b) {
 
 // Tile pass A: per-tile sums.
 __global__ void scan_reduce_kernel(ScanSet s) {
+  pdl_wait();
+  pdl_trigger();
   const int j = scan_job_of(s, blockIdx.x);
   const ScanJob J = s.job[j];
   const int64_t base = ((int64_t)blockIdx.x - s.first[j]) * kScanTile;
@@ -190,6 +192,8 @@ __global__ void scan_reduce_kernel(ScanSet s) {
 // Spine pass B: exclusive scan of one job's tile sums (chunked), total to
 // sums[nb].
 __global__ void scan_spine_kernel(ScanSet s) {
+  pdl_wait();
+  pdl_trigger();
   const ScanJob J = s.job[blockIdx.x];
   int2 carry = make_int2(0, 0);
   for (int64_t c0 = 0; c0 < J.nb; c0 += kScanThreads) {
@@ -206,6 +210,8 @@ __global__ void scan_spine_kernel(ScanSet s) {
 
 // Tile pass C: in-place exclusive scan of each tile with its offset.
 __global__ void scan_down_kernel(ScanSet s) {
+  pdl_wait();
+  pdl_trigger();
   const int j = scan_job_of(s, blockIdx.x);
   const ScanJob J = s.job[j];
   const int64_t tile = (int64_t)blockIdx.x - s.first[j];
@@ -269,6 +275,7 @@ __device__ __forceinline__ void put_row_sentinel(void* rnz, int64_t e) {
 // consecutive ranges, one range per pass (a block runs exactly one pass).
 constexpr int kPackThreads = 256;
 constexpr int kRowsPerBlock = kPackThreads / 32;   // row passes: one warp per row
+constexpr int kRowBatch = 16;   // column passes: rows of a column in flight together
 
 struct PackGeom {
   int64_t M, K, lda, P, T;
@@ -301,15 +308,23 @@ __device__ void col_count(const S* __restrict__ A, const PackGeom& g,
     __syncthreads();
   }
   int c = 0;
-  // bounds are uniform across the block: every lane takes every ballot
-#pragma unroll 8
-  for (int64_t m = m0; m < m1; ++m) {
-    D v;
-    const bool nz = in && Conv<S, D>::get(A[m * g.lda + k], scale ? scale[m] : 1.0f, v);
-    c += nz ? 1 : 0;
-    if (rcnt) {
-      const unsigned mask = __ballot_sync(0xffffffffu, nz);
-      if (lane == 0 && mask) atomicAdd(&row_sum[m - m0], __popc(mask));
+  // bounds are uniform across the block: every lane takes every ballot.  A
+  // panel's loads are issued sixteen rows at a time, before any is tested.
+  for (int64_t mb = m0; mb < m1; mb += kRowBatch) {
+    S a[kRowBatch];
+#pragma unroll
+    for (int i = 0; i < kRowBatch; ++i)
+      a[i] = in && mb + i < m1 ? A[(mb + i) * g.lda + k] : S(0);
+#pragma unroll
+    for (int i = 0; i < kRowBatch; ++i) {
+      if (mb + i >= m1) break;
+      D v;
+      const bool nz = in && Conv<S, D>::get(a[i], scale ? scale[mb + i] : 1.0f, v);
+      c += nz ? 1 : 0;
+      if (rcnt) {
+        const unsigned mask = __ballot_sync(0xffffffffu, nz);
+        if (lane == 0 && mask) atomicAdd(&row_sum[mb + i - m0], __popc(mask));
+      }
     }
   }
   if (rcnt) {
@@ -354,6 +369,8 @@ __global__ void __launch_bounds__(kPackThreads)
                       int2* __restrict__ cnt, int* __restrict__ touched,
                       int* __restrict__ touched_total, int2* __restrict__ rcnt,
                       int2* __restrict__ flag, int64_t b_col) {
+  pdl_wait();
+  pdl_trigger();
   const int64_t b = blockIdx.x;
   if (b < b_col) {
     col_count<S, D>(A, g, scale, b, cnt, touched, touched_total, rcnt, flag);
@@ -383,7 +400,7 @@ struct WriteArgs {
   __nv_bfloat16* dense_A;
   int64_t dense_rows, Kpad, gxd, ry;
   int64_t nnz, n_cols, gu_total;
-  int zero_panels;
+  int zero_panels, a_vec, row_warps;
   int64_t b_scatter, b_row, b_union, b_dense;
 };
 
@@ -406,11 +423,17 @@ __device__ void scatter(const S* __restrict__ A, const PackGeom& g,
   w.colrec[o.y] = make_int2((int32_t)k, o.x);
   const int64_t m0 = p * g.m_r, m1 = min(g.M, m0 + g.m_r);
   int64_t e = o.x;
-  for (int64_t m = m0; m < m1; ++m) {
-    D v;
-    if (Conv<S, D>::get(A[m * g.lda + k], scale ? scale[m] : 1.0f, v)) {
-      put_rec(w.nz, e, v, (int)(m - m0));
-      ++e;
+  for (int64_t mb = m0; mb < m1; mb += kRowBatch) {
+    S a[kRowBatch];
+#pragma unroll
+    for (int i = 0; i < kRowBatch; ++i) a[i] = mb + i < m1 ? A[(mb + i) * g.lda + k] : S(0);
+#pragma unroll
+    for (int i = 0; i < kRowBatch; ++i) {
+      D v;
+      if (mb + i < m1 && Conv<S, D>::get(a[i], scale ? scale[mb + i] : 1.0f, v)) {
+        put_rec(w.nz, e, v, (int)(mb + i - m0));
+        ++e;
+      }
     }
   }
 }
@@ -418,42 +441,73 @@ __device__ void scatter(const S* __restrict__ A, const PackGeom& g,
 // Row-slot stream: each row's records (k ascending) at its scanned offset,
 // then its sentinel; with the gather stream, the same record re-addressed by
 // the slot of k in the tile's union list goes to the same position of gnz.
-template <class S, class D>
+// W warps share a row (W = kRowsPerBlock: the whole block) and take turns of
+// 256 columns each: a step's loads are issued together, the step after is
+// fetched while this one is written, and a warp starts where the counts of
+// the warps before it end.
+template <class S, class D, int W>
 __device__ void row_write(const S* __restrict__ A, const PackGeom& g,
                           const float* __restrict__ scale, int64_t b, const WriteArgs& w) {
-  const int64_t row = b * kRowsPerBlock + threadIdx.x / 32;
-  const int lane = threadIdx.x & 31;
-  if (row >= g.M) return;
+  __shared__ int cnt[2][kRowsPerBlock];
+  const int wid = threadIdx.x / 32, lane = threadIdx.x & 31;
+  const int64_t row = W == 1 ? b * kRowsPerBlock + wid : b;
+  if (row >= g.M) return;   // (uniform over a block that shares a row)
   const float sc = scale ? scale[row] : 1.0f;
   int64_t pos = w.rcnt[row].x;
-  if (lane == 0) w.rowptr[row] = (int32_t)pos;
+  const bool first = lane == 0 && (W == 1 || wid == 0);
+  if (first) w.rowptr[row] = (int32_t)pos;
   const int2* tf = w.flag ? w.flag + (row / kDenseTileRows) * g.K : nullptr;
   const int32_t base = tf ? tf[0].x : 0;
-  // eight 32-column groups per step: their loads are issued together, then
-  // the records are written in k order
   constexpr int G = 8;
-  for (int64_t k0 = 0; k0 < g.K; k0 += 32 * G) {
-    S a[G];
+  const int64_t kw = W == 1 ? 0 : wid * 32 * G;
+  S nx[G];
+  auto fetch = [&](int64_t k0) {
 #pragma unroll
     for (int u = 0; u < G; ++u) {
-      const int64_t k = k0 + u * 32 + lane;
-      a[u] = k < g.K ? A[row * g.lda + k] : S(0);
+      const int64_t k = k0 + kw + u * 32 + lane;
+      nx[u] = k < g.K ? A[row * g.lda + k] : S(0);
+    }
+  };
+  fetch(0);
+  int turn = 0;
+  for (int64_t k0 = 0; k0 < g.K; k0 += 32 * G * W) {
+    D v[G];
+    unsigned mask[G];
+    int total = 0;
+#pragma unroll
+    for (int u = 0; u < G; ++u) {
+      const int64_t k = k0 + kw + u * 32 + lane;
+      mask[u] = __ballot_sync(0xffffffffu, k < g.K && Conv<S, D>::get(nx[u], sc, v[u]));
+      total += __popc(mask[u]);
+    }
+    fetch(k0 + 32 * G * W);
+    int64_t q0 = pos;
+    if constexpr (W > 1) {
+      // (two sets of counts in turn: one barrier per step)
+      if (lane == 0) cnt[turn][wid] = total;
+      __syncthreads();
+#pragma unroll
+      for (int i = 0; i < W; ++i) {
+        const int c = cnt[turn][i];
+        if (i < wid) q0 += c;
+        pos += c;
+      }
+      turn ^= 1;
+    } else {
+      pos += total;
     }
 #pragma unroll
     for (int u = 0; u < G; ++u) {
-      const int64_t k = k0 + u * 32 + lane;
-      D v;
-      const bool nzf = (k < g.K) && Conv<S, D>::get(a[u], sc, v);
-      const unsigned mask = __ballot_sync(0xffffffffu, nzf);
-      if (nzf) {
-        const int64_t q = pos + __popc(mask & ((1u << lane) - 1u));
-        put_row_rec(w.rnz, q, v, (int)k);
-        if (tf) put_row_rec(w.gnz, q, v, (int)(tf[k].x - base));
+      if (mask[u] >> lane & 1u) {
+        const int64_t k = k0 + kw + u * 32 + lane;
+        const int64_t q = q0 + __popc(mask[u] & ((1u << lane) - 1u));
+        put_row_rec(w.rnz, q, v[u], (int)k);
+        if (tf) put_row_rec(w.gnz, q, v[u], (int)(tf[k].x - base));
       }
-      pos += __popc(mask);
+      q0 += __popc(mask[u]);
     }
   }
-  if (lane == 0) {
+  if (first) {
     put_row_sentinel<D>(w.rnz, pos);
     if (tf) put_row_sentinel<D>(w.gnz, pos);
   }
@@ -471,21 +525,42 @@ __device__ void tile_union(const PackGeom& g, int64_t b, const WriteArgs& w) {
 
 // The dense copy holds each entry converted exactly as the packer converts
 // it (BF16 packs: the BF16 value; INT8 packs: the INT8 code, exact in BF16).
+// A thread writes eight columns of a row (16 bytes; Kpad is a multiple of
+// eight), read with 16-byte loads where A's rows are 16-byte aligned.
 template <class S, class D>
 __device__ void densify(const S* __restrict__ A, const PackGeom& g,
                         const float* __restrict__ scale, int64_t b, const WriteArgs& w) {
-  const int64_t k = (b % w.gxd) * kPackThreads + threadIdx.x;
+  const int64_t k = ((b % w.gxd) * kPackThreads + threadIdx.x) * 8;
   if (k >= w.Kpad) return;
+  const bool vec = w.a_vec && k + 8 <= g.K;
   for (int64_t rr = b / w.gxd; rr < w.dense_rows; rr += w.ry) {
     const int64_t row = (int64_t)w.tile_order[rr / kDenseTileRows] * kDenseTileRows +
                         rr % kDenseTileRows;
-    __nv_bfloat16 v = __float2bfloat16_rn(0.0f);
-    if (row < g.M && k < g.K) {
-      D q;
-      Conv<S, D>::get(A[row * g.lda + k], scale ? scale[row] : 1.0f, q);
-      v = to_bf16(q);
+    alignas(16) __nv_bfloat16 o[8];
+    alignas(16) S a[8];
+    const bool in = row < g.M;
+    const S* src = A + row * g.lda + k;
+    if (vec && in) {
+      constexpr int W = (int)sizeof(S) * 8;   // 8, 16 or 32 bytes
+      if constexpr (W == 8) {
+        *reinterpret_cast<uint2*>(a) = __ldg(reinterpret_cast<const uint2*>(src));
+      } else {
+#pragma unroll
+        for (int i = 0; i < W / 16; ++i)
+          reinterpret_cast<uint4*>(a)[i] = __ldg(reinterpret_cast<const uint4*>(src) + i);
+      }
+    } else {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) a[i] = in && k + i < g.K ? src[i] : S(0);
     }
-    w.dense_A[rr * w.Kpad + k] = v;
+    const float sc = scale && in ? scale[row] : 1.0f;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      D q;
+      Conv<S, D>::get(a[i], sc, q);
+      o[i] = in && k + i < g.K ? to_bf16(q) : __float2bfloat16_rn(0.0f);
+    }
+    *reinterpret_cast<uint4*>(w.dense_A + rr * w.Kpad + k) = *reinterpret_cast<const uint4*>(o);
   }
 }
 
@@ -510,11 +585,17 @@ __device__ void tails(const PackGeom& g, const WriteArgs& w) {
 }
 
 // Phase 2 in one launch: scatter, row write (+ gather records), union lists,
-// dense copies, then one block of terminating entries.
+// dense copies, then one block of terminating entries.  A is read from L2 by
+// each of them; what bounds the launch is loads in flight, so a panel column
+// fetches its sixteen rows together, a row its next 256 columns while it writes
+// the last, and a dense copy eight columns per thread (512 x 4608 at 95 %:
+// 35 -> 16 us; transposed 35 -> 14).
 template <class S, class D>
 __global__ void __launch_bounds__(kPackThreads)
     pack_write_kernel(const S* __restrict__ A, PackGeom g, const float* __restrict__ scale,
                       WriteArgs w) {
+  pdl_wait();
+  pdl_trigger();
   int64_t b = blockIdx.x;
   if (b < w.b_scatter) {
     scatter<S, D>(A, g, scale, b, w);
@@ -522,7 +603,10 @@ __global__ void __launch_bounds__(kPackThreads)
   }
   b -= w.b_scatter;
   if (b < w.b_row) {
-    row_write<S, D>(A, g, scale, b, w);
+    if (w.row_warps > 1)
+      row_write<S, D, kRowsPerBlock>(A, g, scale, b, w);
+    else
+      row_write<S, D, 1>(A, g, scale, b, w);
     return;
   }
   b -= w.b_row;
@@ -572,6 +656,10 @@ __global__ void fill_kernel(float* __restrict__ out, int64_t n, float v) {
 // Planned on the device: the host only learns how many pieces each panel has.
 // (Planned on the host, the piece lists and their sorting took 266 us of the
 // 388 us pack of a 4608 x 512 matrix, and 1.9 of 2.7 ms for 11008 x 4096.)
+// What bounds the writing kernel is the chain of row -> records -> entries of a
+// half-warp: one block per 256 rows took 33 us for 512 x 4608 at 95 % (two
+// blocks); several blocks that plan the same rows and share the writing, four
+// pieces of a row in flight: 8 us.
 //
 // lpt order: pieces by length class, longest first, ties in row order.  A
 // class is a range of lengths (kSegClasses of them between the list's piece
@@ -580,6 +668,7 @@ __global__ void fill_kernel(float* __restrict__ out, int64_t n, float v) {
 // offsets, and the writing kernel ranks the pieces inside a block.
 constexpr int kSegRows = 256;      // rows per block of both kernels
 constexpr int kSegClasses = 64;
+constexpr int kSegBatch = 4;       // pieces of a row that are in flight together
 
 __host__ __device__ inline int seg_class_shift(int seg) {
   int s = 0;
@@ -618,6 +707,7 @@ __global__ void __launch_bounds__(kSegRows)
                         const int* __restrict__ touched_total, int64_t M,
                         const int2* __restrict__ flag, int64_t nf, int64_t* __restrict__ sum64,
                         SegCount sc) {
+  pdl_wait();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int nnz = cnt[n].x;
   if (i == 0) {
@@ -698,6 +788,7 @@ struct SegWrite {
   int rec_words, m_r, nblk, lists;
 };
 __global__ void __launch_bounds__(2 * kSegRows) seg_write_kernel(const SegWrite w) {
+  pdl_wait();
   __shared__ int first[kSegRows], len[kSegRows];
   __shared__ int at_full[2][kSegRows], at_rem[2][kSegRows], at_ord[2][kSegRows];
   __shared__ int base[2][kSegRows / 32][kSegClasses];   // per warp and class
@@ -756,25 +847,36 @@ __global__ void __launch_bounds__(2 * kSegRows) seg_write_kernel(const SegWrite 
   __syncthreads();
   const int l16 = threadIdx.x & 15;
   const int words = 12 / w.rec_words * w.rec_words;   // inline words of whole records
-  for (int it = threadIdx.x >> 4; it < w.lists * kSegRows; it += 2 * kSegRows / 16) {
+  const int groups = 2 * kSegRows / 16;
+  for (int it = blockIdx.y * groups + (threadIdx.x >> 4); it < w.lists * kSegRows;
+       it += gridDim.y * groups) {
     const int gg = it >> 8, rr = it & (kSegRows - 1);
     const int n = len[rr];
     if (n < 0) continue;
     const int sg = w.seg[gg];
     const int ns = n > sg ? (n + sg - 1) / sg : 1;
-    for (int k = 0; k < ns; ++k) {
-      const int a = first[rr] + k * sg;
-      const int e = k + 1 < ns ? a + sg : first[rr] + n;
-      uint32_t v = 0;
-      if (l16 == 0) v = (uint32_t)(blockIdx.x * kSegRows + rr);
-      else if (l16 == 1) v = (uint32_t)a;
-      else if (l16 == 2) v = (uint32_t)e;
-      else if (l16 == 3) v = ns > 1 ? 1u : 0u;
-      else if (l16 - 4 < words && l16 - 4 < (e - a) * w.rec_words)
-        v = w.rnz[(int64_t)a * w.rec_words + l16 - 4];
-      const int to = k + 1 < ns ? at_full[gg][rr] + k : at_rem[gg][rr];
-      reinterpret_cast<uint32_t*>(&w.lpt[gg][to])[l16] = v;
-      if (w.ord[gg]) reinterpret_cast<uint32_t*>(&w.ord[gg][at_ord[gg][rr] + k])[l16] = v;
+    for (int k0 = 0; k0 < ns; k0 += kSegBatch) {
+      uint32_t v[kSegBatch];
+#pragma unroll
+      for (int i = 0; i < kSegBatch; ++i) {
+        const int k = k0 + i, a = first[rr] + k * sg;
+        const int e = k + 1 < ns ? a + sg : first[rr] + n;
+        v[i] = 0;
+        if (l16 == 0) v[i] = (uint32_t)(blockIdx.x * kSegRows + rr);
+        else if (l16 == 1) v[i] = (uint32_t)a;
+        else if (l16 == 2) v[i] = (uint32_t)e;
+        else if (l16 == 3) v[i] = ns > 1 ? 1u : 0u;
+        else if (k < ns && l16 - 4 < words && l16 - 4 < (e - a) * w.rec_words)
+          v[i] = w.rnz[(int64_t)a * w.rec_words + l16 - 4];
+      }
+#pragma unroll
+      for (int i = 0; i < kSegBatch; ++i) {
+        const int k = k0 + i;
+        if (k >= ns) break;
+        const int to = k + 1 < ns ? at_full[gg][rr] + k : at_rem[gg][rr];
+        reinterpret_cast<uint32_t*>(&w.lpt[gg][to])[l16] = v[i];
+        if (w.ord[gg]) reinterpret_cast<uint32_t*>(&w.ord[gg][at_ord[gg][rr] + k])[l16] = v[i];
+      }
     }
   }
 }
@@ -930,12 +1032,22 @@ rosko_status pack_typed(const S* A, int64_t lda, const float* scale_in, bool qua
   // still gets its sentinel from a row block
   const int64_t b_row_count = (rows && n == 0) ? (M + kRowsPerBlock - 1) / kRowsPerBlock : 0;
   if (b_col + b_row_count > 0) {
-    pack_count_kernel<S, D><<<(unsigned)(b_col + b_row_count), kPackThreads, 0, st>>>(
-        A, geo, scale, cnt, touched, tot + 2, rcnt, flag, b_col);
+    // (the launches of a phase are programmatic dependents of one another:
+    // each is scheduled while the one before it ends)
+    if (launch_dependent(pack_count_kernel<S, D>, dim3((unsigned)(b_col + b_row_count)),
+                         dim3(kPackThreads), 0, st, A, geo, scale, cnt, touched, tot + 2, rcnt,
+                         flag, b_col) != cudaSuccess)
+      return ROSKO_ERR_CUDA;
     count_launches(1);
   }
   // the writing phase's ranges
-  const int64_t b_row = rows ? (M + kRowsPerBlock - 1) / kRowsPerBlock : 0;
+  // A warp per row is a chain of steps of 256 columns, which few rows leave
+  // exposed: up to 16 warps per SM a block shares each row (whole pack, BF16,
+  // a warp per row -> a block: 512x4608 at 50 % 148 -> 119 us, at 95 % 118 -> 98;
+  // above that it only adds barriers: 4608x512 110 -> 131, 4096x4096 241 -> 250).
+  // Rows of one step stay with a warp.
+  const bool share_rows = M <= 16 * (int64_t)num_sms() && K > 256;
+  const int64_t b_row = !rows ? 0 : share_rows ? M : (M + kRowsPerBlock - 1) / kRowsPerBlock;
   const int64_t b_tile = gather ? geo.gx * T : 0;
   {
     ScanSet ss;
@@ -955,9 +1067,13 @@ rosko_status pack_typed(const S* A, int64_t lda, const float* scale_in, bool qua
     if (gather) add(flag, nf, o_fsums);
     if (ss.count > 0) {
       const unsigned tiles = (unsigned)ss.first[ss.count];
-      scan_reduce_kernel<<<tiles, kScanThreads, 0, st>>>(ss);
-      scan_spine_kernel<<<(unsigned)ss.count, kScanThreads, 0, st>>>(ss);
-      scan_down_kernel<<<tiles, kScanThreads, 0, st>>>(ss);
+      if (launch_dependent(scan_reduce_kernel, dim3(tiles), dim3(kScanThreads), 0, st, ss) !=
+              cudaSuccess ||
+          launch_dependent(scan_spine_kernel, dim3((unsigned)ss.count), dim3(kScanThreads), 0, st,
+                           ss) != cudaSuccess ||
+          launch_dependent(scan_down_kernel, dim3(tiles), dim3(kScanThreads), 0, st, ss) !=
+              cudaSuccess)
+        return ROSKO_ERR_CUDA;
       count_launches(3);
     }
   }
@@ -973,8 +1089,10 @@ rosko_status pack_typed(const S* A, int64_t lda, const float* scale_in, bool qua
       sc.m_r = h->m_r;
       sc.nblk = (int)nblk;
     }
-    pack_summary_kernel<<<(unsigned)((span + kSegRows - 1) / kSegRows), kSegRows, 0, st>>>(
-        cnt, n, P, K, tot + 2, M, flag, nf, reinterpret_cast<int64_t*>(sb + o_sum64), sc);
+    if (launch_dependent(pack_summary_kernel, dim3((unsigned)((span + kSegRows - 1) / kSegRows)),
+                         dim3(kSegRows), 0, st, cnt, n, P, K, tot + 2, M, flag, nf,
+                         reinterpret_cast<int64_t*>(sb + o_sum64), sc) != cudaSuccess)
+      return ROSKO_ERR_CUDA;
     count_launches(1);
   }
   std::vector<int64_t> summary((summary_bytes + 7) / 8);
@@ -1104,19 +1222,22 @@ rosko_status pack_typed(const S* A, int64_t lda, const float* scale_in, bool qua
   w.zero_panels = n == 0 ? 1 : 0;
   w.b_scatter = b_col;
   w.b_row = b_row;
+  w.row_warps = share_rows ? kRowsPerBlock : 1;
   w.b_union = b_tile;
   if (dense && h->n_copy > 0) {
     w.tile_order = h->tile_order_dev;
     w.dense_A = reinterpret_cast<__nv_bfloat16*>(h->dense_A);
     w.dense_rows = h->n_copy * kDenseTileRows;
     w.Kpad = h->Kpad;
-    w.gxd = (h->Kpad + kPackThreads - 1) / kPackThreads;
+    w.gxd = (h->Kpad / 8 + kPackThreads - 1) / kPackThreads;
+    w.a_vec = reinterpret_cast<uintptr_t>(A) % 16 == 0 && (lda * (int64_t)sizeof(S)) % 16 == 0;
     w.ry = std::min<int64_t>(w.dense_rows, 2048);
     w.b_dense = w.gxd * w.ry;
   }
-  pack_write_kernel<S, D>
-      <<<(unsigned)(w.b_scatter + w.b_row + w.b_union + w.b_dense + 1), kPackThreads, 0, st>>>(
-          A, geo, scale, w);
+  if (launch_dependent(pack_write_kernel<S, D>,
+                       dim3((unsigned)(w.b_scatter + w.b_row + w.b_union + w.b_dense + 1)),
+                       dim3(kPackThreads), 0, st, A, geo, scale, w) != cudaSuccess)
+    return ROSKO_ERR_CUDA;
   count_launches(1);
   if (rows) {
     // the work segments, once the row stream is written
@@ -1137,7 +1258,13 @@ rosko_status pack_typed(const S* A, int64_t lda, const float* scale_in, bool qua
     sw.m_r = h->m_r;
     sw.nblk = (int)nblk;
     sw.lists = lists;
-    seg_write_kernel<<<(unsigned)nblk, 2 * kSegRows, 0, st>>>(sw);
+    // several blocks plan the same rows and share the writing until the SMs
+    // have a block each (a part for every half-warp's one row at most)
+    const int64_t parts =
+        std::min<int64_t>(lists * 16 / 2, std::max<int64_t>(1, num_sms() / std::max<int64_t>(nblk, 1)));
+    if (launch_dependent(seg_write_kernel, dim3((unsigned)nblk, (unsigned)parts),
+                         dim3(2 * kSegRows), 0, st, sw) != cudaSuccess)
+      return ROSKO_ERR_CUDA;
     count_launches(1);
   }
   // the scratch is released on return: wait for the writes that read it
