@@ -236,8 +236,8 @@ rosko_status rosko_spmm_plan(rosko_packed_t A, const void* B_dev, rosko_dtype b_
  * width (128 or 256 columns, each problem taking the width its tile or the
  * analytic rule gives it), whose work list
  * (per-problem TMA descriptors and sizes) is passed in the kernel
- * parameters; the row-direct sparse remainders share one launch, other
- * remainders run one launch per problem.  Per-problem arrays: A, B (device),
+ * parameters; the row-direct sparse remainders of one strip width share one
+ * launch, other remainders run one launch per problem.  Per-problem arrays: A, B (device),
  * N, ldb, C (device), ldc; all problems share b_dtype and c_dtype.  tiles:
  * NULL (analytic rule) or `count` tiles (e.g. from rosko_autotune).  No
  * device memory is allocated

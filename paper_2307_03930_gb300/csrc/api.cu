@@ -474,8 +474,8 @@ rosko_status spmm_run(rosko_packed_s* A, const void* B_dev, rosko_dtype b_dtype,
                       int64_t ldb, const float* col_scale_dev, void* C_dev, rosko_dtype c_dtype,
                       int64_t ldc, int accumulate, const rosko_tile* tile, cudaStream_t st,
                       int flags) {
-  // flags: kRunSkipDense = the dense tiles were launched elsewhere (batch);
-  //        kRunZeroed    = C was zeroed by the caller
+  // flags: kRunSkipDense = the dense tiles were launched elsewhere (batch), and C was
+  //        zeroed before them where anything adds into it
   const rosko_dtype p = A->dt;
   const size_t bsz = dtype_size(b_dtype);
   const size_t csz = dtype_size(c_dtype);
@@ -617,7 +617,8 @@ rosko_status spmm_run(rosko_packed_s* A, const void* B_dev, rosko_dtype b_dtype,
   // the zero fill runs under the tensor-core launch when there is one (a
   // small kernel it depends on programmatically), else as a memset
   const bool run_dense = n_dense > 0 && !skip_dense;
-  const bool fill = zero_c && !(flags & kRunZeroed);
+  // (never after the batch's tensor-core launch: it would erase finished tiles)
+  const bool fill = zero_c && !skip_dense;
   const ZeroFill zf{C_dev, ldc * (int64_t)csz, N * (int64_t)csz, A->M};
   if (fill && !run_dense &&
       cudaMemset2DAsync(C_dev, (size_t)ldc * csz, 0, (size_t)N * csz, (size_t)A->M, st) !=
@@ -721,6 +722,10 @@ rosko_status spmm_batched_impl(int32_t count, rosko_packed_s* const* A, const vo
   std::vector<int> job_of;        // problem index of each dense job
   std::vector<rosko_tile> rest;   // per problem: tile for the sparse remainder
   std::vector<char> active((size_t)count, 0), dense_any((size_t)count, 0);
+  // row-direct remainders: columns per lane (0: another traversal) and whether
+  // a row of theirs is cut.  Resolved once: the zero fill ahead of every launch
+  // and the launch itself have to agree on both.
+  std::vector<int> direct_V((size_t)count, 0);
   std::vector<char> direct_cut((size_t)count, 0);
   rest.resize((size_t)count);
   // dense tiles run in one launch per tile width: each problem takes the
@@ -785,13 +790,15 @@ rosko_status spmm_batched_impl(int32_t count, rosko_packed_s* const* A, const vo
     if (r.split_k <= 0) r.split_k = t.split_k;
     if ((r.order > 0 ? r.order : t.order) == 4) {
       r.split_k = 1;   // row-direct: no K split, but cut rows add into C
-      int64_t ns = 0;
-      bool cut = false;
       const int V = r.n_r > 0 ? r.n_r / 32 : sparse_default_V(A[i]->dt, A[i]->m_r, 4);
-      const int which = direct_pick(A[i], A[i]->panel_order_dev, A[i]->P - dp, N[i], V);
-      if (A[i]->rnz &&
-          direct_segments(A[i], A[i]->panel_order_dev, A[i]->P - dp, which, &ns, &cut) && cut)
-        direct_cut[(size_t)i] = 1;
+      if (A[i]->rnz && sparse_config_supported(A[i]->dt, b_dt, c_dt, A[i]->m_r, V, 4)) {
+        int64_t ns = 0;
+        bool cut = false;
+        const int which = direct_pick(A[i], A[i]->panel_order_dev, A[i]->P - dp, N[i], V);
+        direct_V[(size_t)i] = V;
+        if (direct_segments(A[i], A[i]->panel_order_dev, A[i]->P - dp, which, &ns, &cut) && cut)
+          direct_cut[(size_t)i] = 1;
+      }
     }
     rest[(size_t)i] = r;
     // whole-dense problems need no sparse launch
@@ -799,7 +806,6 @@ rosko_status spmm_batched_impl(int32_t count, rosko_packed_s* const* A, const vo
   }
   // zero every C that some kernel adds into: dense tiles cut by the stream-K
   // split, or a sparse remainder split along K (before any launch)
-  std::vector<char> zeroed((size_t)count, 0);
   if (!accumulate) {
     std::vector<char> need((size_t)count, 0);
     for (int g = 0; g < 2; ++g) {
@@ -826,7 +832,6 @@ rosko_status spmm_batched_impl(int32_t count, rosko_packed_s* const* A, const vo
       if (cudaMemset2DAsync(C[i], (size_t)ldc[i] * csz, 0, (size_t)N[i] * csz, (size_t)A[i]->M,
                             st) != cudaSuccess)
         return ROSKO_ERR_CUDA;
-      zeroed[(size_t)i] = 1;
     }
   }
   for (int g = 0; g < 2; ++g) {
@@ -839,39 +844,30 @@ rosko_status spmm_batched_impl(int32_t count, rosko_packed_s* const* A, const vo
     if (s != ROSKO_OK) return s;
   }
   // sparse remainders (the dense tiles were launched above): the row-direct
-  // ones (order 4, one V) share one launch, the others run one per problem
-  std::vector<DirectJob> direct;
-  std::vector<char> in_direct((size_t)count, 0);
-  int direct_V = 0;
-  for (int32_t i = 0; i < count; ++i) {
-    if (!active[(size_t)i] || rest[(size_t)i].m_r == -1) continue;
-    const rosko_tile& r = rest[(size_t)i];
-    rosko_tile t{};
-    schedule_analytic(A[i]->M, A[i]->K, N[i], A[i]->nnz, A[i]->m_r, A[i]->dt, sms, &t);
-    const int ord = r.order > 0 ? r.order : t.order;
-    if (ord != 4 || !A[i]->rnz) continue;
-    const int V = r.n_r > 0 ? r.n_r / 32 : sparse_default_V(A[i]->dt, A[i]->m_r, 4);
-    if (!sparse_config_supported(A[i]->dt, b_dt, c_dt, A[i]->m_r, V, 4)) continue;
-    if (direct_V != 0 && V != direct_V) continue;
-    int64_t nd = 0, dp = 0;
-    dense_prefix(A[i], r.dense_split_pm, &nd, &dp);
-    DirectJob j{A[i], B[i], b_dt, N[i], ldb[i], nullptr, C[i], c_dt, ldc[i], accumulate,
-                A[i]->panel_order_dev, A[i]->P - dp};
-    direct.push_back(j);
-    direct_V = V;
-    in_direct[(size_t)i] = 1;
-  }
-  if (!direct.empty()) {
-    rosko_status s = direct_batch_launch(direct.data(), (int)direct.size(), direct_V, st);
+  // ones of one width share a launch, the others run one per problem
+  std::vector<char> launched((size_t)count, 0);
+  for (int32_t first = 0; first < count; ++first) {
+    if (direct_V[(size_t)first] == 0 || launched[(size_t)first] || rest[(size_t)first].m_r == -1)
+      continue;
+    const int V = direct_V[(size_t)first];
+    std::vector<DirectJob> direct;
+    for (int32_t i = first; i < count; ++i) {
+      if (direct_V[(size_t)i] != V || rest[(size_t)i].m_r == -1) continue;
+      int64_t nd = 0, dp = 0;
+      dense_prefix(A[i], rest[(size_t)i].dense_split_pm, &nd, &dp);
+      direct.push_back(DirectJob{A[i], B[i], b_dt, N[i], ldb[i], nullptr, C[i], c_dt, ldc[i],
+                                 accumulate, A[i]->panel_order_dev, A[i]->P - dp});
+      launched[(size_t)i] = 1;
+    }
+    rosko_status s = direct_batch_launch(direct.data(), (int)direct.size(), V, st);
     if (s != ROSKO_OK) return s;
   }
   for (int32_t i = 0; i < count; ++i) {
-    if (!active[(size_t)i] || rest[(size_t)i].m_r == -1 || in_direct[(size_t)i]) continue;
+    if (!active[(size_t)i] || rest[(size_t)i].m_r == -1 || launched[(size_t)i]) continue;
     rosko_tile r = rest[(size_t)i];
     r.m_r = 0;
-    const int flags = kRunSkipDense | (zeroed[(size_t)i] ? kRunZeroed : 0);
     rosko_status s = spmm_run(A[i], B[i], b_dt, N[i], ldb[i], nullptr, C[i], c_dt, ldc[i],
-                              accumulate, &r, st, flags);
+                              accumulate, &r, st, kRunSkipDense);
     if (s != ROSKO_OK) return s;
   }
   return ROSKO_OK;

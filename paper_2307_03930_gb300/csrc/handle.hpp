@@ -277,7 +277,6 @@ rosko_status spmm_validate(rosko_packed_s* A, const void* B_dev, rosko_dtype b_d
                            rosko_dtype c_dtype, int64_t ldc, int accumulate, cudaStream_t st,
                            bool* done);
 constexpr int kRunSkipDense = 1;
-constexpr int kRunZeroed = 2;
 constexpr int kRunPlanOnly = 4;   // resolve the schedule, launch nothing (rosko_spmm_plan)
 rosko_status spmm_run(rosko_packed_s* A, const void* B_dev, rosko_dtype b_dtype, int64_t N,
                       int64_t ldb, const float* col_scale_dev, void* C_dev, rosko_dtype c_dtype,
