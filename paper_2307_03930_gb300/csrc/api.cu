@@ -211,6 +211,21 @@ constexpr int kDenseCopyPm = 1;
 constexpr int kDenseSplitPmI8 = 15;
 constexpr int kDenseCopyPmI8 = 10;
 
+// BF16 layers of little work stay with the FMAs, whatever the tensor cores
+// would save: the tensor core truncates every addition where an FMA rounds,
+// and its sums are 1.1 to 6 times as far from the 64-bit result (176x1465x29
+// at 58 %: 8.1e-8 / 4.9e-7; 1053x148x8325 at 76 %: 1.3e-8 / 1.6e-8).  The line
+// is where the time that is saved gets to several times the launch: it
+// compares the multiply-adds of the whole layer with those of its nonzeros.
+// (Letting 16 uneven layers of a batch cross it takes 102 us, 135 with it, and
+// up to 5 times the error in the layers that cross; a caller who wants that
+// gives dense_split_pm.)
+static bool bf16_little_work(int64_t M, int64_t K, int64_t N, int64_t nnz) {
+  const double all = 10.8 + 2.0 * (double)M * (double)K * (double)N / 0.58e15 * 1e6;
+  const double nonzeros = 5.3 + (double)nnz * (double)N * 2.0 / 10.9e12 * 1e6;
+  return nonzeros < all;
+}
+
 // ---------------------------------------------------------------------------
 // Analytic schedule: Sec. 4.2 re-derived for one GB300.
 //
@@ -281,7 +296,8 @@ rosko_status schedule_analytic(int64_t M, int64_t K, int64_t N, int64_t nnz, int
     double t_direct = direct_time_us(M, N, nnz, dt, sms);
     const int lpr = narrow_pick(M, K, N, nnz, dt, sms);
     if (lpr > 0) t_direct = std::min(t_direct, narrow_time_us(M, K, N, nnz, dt, lpr, sms));
-    if (t_direct < t_dense) t->dense_split_pm = 1001;
+    if (t_direct < t_dense || (dt == ROSKO_BF16 && bf16_little_work(M, K, N, nnz)))
+      t->dense_split_pm = 1001;
   }
   t->dense_n_r = TN;
   t->dense_split_k = ds;
@@ -669,50 +685,6 @@ static void dense_prefix(const rosko_packed_s* A, int32_t pm, int64_t* n_dense,
   }
 }
 
-// The dense-split threshold of every problem of a batch whose caller gives
-// none.  A problem alone is kept sparse when row-direct is predicted faster
-// (schedule_analytic), fixed costs of the launch included; in a batch those
-// are paid once, so each problem goes where it adds less, and when the
-// remaining row-direct problems could all be dense they are, unless their own
-// launch (its ~4 us, their longest chain of records) is predicted cheaper.
-// 16 uneven layers: 135 -> 98 us.
-static void batch_split(int32_t count, rosko_packed_s* const* A, const int64_t* N,
-                        const rosko_tile* tiles, const std::vector<char>& active, int sms,
-                        std::vector<int32_t>* pm) {
-  double direct_work = 0.0, chain = 0.0, dense_work = 0.0;
-  bool must = false;   // some problem has to run row-direct
-  bool any = false;    // there is a tensor-core launch at all
-  std::vector<int32_t> movable;
-  for (int32_t i = 0; i < count; ++i)
-    any |= active[(size_t)i] && A[i]->dt == ROSKO_BF16 && (*pm)[(size_t)i] <= 1000;
-  if (!any) return;
-  for (int32_t i = 0; i < count; ++i) {
-    if (!active[(size_t)i] || A[i]->dt != ROSKO_BF16) continue;
-    if (tiles && tiles[i].dense_split_pm > 0) continue;
-    const rosko_packed_s* h = A[i];
-    // whole problems only: every tile dense enough for the tensor cores
-    const bool can = h->n_copy == h->n_tiles && h->n_tiles > 0 && h->rnz &&
-                     h->tile_density.back() * 1000.0 >= (double)kDenseSplitPm;
-    if (!can) {
-      must |= (*pm)[(size_t)i] > 1000;
-      continue;
-    }
-    int TN = 256, ds = 1, mc = 128;
-    dense_config(h->n_tiles, N[i], h->K, sms, &TN, &ds, &mc, false);
-    const double de = dense_marginal_us(h->n_tiles, N[i], h->K, TN);
-    const double di = direct_marginal_us(h->M, N[i], h->nnz, h->dt, sms);
-    (*pm)[(size_t)i] = de < di ? kDenseSplitPm : 1001;
-    if (de >= di) {
-      movable.push_back(i);
-      direct_work += di;
-      dense_work += de;
-      chain = std::max(chain, (double)h->nnz / (double)h->M * 0.05);
-    }
-  }
-  if (!must && 4.0 + std::max(direct_work, chain) > dense_work)
-    for (int32_t i : movable) (*pm)[(size_t)i] = kDenseSplitPm;
-}
-
 rosko_status spmm_batched_impl(int32_t count, rosko_packed_s* const* A, const void* const* B,
                                const int64_t* N, const int64_t* ldb, void* const* C,
                                const int64_t* ldc, rosko_dtype b_dt, rosko_dtype c_dt,
@@ -733,8 +705,6 @@ rosko_status spmm_batched_impl(int32_t count, rosko_packed_s* const* A, const vo
   // as soon as one of its problems has two row tiles
   std::vector<int> job_tn;
   int group_cg[2] = {1, 1};
-  std::vector<rosko_tile> rule((size_t)count);
-  std::vector<int32_t> pm((size_t)count, 1001);
   for (int32_t i = 0; i < count; ++i) {
     bool done = false;
     rosko_status v = spmm_validate(A[i], B[i], b_dt, N[i], ldb[i], nullptr, C[i], c_dt, ldc[i],
@@ -742,16 +712,13 @@ rosko_status spmm_batched_impl(int32_t count, rosko_packed_s* const* A, const vo
     if (v != ROSKO_OK) return v;
     if (done) continue;
     active[(size_t)i] = 1;
-    schedule_analytic(A[i]->M, A[i]->K, N[i], A[i]->nnz, A[i]->m_r, A[i]->dt, sms,
-                      &rule[(size_t)i]);
-    pm[(size_t)i] = rule[(size_t)i].dense_split_pm;
-    if (tiles && tiles[i].dense_split_pm > 0) pm[(size_t)i] = tiles[i].dense_split_pm;
-  }
-  batch_split(count, A, N, tiles, active, sms, &pm);
-  for (int32_t i = 0; i < count; ++i) {
-    if (!active[(size_t)i]) continue;
-    rosko_tile& t = rule[(size_t)i];
-    t.dense_split_pm = pm[(size_t)i];
+    rosko_tile t{};
+    schedule_analytic(A[i]->M, A[i]->K, N[i], A[i]->nnz, A[i]->m_r, A[i]->dt, sms, &t);
+    // the launches' fixed costs are shared: only the work decides
+    if (A[i]->dt == ROSKO_BF16 && t.order == 4)
+      t.dense_split_pm =
+          bf16_little_work(A[i]->M, A[i]->K, N[i], A[i]->nnz) ? 1001 : kDenseSplitPm;
+    if (tiles && tiles[i].dense_split_pm > 0) t.dense_split_pm = tiles[i].dense_split_pm;
     // the batch's tensor-core launches are BF16 only: other packs run sparse
     if (A[i]->dt != ROSKO_BF16) t.dense_split_pm = 1001;
     int64_t nd = 0, dp = 0;

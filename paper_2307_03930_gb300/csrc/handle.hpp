@@ -179,7 +179,6 @@ struct SparseLaunch {
 int narrow_chunks(rosko_dtype p_dt, int64_t K, int64_t N);
 double narrow_time_us(int64_t M, int64_t K, int64_t N, int64_t nnz, rosko_dtype dt, int lpr,
                       int sms);
-double direct_marginal_us(int64_t M, int64_t N, int64_t nnz, rosko_dtype dt, int sms);
 double direct_time_us(int64_t M, int64_t N, int64_t nnz, rosko_dtype dt, int sms);
 // The narrow kernel's chunks per strip where it is predicted faster than the
 // general row-direct kernel, else 0.
@@ -267,7 +266,6 @@ void dense_batch_needs_zero(const DenseJob* jobs, int count, int TN, int cg, boo
 // split over `ctas` CTAs cuts a tile
 int dense_group(int64_t n_tiles);
 // Estimated time (us) of a single problem's launches on the tensor cores.
-double dense_marginal_us(int64_t n_tiles, int64_t N, int64_t K, int TN);
 double dense_time_us(int64_t n_tiles, int64_t N, int64_t K, int TN, int ctas, bool i8);
 bool dense_needs_zero(int64_t n_tiles, int64_t N, int64_t K, int TN, int ctas, bool i8);
 

@@ -1024,14 +1024,6 @@ double dense_time_us(int64_t n_tiles, int64_t N, int64_t K, int TN, int ctas, bo
          (cut && !i8 ? 4.0 : 0.0);
 }
 
-// What a problem adds to a batch's tensor-core launch: its tiles' share of the
-// workers (the launch's fixed costs are there already).
-double dense_marginal_us(int64_t n_tiles, int64_t N, int64_t K, int TN) {
-  const int64_t tiles = (n_tiles + 1) / 2 * ((N + TN - 1) / TN);
-  const double cost = (double)std::max<int64_t>(slabs_of(K), kEpiCost);
-  return (double)tiles * cost * (TN == 256 ? 0.275 : 0.185) / (num_sms() / 2);
-}
-
 rosko_status dense_batch_launch(const DenseJob* jobs, int count, int TN, int cg, cudaStream_t st) {
   return dispatch_jobs(jobs, count, TN, cg, num_sms(), false, false, st);
 }
