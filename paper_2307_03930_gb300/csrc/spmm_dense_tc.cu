@@ -53,9 +53,9 @@
 // hands the tile to TMA: a tensor store for a whole tile, a tensor
 // reduce-add (element-wise add in L2) for a cut tile or C += A.B.
 //
-// Accumulators end every kChunkSlabs K slabs; the epilogue adds each chunk to
-// its sums in registers while the next chunk's MMAs run, and writes C once
-// per range.  INT8 packs run through the same BF16 pipe (GB300's INT8 tensor
+// Accumulators end every kChunkSlabs K slabs (kShortSlabs in a short range);
+// the epilogue adds each chunk to its sums in registers while the next chunk's
+// MMAs run, and writes C once per range.  INT8 packs run through the same BF16 pipe (GB300's INT8 tensor
 // rate is far below it): the codes are exact in BF16, every chunk's FP32 sum
 // is still an exact integer and is converted and summed in INT32; C is INT32,
 // or FP32 times the row and column scales.  (Adding every chunk into INT32 C in
@@ -107,7 +107,25 @@ static_assert(128 * kRegsRest + 32 * kEpiWarps * kRegsEpi <= kThreads * kRegsLau
 // bits: 2.1e-6 in chains of 54 slabs, 1.0e-6 of 27); chunks of 16 slabs added
 // with round-to-nearest keep it below 1e-6 whatever K and the split are, and
 // draining them costs nothing (the MMAs of the next chunk run meanwhile).
+// Short ranges (a whole tile of 16 to 32 slabs, a piece of up to 16, any range
+// of a batch) close their sums every 8 at the latest: a split of all the work
+// over every SM would cut them there, and dealing them whole must not cost
+// precision (1827x1157x1232 at 80 %: 2.6e-7 with a chain of 16 slabs, 1.4e-7
+// so; 175x3497x2048 at 77 % in a batch: 1.7e-7, 1.0e-7).  For all ranges 8
+// would cost the long ones 8 % (11008x4096x2048 102 -> 111 us: the drains take
+// TMEM from the MMAs), 4 would cost 36 %; tiles of fewer than 16 slabs, which
+// no split of a single product cuts, 7 % (7541x545x6775 184 -> 198 us).
 constexpr int kChunkSlabs = 16;
+constexpr int kShortSlabs = 8;
+template <int NP, bool I8>
+__device__ __forceinline__ int chunk_slabs(int range, bool whole) {
+  const bool is_short = NP > 1 ? range > kShortSlabs
+                               : whole ? range >= kChunkSlabs && range <= 2 * kChunkSlabs
+                                       : range <= kChunkSlabs;
+  if (I8 || !is_short) return kChunkSlabs;
+  const int n = (range + kShortSlabs - 1) / kShortSlabs;   // equal chunks
+  return (range + n - 1) / n;
+}
 // A tile's cost in K slabs is at least its epilogue's time (128 KB per
 // 128 x 256 accumulator at ~28 B/clk: about nine slabs of 512 cycles; the
 // same ratio for 128-column tiles).
@@ -420,9 +438,10 @@ __global__ void __cluster_dims__(CG, 1, 1) __maxnreg__(kRegsLaunch)
     uint32_t used0 = 0, used1 = 0;       // chunks given to each group so far
     while (rank == 0 && ok && it.next(sg)) {
       if (kParts == 1) grp ^= 1;
+      const int slabs = chunk_slabs<NP, I8>(sg.s1 - sg.s0, sg.whole);
       for (int c0 = sg.s0; ok && c0 < sg.s1;) {
         // slabs [c0, c1) sum in one accumulator
-        const int c1 = min(sg.s1, c0 + kChunkSlabs);
+        const int c1 = min(sg.s1, c0 + slabs);
         const uint32_t u = grp ? used1++ : used0++;
         const int b = 2 * grp + (int)(u & 1u);
         // the epilogue (of both CTAs) must have drained this accumulator
@@ -517,7 +536,8 @@ __global__ void __cluster_dims__(CG, 1, 1) __maxnreg__(kRegsLaunch)
 #pragma unroll
         for (int j = 0; j < 32; ++j) sum[cc][j] = 0;
       bool ok = true;
-      for (int c0 = sg.s0; c0 < sg.s1; c0 += kChunkSlabs) {
+      const int slabs = chunk_slabs<NP, I8>(sg.s1 - sg.s0, sg.whole);
+      for (int c0 = sg.s0; c0 < sg.s1; c0 += slabs) {
         ok = wait_acc() && ok;
 #pragma unroll
         for (int h = 0; h < 2 * kChunks; ++h) {
