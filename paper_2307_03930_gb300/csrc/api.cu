@@ -255,8 +255,15 @@ rosko_status schedule_analytic(int64_t M, int64_t K, int64_t N, int64_t nnz, int
   // chunks per lane) halve the work items, and with them the dependent
   // segment and record loads per byte of B (512 x 4608 x 3136 layer: 7.4
   // against 8.3 us at 99.8%, 18.3 against 18.6 us at 99%; denser layers are
-  // faster with 256 columns)
-  if (order == 4 && dt == ROSKO_BF16 && d < 0.015 && N >= 1024) V = 16;
+  // faster with 256 columns).  They have no second set of sums, so long rows
+  // would be cut there (direct_pick) where 256-column strips keep them whole,
+  // as exactly and faster, unless there are four waves of rows: 600x11008x2048
+  // at 98.8% (132 a row) 35.7 us cut / 28.0, 512x4608x3136 at 98.6% (65) 26.6 /
+  // 19.4, at 98.8% (55, whole in both) 16.1 / 17.3; 4096x11008x2048 at 99%
+  // (110, whole in both) 103.7 / 122.9.
+  if (order == 4 && dt == ROSKO_BF16 && d < 0.015 && N >= 1024 &&
+      (nnz <= 56 * M || M * ((N + 511) / 512) >= 4LL * 24 * sms))
+    V = 16;
   const int NR = 32 * V;
   const int64_t P = (M + m_r - 1) / m_r;
   int W = 4;

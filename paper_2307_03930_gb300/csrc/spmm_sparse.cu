@@ -1234,6 +1234,11 @@ const SegEntry* direct_segments(const rosko_packed_s* h, const int32_t* panel_li
 // 1024x1024x1024 at 90 % 28.8 / 25.0 (FP32), 24.8 / 17.0 (BF16), 512x4608x3136
 // at 90 % 127 / 94 (BF16), 117 / 91 (INT8); 128x4000x300 at 90 % (400 per row)
 // 14.5 / 35.8 (FP32), 300x4000x500 at 95 % 12.5 / 15.4 (BF16).
+// V > 8: 512-column strips have no second set of sums (see two_level), so that
+// a whole row is one chain, and rows stay whole only from four waves on
+// (2048x32768x1024 at 98.8 %, ~390 records a row, against 64 bits: 1.4e-7 whole,
+// 7.3e-8 in pieces of 64; the analytic rule takes 256 columns there, whole at
+// 7.3e-8 and 108 against 136 us).
 // narrow: the few-column kernel, whose pieces each end in a shuffle tree: rows
 // stay whole (11008x4096x16 at 90 %: 31 us in pieces of 64, 14.4 whole).
 constexpr int kCutRecords = 320;
@@ -1241,9 +1246,14 @@ int direct_pick(const rosko_packed_s* h, const int32_t* panel_list, int64_t n_pa
                 int V, int narrow) {
   int64_t ns = 0, ns_fine = 0;
   if (!direct_segments(h, panel_list, n_panels, 1, &ns, nullptr)) return 0;
-  if (narrow || h->segs[1].records < kCutRecords) return 1;
+  if (narrow) return 1;
   const int64_t strips = (N + 32 * V - 1) / (32 * V);
-  if (ns * strips >= 24LL * num_sms()) return 1;
+  if (V <= 8) {
+    if (h->segs[1].records < kCutRecords) return 1;
+    if (ns * strips >= 24LL * num_sms()) return 1;
+  } else if (ns * strips >= 4LL * 24 * num_sms()) {
+    return 1;
+  }
   if (!direct_segments(h, panel_list, n_panels, 0, &ns_fine, nullptr)) return 1;
   return 4 * ns_fine >= 5 * ns ? 0 : 1;
 }
