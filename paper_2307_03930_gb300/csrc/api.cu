@@ -520,6 +520,16 @@ rosko_status spmm_run(rosko_packed_s* A, const void* B_dev, rosko_dtype b_dtype,
     if (tile->dense_m_c > 0) t.dense_m_c = tile->dense_m_c;
     if (tile->order > 0) t.order = tile->order;
   }
+  if (p == ROSKO_I8 && c_dtype == ROSKO_F32 && t.dense_split_pm <= 1000 &&
+      !(tile && tile->dense_split_pm > 0)) {
+    // a dequantised result rounds every piece of a cut tile, so the tensor cores
+    // do not take tiles in many more pieces than the CUDA cores would take rows
+    // (881x8331x58 at 97.2%: 16 pieces, 8.2e-8 from the 64-bit result in 16 us;
+    // rows in 4, 5.5e-8 in 13; 2458x8181x12 at 95.3%: 8 and 6 pieces, 6.4e-8 both,
+    // 19 and 34 us)
+    const int64_t pieces = dense_pieces((A->M + 127) / 128, N, A->K, t.dense_n_r, t.dense_split_k);
+    if (pieces > std::max<int64_t>(4, A->nnz / (48 * A->M))) t.dense_split_pm = 1001;
+  }
   // ---- dense-panel split: a prefix of the density-sorted dense copies ----
   int64_t n_dense = 0, dense_panels = 0;
   // tensor-core tiles: BF16, or INT8 codes (integer sums exact)

@@ -268,6 +268,8 @@ int dense_group(int64_t n_tiles);
 // Estimated time (us) of a single problem's launches on the tensor cores.
 double dense_time_us(int64_t n_tiles, int64_t N, int64_t K, int TN, int ctas, bool i8);
 bool dense_needs_zero(int64_t n_tiles, int64_t N, int64_t K, int TN, int ctas, bool i8);
+// Pieces that an INT8 product's split cuts a tile into (1: every tile whole).
+int64_t dense_pieces(int64_t n_tiles, int64_t N, int64_t K, int TN, int ctas);
 
 // api.cu
 rosko_status spmm_validate(rosko_packed_s* A, const void* B_dev, rosko_dtype b_dtype, int64_t N,

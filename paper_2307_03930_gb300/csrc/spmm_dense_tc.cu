@@ -1021,6 +1021,21 @@ bool dense_needs_zero(int64_t n_tiles, int64_t N, int64_t K, int TN, int ctas, b
   return !cut.empty() && cut[0];
 }
 
+int64_t dense_pieces(int64_t n_tiles, int64_t N, int64_t K, int TN, int ctas) {
+  if (n_tiles <= 0 || N <= 0) return 1;
+  if (ctas <= 0) ctas = num_sms();
+  DenseJob j{};
+  j.n_tiles = n_tiles;
+  j.N = N;
+  j.K = K;
+  j.i8 = 1;
+  DenseProb p{};
+  DenseSplit S{};
+  if (!plan_split(&j, 1, TN, ctas, group_of(n_tiles, ctas), &p, &S) || !S.cut) return 1;
+  const int64_t share = std::max(1, S.units / S.workers);
+  return (p.slabs + share - 1) / share;
+}
+
 // ~4.6 us around the first and last slabs, the longest share at the measured
 // rate per slab (a 256-column slab runs at ~530 cycles of the 512 that the
 // pipe needs, a 128-column one at ~350: it moves 96 bytes per pipe cycle into
