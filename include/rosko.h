@@ -72,7 +72,11 @@ typedef enum {
  * Tile parameters (Sec. 4.2 and Sec. 6 expose m_c, k_c, m_r, n_r).
  *   m_r   rows per packed panel = C rows one warp holds in registers
  *         (8, 16 or 32); fixed when A is packed.
- *   n_r   C columns per CTA tile (32 lanes x columns per lane).
+ *   n_r   C columns per CTA tile (32 lanes x columns per lane).  Order 4 with
+ *         few columns of C may run a kernel that keeps a narrower strip of B in
+ *         shared memory instead (FP32, BF16), where n_r is left to the library
+ *         or is the analytic rule's own (a plan passed back; not in
+ *         ROSKO_SCHED_FORCED); rosko_plan.few_n_r reports it.
  *   k_c   rows of B staged in shared memory per pipeline slab.
  *   m_c   C rows per CTA = warps per CTA x m_r.
  *   split_k  number of K ranges reduced into C with atomics (>= 1).
@@ -213,6 +217,8 @@ typedef struct {
   int32_t order;          /* CUDA-core traversal (1..4), 0 when no panel      */
   int32_t zero_fill;      /* 1 when C is zero-filled before the kernels       */
   rosko_tile tile;        /* the schedule resolved for the call               */
+  int32_t few_n_r;        /* columns per strip of the few-column kernel, 0 when
+                             another one runs the CUDA-core path              */
 } rosko_plan;
 
 /*

@@ -239,8 +239,9 @@ static bool bf16_little_work(int64_t M, int64_t K, int64_t N, int64_t nnz) {
 // ceil(M / m_c) times, so m_c = W m_r grows with M; K is split only as far as
 // needed to put ~2 CTAs on every SM.
 // ---------------------------------------------------------------------------
+// few: the caller can run the few-column kernel, which n_r does not describe.
 rosko_status schedule_analytic(int64_t M, int64_t K, int64_t N, int64_t nnz, int32_t m_r,
-                               rosko_dtype dt, int sms, rosko_tile* t) {
+                               rosko_dtype dt, int sms, rosko_tile* t, bool few) {
   if (m_r <= 0) m_r = 16;
   const double d = (M * K > 0) ? (double)nnz / ((double)M * (double)K) : 0.0;
   // Traversal: row-direct (each C row walks its own nonzeros, k ascending,
@@ -301,7 +302,7 @@ rosko_status schedule_analytic(int64_t M, int64_t K, int64_t N, int64_t nnz, int
     double t_dense = dense_time_us((M + 127) / 128, N, K, TN, ds, dt == ROSKO_I8);
     if (dt == ROSKO_I8) t_dense += 3.5 + 3.0 * (double)K * (double)N / 5e6;
     double t_direct = direct_time_us(M, N, nnz, dt, sms);
-    const int lpr = narrow_pick(M, K, N, nnz, dt, sms);
+    const int lpr = few ? narrow_pick(M, K, N, nnz, dt, sms) : 0;
     if (lpr > 0) t_direct = std::min(t_direct, narrow_time_us(M, K, N, nnz, dt, lpr, sms));
     if (t_direct < t_dense || (dt == ROSKO_BF16 && bf16_little_work(M, K, N, nnz)))
       t->dense_split_pm = 1001;
@@ -491,6 +492,7 @@ rosko_status spmm_validate(rosko_packed_s* A, const void* B_dev, rosko_dtype b_d
 // Resolve the tile (fields <= 0 take the analytic rule) and launch the dense
 // and sparse paths.  Arguments were validated by spmm_validate.
 // Output of a plan-only run (kRunPlanOnly), per calling thread.
+static_assert(sizeof(rosko_plan) == 72, "rosko_plan keeps its size");
 thread_local rosko_plan* g_plan_out = nullptr;
 
 rosko_status spmm_run(rosko_packed_s* A, const void* B_dev, rosko_dtype b_dtype, int64_t N,
@@ -505,7 +507,17 @@ rosko_status spmm_run(rosko_packed_s* A, const void* B_dev, rosko_dtype b_dtype,
   rosko_tile t{};
   const bool forced = tile && tile->mode == ROSKO_SCHED_FORCED;
   const int sms = num_sms();
-  schedule_analytic(A->M, A->K, N, A->nnz, A->m_r, p, sms, &t);
+  // The few-column kernel stands for row-direct in the rule, so only a call that
+  // leaves traversal and width to the library runs it: none given, or (a plan
+  // passed back) those of the rule itself.  For another width the rule weighs
+  // the tensor cores against the general kernel (11008x4096x16 at 90%: 14 us
+  // few-column, 20 tensor cores, 165 general).
+  bool few = !(tile && tile->order > 0 && tile->order != 4);
+  schedule_analytic(A->M, A->K, N, A->nnz, A->m_r, p, sms, &t, few);
+  if (few && tile && tile->n_r > 0 && (forced || tile->n_r != t.n_r)) {
+    few = false;
+    schedule_analytic(A->M, A->K, N, A->nnz, A->m_r, p, sms, &t, few);
+  }
   if (tile) {
     if (tile->m_r > 0 && tile->m_r != A->m_r) return ROSKO_ERR_INVALID_ARG;
     if (forced && (tile->n_r <= 0 || tile->k_c <= 0 || tile->m_c <= 0 || tile->split_k <= 0))
@@ -577,11 +589,9 @@ rosko_status spmm_run(rosko_packed_s* A, const void* B_dev, rosko_dtype b_dtype,
     if (t.k_c < 8) t.k_c = 32;
     L.KC = t.k_c;
   }
-  if (L.order == 4 && !(tile && tile->n_r > 0)) {
-    // few columns: the kernel that keeps a strip of B in shared memory, where
-    // it is predicted faster (a width that the caller gives is kept)
-    L.narrow = narrow_pick(A->M, A->K, N, A->nnz, p, sms);
-  }
+  // few columns: the kernel that keeps a strip of B in shared memory, where it
+  // is predicted faster
+  if (L.order == 4 && few) L.narrow = narrow_pick(A->M, A->K, N, A->nnz, p, sms);
   if (L.order == 4) {
     // one warp per C row, B from L2: no slabs, no K split
     L.W = 1;
@@ -644,6 +654,7 @@ rosko_status spmm_run(rosko_packed_s* A, const void* B_dev, rosko_dtype b_dtype,
       out->tile.order = L.order;
       out->tile.n_r = 32 * L.V;
       out->tile.split_k = L.split;
+      out->few_n_r = n_sparse > 0 ? L.narrow * 16 / (int)bsz : 0;
     }
     return ROSKO_OK;
   }

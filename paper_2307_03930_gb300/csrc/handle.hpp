@@ -290,7 +290,7 @@ rosko_status spmm_forced(rosko_packed_s* h, const void* B, rosko_dtype b_dt, int
                          const float* col_scale, void* C, rosko_dtype c_dt, int64_t ldc,
                          const rosko_tile* t, cudaStream_t st);
 rosko_status schedule_analytic(int64_t M, int64_t K, int64_t N, int64_t nnz, int32_t m_r,
-                               rosko_dtype dt, int sms, rosko_tile* t);
+                               rosko_dtype dt, int sms, rosko_tile* t, bool few = true);
 
 // autotune.cu
 int num_candidates();

@@ -47,11 +47,13 @@ class rosko_tile(ctypes.Structure):
 
 class rosko_plan(ctypes.Structure):
     _fields_ = [("dense_tiles", ctypes.c_int64), ("sparse_panels", ctypes.c_int64),
-                ("order", ctypes.c_int32), ("zero_fill", ctypes.c_int32), ("tile", rosko_tile)]
+                ("order", ctypes.c_int32), ("zero_fill", ctypes.c_int32), ("tile", rosko_tile),
+                ("few_n_r", ctypes.c_int32)]
 
     def as_dict(self):
         return {"dense_tiles": self.dense_tiles, "sparse_panels": self.sparse_panels,
-                "order": self.order, "zero_fill": self.zero_fill, "tile": self.tile.as_dict()}
+                "order": self.order, "zero_fill": self.zero_fill, "tile": self.tile.as_dict(),
+                "few_n_r": self.few_n_r}
 
 
 def make_tile(**kw) -> rosko_tile:
