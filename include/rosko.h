@@ -243,7 +243,8 @@ rosko_status rosko_spmm_plan(rosko_packed_t A, const void* B_dev, rosko_dtype b_
  * analytic rule gives it), whose work list
  * (per-problem TMA descriptors and sizes) is passed in the kernel
  * parameters; the row-direct sparse remainders of one strip width share one
- * launch, other remainders run one launch per problem.  Per-problem arrays: A, B (device),
+ * launch, other remainders (few columns, slab traversals) run one launch per
+ * problem.  Per-problem arrays: A, B (device),
  * N, ldb, C (device), ldc; all problems share b_dtype and c_dtype.  tiles:
  * NULL (analytic rule) or `count` tiles (e.g. from rosko_autotune).  No
  * device memory is allocated

@@ -722,10 +722,11 @@ rosko_status spmm_batched_impl(int32_t count, rosko_packed_s* const* A, const vo
   std::vector<int> job_of;        // problem index of each dense job
   std::vector<rosko_tile> rest;   // per problem: tile for the sparse remainder
   std::vector<char> active((size_t)count, 0), dense_any((size_t)count, 0);
-  // row-direct remainders: columns per lane (0: another traversal) and whether
-  // a row of theirs is cut.  Resolved once: the zero fill ahead of every launch
-  // and the launch itself have to agree on both.
-  std::vector<int> direct_V((size_t)count, 0);
+  // row-direct remainders: columns per lane (0: another traversal), chunks per
+  // strip of the few-column kernel (0: the general one) and whether a row of
+  // theirs is cut.  Resolved once: the zero fill ahead of every launch and the
+  // launch itself have to agree.
+  std::vector<int> direct_V((size_t)count, 0), narrow((size_t)count, 0);
   std::vector<char> direct_cut((size_t)count, 0);
   rest.resize((size_t)count);
   // dense tiles run in one launch per tile width: each problem takes the
@@ -789,7 +790,18 @@ rosko_status spmm_batched_impl(int32_t count, rosko_packed_s* const* A, const vo
       if (A[i]->rnz && sparse_config_supported(A[i]->dt, b_dt, c_dt, A[i]->m_r, V, 4)) {
         int64_t ns = 0;
         bool cut = false;
-        const int which = direct_pick(A[i], A[i]->panel_order_dev, A[i]->P - dp, N[i], V);
+        // the few-column kernel is a launch of its own: where all of it takes less
+        // than what the problem adds to the shared one (two layers 11008x4096x16
+        // at 90% kept off the tensor cores: 311 us shared, 30 so)
+        if (r.n_r <= 0 || (r.mode != ROSKO_SCHED_FORCED && r.n_r == t.n_r)) {
+          const int lpr = narrow_pick(A[i]->M, A[i]->K, N[i], A[i]->nnz, A[i]->dt, sms);
+          if (lpr > 0 &&
+              narrow_time_us(A[i]->M, A[i]->K, N[i], A[i]->nnz, A[i]->dt, lpr, sms) <
+                  direct_work_us(A[i]->M, N[i], A[i]->nnz, A[i]->dt, sms))
+            narrow[(size_t)i] = lpr;
+        }
+        const int which = direct_pick(A[i], A[i]->panel_order_dev, A[i]->P - dp, N[i], V,
+                                      narrow[(size_t)i]);
         direct_V[(size_t)i] = V;
         if (direct_segments(A[i], A[i]->panel_order_dev, A[i]->P - dp, which, &ns, &cut) && cut)
           direct_cut[(size_t)i] = 1;
@@ -839,15 +851,27 @@ rosko_status spmm_batched_impl(int32_t count, rosko_packed_s* const* A, const vo
     if (s != ROSKO_OK) return s;
   }
   // sparse remainders (the dense tiles were launched above): the row-direct
-  // ones of one width share a launch, the others run one per problem
+  // ones of one width share a launch, the others (few columns, slab
+  // traversals) run one per problem
   std::vector<char> launched((size_t)count, 0);
   for (int32_t first = 0; first < count; ++first) {
     if (direct_V[(size_t)first] == 0 || launched[(size_t)first] || rest[(size_t)first].m_r == -1)
       continue;
     const int V = direct_V[(size_t)first];
+    if (narrow[(size_t)first]) {
+      int64_t nd = 0, dp = 0;
+      dense_prefix(A[first], rest[(size_t)first].dense_split_pm, &nd, &dp);
+      SparseLaunch L{A[first]->m_r, V, 1, 8, 2, 1, 4, narrow[(size_t)first]};
+      rosko_status s = sparse_spmm_launch(A[first], B[first], b_dt, N[first], ldb[first], nullptr,
+                                          C[first], c_dt, ldc[first], accumulate, L,
+                                          A[first]->panel_order_dev, A[first]->P - dp, false, st);
+      if (s != ROSKO_OK) return s;
+      launched[(size_t)first] = 1;
+      continue;
+    }
     std::vector<DirectJob> direct;
     for (int32_t i = first; i < count; ++i) {
-      if (direct_V[(size_t)i] != V || rest[(size_t)i].m_r == -1) continue;
+      if (direct_V[(size_t)i] != V || narrow[(size_t)i] || rest[(size_t)i].m_r == -1) continue;
       int64_t nd = 0, dp = 0;
       dense_prefix(A[i], rest[(size_t)i].dense_split_pm, &nd, &dp);
       direct.push_back(DirectJob{A[i], B[i], b_dt, N[i], ldb[i], nullptr, C[i], c_dt, ldc[i],

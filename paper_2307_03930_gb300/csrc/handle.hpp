@@ -180,6 +180,7 @@ int narrow_chunks(rosko_dtype p_dt, int64_t K, int64_t N);
 double narrow_time_us(int64_t M, int64_t K, int64_t N, int64_t nnz, rosko_dtype dt, int lpr,
                       int sms);
 double direct_time_us(int64_t M, int64_t N, int64_t nnz, rosko_dtype dt, int sms);
+double direct_work_us(int64_t M, int64_t N, int64_t nnz, rosko_dtype dt, int sms);
 // The narrow kernel's chunks per strip where it is predicted faster than the
 // general row-direct kernel, else 0.
 int narrow_pick(int64_t M, int64_t K, int64_t N, int64_t nnz, rosko_dtype dt, int sms);

@@ -1315,12 +1315,19 @@ int narrow_chunks(rosko_dtype p_dt, int64_t K, int64_t N) {
 // row's records are one chain of L2 latencies, or (long rows of few items, see
 // direct_pick) cut into short ones after a memset; and every wave of resident
 // warps costs ~1.4 us however short its rows are.
+// What a problem adds to a batch's shared launch: its records' or its work
+// items' share of the GPU.
+double direct_work_us(int64_t M, int64_t N, int64_t nnz, rosko_dtype dt, int sms) {
+  const double strips = (double)((N + 255) / 256);
+  return std::max((double)nnz * strips / sms * (dt == ROSKO_F32 ? 14.5 : 9.3) / 1.93e3,
+                  (double)M * strips / (24.0 * sms) * 1.4);
+}
+
 double direct_time_us(int64_t M, int64_t N, int64_t nnz, rosko_dtype dt, int sms) {
   const double mean = (double)nnz / (double)std::max<int64_t>(M, 1);
   const double strips = (double)((N + 255) / 256);
   const double waves = (double)M * strips / (24.0 * sms);
-  const double work = std::max(
-      (double)nnz * strips / sms * (dt == ROSKO_F32 ? 14.5 : 9.3) / 1.93e3, waves * 1.4);
+  const double work = direct_work_us(M, N, nnz, dt, sms);
   const bool cut = 2.0 * mean >= kCutRecords && waves < 1.0;
   const double per_record = dt == ROSKO_F32 ? 0.075 : (dt == ROSKO_BF16 ? 0.05 : 0.03);
   const double chain = (cut ? kSegRecords : mean) * per_record;
