@@ -359,14 +359,16 @@ rosko_status rosko_candidate(rosko_packed_t A, int64_t N, int32_t index, rosko_t
  * rule's, from rosko_schedule_analytic; tile->m_r = the handle's panel
  * height) for handles of packed_dtype, or -1 if no candidate has it.  Host
  * only.  ROSKO_SCHED_LEARNED keeps the analytic rule unless the network's
- * logit for its pick exceeds this candidate's by ln 2. */
+ * logit for its pick exceeds this candidate's by ln 2, and always where the
+ * rule runs what no candidate names (few columns, INT8 on the tensor cores). */
 int32_t rosko_candidate_index(const rosko_tile* tile, rosko_dtype packed_dtype);
 
 /*
  * rosko_autotune - per-shape search (Sec. 6: the tile parameters are exposed
  * for auto-tuning).  Times every applicable candidate on (A, B, C) with CUDA
- * events on `stream` (one untimed launch, then `reps` timed launches), writes
- * the fastest to *best and caches it for (A, N): a later rosko_spmm with
+ * events on `stream` (one untimed launch, then `reps` timed launches), and the
+ * analytic rule where it runs what no candidate names; writes the fastest to
+ * *best (the rule: mode ROSKO_SCHED_ANALYTIC, every other field 0) and caches it for (A, N): a later rosko_spmm with
  * tile->mode = ROSKO_SCHED_AUTOTUNE uses it.  C is used as scratch output.
  * times_ms (optional, rosko_num_candidates() floats) receives each
  * candidate's mean time in ms, -1 where it does not apply.  Synchronises.

@@ -88,10 +88,14 @@ int candidate_index(const rosko_tile* t, rosko_dtype dt) {
 }
 
 // The applicable candidate whose schedule is the analytic rule's for this
-// handle and width, or -1.
+// handle and width, or -1: the rule also runs kernels that no candidate names
+// (few columns of C, INT8 on the tensor cores).
 int analytic_candidate(const rosko_packed_s* h, int64_t N) {
   rosko_tile a;
   schedule_analytic(h->M, h->K, N, h->nnz, h->m_r, h->dt, num_sms(), &a);
+  if (a.order == 4 && a.dense_split_pm > 1000 &&
+      narrow_pick(h->M, h->K, N, h->nnz, h->dt, num_sms()) > 0)
+    return -1;
   const int i = candidate_index(&a, h->dt);
   rosko_tile t;
   return (i >= 0 && candidate_tile(h, N, i, &t)) ? i : -1;
@@ -248,6 +252,22 @@ rosko_status autotune_impl(rosko_packed_s* h, const void* B, rosko_dtype b_dt, i
     if (ms < best_ms) {
       best_ms = ms;
       best_i = i;
+      bt = t;
+    }
+  }
+  if (ret == ROSKO_OK && analytic_candidate(h, N) < 0) {
+    // the rule's own schedule is none of the candidates: it competes as a tile
+    // that leaves everything to the rule (dequantised 512x4608x3136 at 90%: 28
+    // us, the best candidate 90; 11008x4096x16 at 90%: 14.7 / 19.6)
+    rosko_tile t{};
+    t.mode = ROSKO_SCHED_ANALYTIC;
+    rosko_status s = ROSKO_OK;
+    const float ms = time_candidate(h, B, b_dt, N, ldb, col_scale, C, c_dt, ldc, &t, reps, ts, e0,
+                                    e1, &s);
+    if (s != ROSKO_OK) {
+      ret = s;
+    } else if (ms < best_ms) {
+      best_i = nc;
       bt = t;
     }
   }
