@@ -9,6 +9,7 @@
 #include <utility>
 
 #include "../../include/rosko.h"
+#include "per_device.hpp"
 
 namespace rosko {
 
@@ -278,6 +279,16 @@ CUresult encode_tiled(CUtensorMap* map, CUtensorMapDataType dt, cuuint32_t rank,
 int num_sms();
 // Count of kernels launched by the library (rosko_kernel_launches).
 void count_launches(int n);
+
+// fn's dynamic shared memory limit on the current device is at least `bytes`.
+template <class... P>
+bool allow_smem(SmemLimit& limit, void (*fn)(P...), size_t bytes) {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return false;
+  return limit.ensure(dev, (int)bytes, [fn](int n) {
+    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, n) == cudaSuccess;
+  });
+}
 
 // Launch as a programmatic dependent of the launch before it on the stream:
 // scheduled while that one ends, its kernel waits (pdl_wait) before it touches

@@ -779,14 +779,9 @@ template <int TN, int NP, int CG, bool I8>
 rosko_status launch_table(const DenseTable<NP>& T, cudaStream_t st) {
   constexpr int stages = dense_stages<TN, CG>();
   const size_t smem = dense_smem_bytes<TN, CG>();
-  static bool set = false;
+  static SmemLimit limit;
   auto fn = dense_panel_kernel<TN, NP, CG, I8>;
-  if (!set) {
-    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-        cudaSuccess)
-      return ROSKO_ERR_CUDA;
-    set = true;
-  }
+  if (!allow_smem(limit, fn, smem)) return ROSKO_ERR_CUDA;
   if (launch_dependent(fn, dim3((unsigned)(T.split.workers * CG)), dim3(kThreads), smem, st, T,
                        stages) != cudaSuccess)
     return ROSKO_ERR_CUDA;

@@ -20,7 +20,6 @@
 //     contiguous 512-byte run (conflict free);
 //   * C is written once at the end (or added with atomics when K is split
 //     across CTAs).
-#include <atomic>
 #include <type_traits>
 #include <algorithm>
 #include <climits>
@@ -1081,15 +1080,15 @@ struct Entry {
   rosko_dtype a, b, c;
   int R, V, order;
   KernelFn fn;
-  size_t smem_set;
+  SmemLimit limit;
 };
 
 #define ROSKO_COL(TA, TB, TC, DA, DB, DC, R, V) \
-  {DA, DB, DC, R, V, 1, sparse_spmm_kernel<TA, TB, TC, R, V, 1>, 0}
+  {DA, DB, DC, R, V, 1, sparse_spmm_kernel<TA, TB, TC, R, V, 1>, {}}
 #define ROSKO_ROW(TA, TB, TC, DA, DB, DC, R, V) \
-  {DA, DB, DC, R, V, 2, sparse_spmm_kernel<TA, TB, TC, R, V, 2>, 0}
+  {DA, DB, DC, R, V, 2, sparse_spmm_kernel<TA, TB, TC, R, V, 2>, {}}
 #define ROSKO_GATHER(TA, TB, TC, DA, DB, DC, R, V) \
-  {DA, DB, DC, R, V, 3, sparse_spmm_kernel<TA, TB, TC, R, V, 3>, 0}
+  {DA, DB, DC, R, V, 3, sparse_spmm_kernel<TA, TB, TC, R, V, 3>, {}}
 // order 4 has its own kernel and signature (see DirectEntry)
 
 // Column order: m_r x V = 128 accumulators per lane (wide strips amortise the
@@ -1140,7 +1139,7 @@ struct DirectEntry {
   void (*one)(const DirectTable<1>);
   void (*many)(const DirectTable<64>);
   size_t smem;                   // dynamic shared memory (the warps' rings)
-  mutable bool attr_set = false;
+  mutable SmemLimit one_limit = {}, many_limit = {};
 };
 
 #define ROSKO_DIRECT(TA, TB, TC, DA, DB, DC, V)                                              \
@@ -1262,14 +1261,9 @@ namespace {
 template <class TA, class TB>
 rosko_status narrow_launch(const NarrowParams& p, int lpr, bool is_long, int grid, size_t smem,
                            cudaStream_t st) {
-  static std::atomic<bool> set[8];
+  static SmemLimit limit[8];
   auto go = [&](auto fn, int i) -> rosko_status {
-    if (!set[i].load(std::memory_order_acquire)) {
-      if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kNarrowSmem) !=
-          cudaSuccess)
-        return ROSKO_ERR_CUDA;
-      set[i].store(true, std::memory_order_release);
-    }
+    if (!allow_smem(limit[i], fn, kNarrowSmem)) return ROSKO_ERR_CUDA;
     if (launch_dependent(fn, dim3((unsigned)grid), dim3(32 * kNarrowWarps), smem, st, p) !=
         cudaSuccess)
       return ROSKO_ERR_CUDA;
@@ -1417,14 +1411,9 @@ rosko_status direct_batch_launch(const DirectJob* jobs, int count, int V, cudaSt
     T.total = items;
     return items;
   };
-  if (!e->attr_set) {
-    if (cudaFuncSetAttribute(e->one, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)e->smem) !=
-            cudaSuccess ||
-        cudaFuncSetAttribute(e->many, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)e->smem) !=
-            cudaSuccess)
-      return ROSKO_ERR_CUDA;
-    e->attr_set = true;
-  }
+  if (!(count == 1 ? allow_smem(e->one_limit, e->one, e->smem)
+                   : allow_smem(e->many_limit, e->many, e->smem)))
+    return ROSKO_ERR_CUDA;
   if (count == 1) {
     DirectTable<1> T;
     std::memset(static_cast<void*>(&T), 0, sizeof(T));
@@ -1496,12 +1485,7 @@ rosko_status sparse_spmm_launch(rosko_packed_s* h, const void* B, rosko_dtype b_
   const int NR = 32 * L.V;
   const size_t bsz = dtype_size(b_dt), csz = dtype_size(c_dt);
   const size_t smem = 1024 + (size_t)L.stages * L.KC * NR * bsz;
-  if (smem > e->smem_set) {
-    if (cudaFuncSetAttribute(e->fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-        cudaSuccess)
-      return ROSKO_ERR_CUDA;
-    e->smem_set = smem;
-  }
+  if (!allow_smem(e->limit, e->fn, smem)) return ROSKO_ERR_CUDA;
   // a TMA box is at most 256 elements wide: wide strips take several boxes
   const int boxes = NR > 256 ? NR / 256 : 1;
   CUtensorMap map;
