@@ -69,6 +69,7 @@
 
 #include "handle.hpp"
 #include "tc_common.cuh"
+#include "wait_gate.hpp"
 
 namespace rosko {
 namespace {
@@ -418,7 +419,7 @@ __global__ void __cluster_dims__(CG, 1, 1) __maxnreg__(kRegsLaunch)
     __syncwarp();
   } else if (warp == 1) {
     // ---------------- MMA issuer --------------------------------------------
-    // The warp waits together; lane 0 issues the MMAs and the commits.  The
+    // The warp waits together; an elected lane issues the MMAs and the commits.  The
     // smem descriptors of stage 0 are built once; stage s and K step kk only
     // move the start address (a 14-bit field in 16-byte units: shared memory
     // is below 256 KB, so the sum never carries out of it).
@@ -504,10 +505,13 @@ __global__ void __cluster_dims__(CG, 1, 1) __maxnreg__(kRegsLaunch)
     uint32_t used = 0;             // chunks of this group so far
     int b = 0;                     // accumulator of the current one
     const bool i32 = I8 && !T.row_scale;
+    WaitGate gate;   // (warp-uniform)
     auto wait_acc = [&]() -> bool {
       b = (kParts == 1 ? 2 * group : 0) + (int)(used & 1u);
-      const bool ok = __all_sync(0xffffffffu,
-                                 mbar_wait_bounded(&acc_full[b], (used >> 1) & 1u, T.status));
+      const bool ok = gate([&] {
+        return __all_sync(0xffffffffu,
+                          mbar_wait_bounded(&acc_full[b], (used >> 1) & 1u, T.status)) != 0;
+      });
       ++used;
       tc::fence_after_sync();
       return ok;
@@ -522,7 +526,7 @@ __global__ void __cluster_dims__(CG, 1, 1) __maxnreg__(kRegsLaunch)
         else mbar_arrive(&acc_empty[b]);
       }
     };
-    while (it.next(sg)) {
+    while (gate.open && it.next(sg)) {
       if (kParts == 1 && (turn++ & 1) != group) continue;   // the other group's tile
       const int copy = sg.mt * CG + rank;
       // the tile's C rows, fetched while the MMAs run (what else the stores
@@ -535,10 +539,9 @@ __global__ void __cluster_dims__(CG, 1, 1) __maxnreg__(kRegsLaunch)
       for (int cc = 0; cc < kChunks; ++cc)
 #pragma unroll
         for (int j = 0; j < 32; ++j) sum[cc][j] = 0;
-      bool ok = true;
       const int slabs = chunk_slabs<NP, I8>(sg.s1 - sg.s0, sg.whole);
       for (int c0 = sg.s0; c0 < sg.s1; c0 += slabs) {
-        ok = wait_acc() && ok;
+        if (!wait_acc()) break;
 #pragma unroll
         for (int h = 0; h < 2 * kChunks; ++h) {
           uint32_t r[16];
@@ -554,6 +557,7 @@ __global__ void __cluster_dims__(CG, 1, 1) __maxnreg__(kRegsLaunch)
         }
         release_acc();
       }
+      if (!gate.open) break;   // a wait ran out: nothing more is waited for or written
       const DenseProb& P = T.p[sg.q];
       const int q = sg.q;
       const int PM = P.M, PN = P.N;
@@ -626,7 +630,7 @@ __global__ void __cluster_dims__(CG, 1, 1) __maxnreg__(kRegsLaunch)
 #pragma unroll
       for (int cc = 0; cc < kChunks; ++cc) {
         const int col0 = n0 + (part * kChunks + cc) * 32;
-        if (ok && rows_ok && col0 < PN) {   // warp-uniform
+        if (rows_ok && col0 < PN) {   // warp-uniform
           if (I8 && !i32) {
             const float cs = col0 + lane < PN ? __ldg(&T.col_scale[col0 + lane]) : 0.0f;
 #pragma unroll
