@@ -89,7 +89,7 @@ typedef enum {
  *   dense_split_k  CTAs over which the tensor-core path divides its (tile, K
  *         slab) work, at most one per SM (default: one per SM); a tile whose
  *         K range is divided is added into C with atomics.
- *   order traversal of a panel inside a B slab by the CUDA-core path:
+ *   order traversal of the CUDA-core path (1 to 3: of a panel inside a B slab):
  *         1 = column order, Alg. 2 as printed (one B row per packed column,
  *         the C row picked by a run-time switch over loc_m);
  *         2 = row-slot order (each register row of C walks its own
@@ -97,12 +97,15 @@ typedef enum {
  *         K < 65280);
  *         3 = row-slot order over a gather of only the B rows the CTA's
  *         128-row tile touches (the tile's col_ind); needs m_r = 16,
- *         m_c = 128.
+ *         m_c = 128;
+ *         4 = row-direct, the default where K < 65280: every C row walks its
+ *         own nonzeros and reads their B rows from L2.
  *   mode  a rosko_sched_mode.
- *   dense_m_c  128 or 256.  The tile height follows from the work: a pair
- *         of CTAs computes 256 rows together (128 in each, sharing every
- *         staged B slab) whenever there are at least two 128-row tiles and
- *         two CTAs, else one CTA computes 128.
+ *   dense_m_c  128 or 256: checked and reported, without effect on the launch.
+ *         The tile height follows from the work: a pair of CTAs computes 256
+ *         rows together (128 in each, sharing every staged B slab) whenever
+ *         there are at least two 128-row tiles and two CTAs, else one CTA
+ *         computes 128.
  * A field <= 0 means "library chooses" (except in ROSKO_SCHED_FORCED, where
  * the sparse fields must be set and dense fields <= 0 still mean default).
  */
@@ -194,9 +197,11 @@ rosko_status rosko_pack_transposed(const void* A_dev, rosko_dtype a_dtype, int64
  * pool on `stream`, released in stream order).
  * Stream order: when C must be zero-filled first (tiles or rows cut along K
  * and added), the fill is a small kernel ahead of a tensor-core launch (of
- * the cut tiles only, unless the sparse part adds too), else a memset.  Every
- * kernel of the call is launched as a programmatic dependent of whatever
- * kernel precedes it on `stream`: it is scheduled while that one ends and
+ * the cut tiles only, unless the sparse part adds too), else a memset.  The
+ * kernels of the tensor-core path and of order 4 (the default CUDA-core
+ * traversal) are launched as programmatic dependents of whatever kernel
+ * precedes them on `stream`, those of orders 1 to 3 ordinarily.  A dependent
+ * is scheduled while the kernel before it ends and
  * reads and writes nothing before it has completed (the tensor-core kernel
  * after a fill reads A and B while the fill runs and writes C after it).
  * This keeps ordinary stream-order semantics for the caller; it only takes

@@ -663,8 +663,7 @@ __global__ void __cluster_dims__(CG, 1, 1) __maxnreg__(kRegsLaunch)
 // zeroes its part of the tile when that is the tile's first cut.
 constexpr int kFillParts = 8;
 constexpr int kFillThreads = 128;   // few registers a block: see kRegsLaunch
-template <int NP>
-__device__ __forceinline__ void fill_cut_tile(const DenseTable<NP>& T, int CG, int TN, int b,
+__device__ __forceinline__ void fill_cut_tile(const DenseTable<1>& T, int CG, int TN, int b,
                                               int part) {
   const DensePos c = T.start[b + 1];
   if (c.q >= T.split.count || c.slab == 0) return;
@@ -696,9 +695,8 @@ __device__ __forceinline__ void fill_cut_tile(const DenseTable<NP>& T, int CG, i
 // A programmatic dependent of the launch before it that lets the tensor-core
 // launch start once that one has completed: its A and B are then final and
 // only its writes of C wait for this fill.
-template <int NP>
 __global__ void __launch_bounds__(kFillThreads)
-    dense_cut_fill_kernel(const __grid_constant__ DenseTable<NP> T, int CG, int TN) {
+    dense_cut_fill_kernel(const __grid_constant__ DenseTable<1> T, int CG, int TN) {
   pdl_wait();
   pdl_trigger();
   fill_cut_tile(T, CG, TN, (int)blockIdx.x / kFillParts, (int)blockIdx.x % kFillParts);
@@ -965,11 +963,13 @@ rosko_status run_jobs(const DenseJob* jobs, int count, int ctas, bool zero_cut, 
                          0, st, c, T, CG, TN) != cudaSuccess)
       return ROSKO_ERR_CUDA;
     count_launches(1);
-  } else if (fill_blocks > 0) {
-    if (launch_dependent(dense_cut_fill_kernel<NP>, dim3((unsigned)fill_blocks),
-                         dim3(kFillThreads), 0, st, T, CG, TN) != cudaSuccess)
-      return ROSKO_ERR_CUDA;
-    count_launches(1);
+  } else if constexpr (NP == 1) {   // (a batch's caller zero-fills before the launch)
+    if (fill_blocks > 0) {
+      if (launch_dependent(dense_cut_fill_kernel, dim3((unsigned)fill_blocks), dim3(kFillThreads),
+                           0, st, T, CG, TN) != cudaSuccess)
+        return ROSKO_ERR_CUDA;
+      count_launches(1);
+    }
   }
   return launch_table<TN, NP, CG, I8>(T, st);
 }
@@ -1183,9 +1183,8 @@ rosko_status dense_spmm_launch(const rosko_packed_s* h, int64_t n_tiles, const v
   j.ldc = ldc;
   j.M = h->M;
   j.accumulate = accumulate;
-  // a programmatic dependent of its zero fill only (it reads A and B before
-  // any wait, which is safe only after a launch that started after every
-  // earlier one had completed)
+  // (after its zero fill the launch reads A and B before any wait: the fill
+  // started after every earlier launch had completed)
   return dispatch_jobs(&j, 1, TN, group_of(n_tiles, ctas), ctas, zero_cut, zf != nullptr, st);
 }
 
