@@ -1233,6 +1233,10 @@ const SegEntry* direct_segments(const rosko_packed_s* h, const int32_t* panel_li
 // 1024x1024x1024 at 90 % 28.8 / 25.0 (FP32), 24.8 / 17.0 (BF16), 512x4608x3136
 // at 90 % 127 / 94 (BF16), 117 / 91 (INT8); 128x4000x300 at 90 % (400 per row)
 // 14.5 / 35.8 (FP32), 300x4000x500 at 95 % 12.5 / 15.4 (BF16).
+// Rows of very uneven length are cut in the coarse list too, whose longest
+// pieces then set the time: the fine list costs no more there, and serves below
+// four waves (3387x2647x101 with power-law rows, 5 % dense, dequantised INT8:
+// 33.3 us coarse, 29.5 fine; 3473x7946x70: 27.1 / 25.3).
 // V > 8: 512-column strips have no second set of sums (see two_level), so that
 // a whole row is one chain, and rows stay whole only from four waves on
 // (2048x32768x1024 at 98.8 %, ~390 records a row, against 64 bits: 1.4e-7 whole,
@@ -1244,10 +1248,11 @@ constexpr int kCutRecords = 320;
 int direct_pick(const rosko_packed_s* h, const int32_t* panel_list, int64_t n_panels, int64_t N,
                 int V, int narrow) {
   int64_t ns = 0, ns_fine = 0;
-  if (!direct_segments(h, panel_list, n_panels, 1, &ns, nullptr)) return 0;
+  bool cut = false;
+  if (!direct_segments(h, panel_list, n_panels, 1, &ns, &cut)) return 0;
   if (narrow) return 1;
   const int64_t strips = (N + 32 * V - 1) / (32 * V);
-  if (V <= 8) {
+  if (V <= 8 && !cut) {
     if (h->segs[1].records < kCutRecords) return 1;
     if (ns * strips >= 24LL * num_sms()) return 1;
   } else if (ns * strips >= 4LL * 24 * num_sms()) {
