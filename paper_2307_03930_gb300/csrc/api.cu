@@ -211,6 +211,11 @@ constexpr int kDenseCopyPm = 1;
 constexpr int kDenseSplitPmI8 = 15;
 constexpr int kDenseCopyPmI8 = 10;
 
+// INT8: time (us) of B to BF16 ahead of the tensor cores.
+static double convert_us(int64_t K, int64_t N) {
+  return 3.5 + 3.0 * (double)K * (double)N / 5e6;
+}
+
 // BF16 layers of little work stay with the FMAs, whatever the tensor cores
 // would save: the tensor core truncates every addition where an FMA rounds,
 // and its sums are 1.1 to 6 times as far from the 64-bit result (176x1465x29
@@ -239,9 +244,10 @@ static bool bf16_little_work(int64_t M, int64_t K, int64_t N, int64_t nnz) {
 // ceil(M / m_c) times, so m_c = W m_r grows with M; K is split only as far as
 // needed to put ~2 CTAs on every SM.
 // ---------------------------------------------------------------------------
-// few: the caller can run the few-column kernel, which n_r does not describe.
+// few: the caller can run the few-column kernel, which n_r does not describe;
+// c16: rows of C are 16-byte aligned.
 rosko_status schedule_analytic(int64_t M, int64_t K, int64_t N, int64_t nnz, int32_t m_r,
-                               rosko_dtype dt, int sms, rosko_tile* t, bool few) {
+                               rosko_dtype dt, int sms, rosko_tile* t, bool few, bool c16) {
   if (m_r <= 0) m_r = 16;
   const double d = (M * K > 0) ? (double)nnz / ((double)M * (double)K) : 0.0;
   // Traversal: row-direct (each C row walks its own nonzeros, k ascending,
@@ -299,8 +305,8 @@ rosko_status schedule_analytic(int64_t M, int64_t K, int64_t N, int64_t nnz, int
     // Estimate both on the uniform-density assumption (every tile on one side
     // of the threshold) and keep the layer sparse when row-direct is
     // predicted faster.  INT8 pays the conversion of B besides.
-    double t_dense = dense_time_us((M + 127) / 128, N, K, TN, ds, dt == ROSKO_I8);
-    if (dt == ROSKO_I8) t_dense += 3.5 + 3.0 * (double)K * (double)N / 5e6;
+    double t_dense = dense_time_us((M + 127) / 128, N, K, TN, ds, dt == ROSKO_I8, c16);
+    if (dt == ROSKO_I8) t_dense += convert_us(K, N);
     double t_direct = direct_time_us(M, N, nnz, dt, sms);
     const int lpr = few ? narrow_pick(M, K, N, nnz, dt, sms) : 0;
     if (lpr > 0) t_direct = std::min(t_direct, narrow_time_us(M, K, N, nnz, dt, lpr, sms));
@@ -513,10 +519,11 @@ rosko_status spmm_run(rosko_packed_s* A, const void* B_dev, rosko_dtype b_dtype,
   // the tensor cores against the general kernel (11008x4096x16 at 90%: 14 us
   // few-column, 20 tensor cores, 165 general).
   bool few = !(tile && tile->order > 0 && tile->order != 4);
-  schedule_analytic(A->M, A->K, N, A->nnz, A->m_r, p, sms, &t, few);
+  const bool c16 = reinterpret_cast<uintptr_t>(C_dev) % 16 == 0 && ldc * (int64_t)csz % 16 == 0;
+  schedule_analytic(A->M, A->K, N, A->nnz, A->m_r, p, sms, &t, few, c16);
   if (few && tile && tile->n_r > 0 && (forced || tile->n_r != t.n_r)) {
     few = false;
-    schedule_analytic(A->M, A->K, N, A->nnz, A->m_r, p, sms, &t, few);
+    schedule_analytic(A->M, A->K, N, A->nnz, A->m_r, p, sms, &t, few, c16);
   }
   if (tile) {
     if (tile->m_r > 0 && tile->m_r != A->m_r) return ROSKO_ERR_INVALID_ARG;
@@ -551,6 +558,32 @@ rosko_status spmm_run(rosko_packed_s* A, const void* B_dev, rosko_dtype b_dtype,
            A->tile_density[(size_t)n_dense] * 1000.0 >= (double)t.dense_split_pm) {
       dense_panels += A->tile_panels[(size_t)A->tile_order[(size_t)n_dense]];
       ++n_dense;
+    }
+  }
+  if (n_dense > 0 && n_dense < A->n_tiles && t.order == 4 &&
+      !(tile && tile->dense_split_pm > 0)) {
+    // The rule took every tile for as dense as the mean.  Where only some pass
+    // the threshold, both launches have to be worth it (7911x810x4934 with
+    // power-law rows at 99%, dequantised INT8: 206 us with one tile split off,
+    // 167 without).
+    double dense_nnz = 0.0;
+    for (int64_t c = 0; c < n_dense; ++c)
+      dense_nnz += A->tile_density[(size_t)c] * 128.0 * (double)A->K;
+    const int64_t rest = std::max<int64_t>(0, A->nnz - (int64_t)dense_nnz);
+    const int64_t rest_rows = std::max<int64_t>(1, A->M - 128 * n_dense);
+    int TN = 256, ds = 1, mc = 128;
+    dense_config(n_dense, N, A->K, sms, &TN, &ds, &mc, p == ROSKO_I8);
+    auto sparse_us = [&](int64_t rows, int64_t nnz) {
+      const double us = direct_time_us(rows, N, nnz, p, sms);
+      const int lpr = few ? narrow_pick(rows, A->K, N, nnz, p, sms) : 0;
+      return lpr > 0 ? std::min(us, narrow_time_us(rows, A->K, N, nnz, p, lpr, sms)) : us;
+    };
+    const double both = dense_time_us(n_dense, N, A->K, TN, ds, p == ROSKO_I8, c16) +
+                        (p == ROSKO_I8 ? convert_us(A->K, N) : 0.0) +
+                        sparse_us(rest_rows, rest);
+    if (sparse_us(A->M, A->nnz) < both) {
+      n_dense = 0;
+      dense_panels = 0;
     }
   }
   if (n_dense > 0) {

@@ -267,7 +267,7 @@ void dense_batch_needs_zero(const DenseJob* jobs, int count, int TN, int cg, boo
 // split over `ctas` CTAs cuts a tile
 int dense_group(int64_t n_tiles);
 // Estimated time (us) of a single problem's launches on the tensor cores.
-double dense_time_us(int64_t n_tiles, int64_t N, int64_t K, int TN, int ctas, bool i8);
+double dense_time_us(int64_t n_tiles, int64_t N, int64_t K, int TN, int ctas, bool i8, bool c16);
 bool dense_needs_zero(int64_t n_tiles, int64_t N, int64_t K, int TN, int ctas, bool i8);
 // Pieces that an INT8 product's split cuts a tile into (1: every tile whole).
 int64_t dense_pieces(int64_t n_tiles, int64_t N, int64_t K, int TN, int ctas);
@@ -291,7 +291,8 @@ rosko_status spmm_forced(rosko_packed_s* h, const void* B, rosko_dtype b_dt, int
                          const float* col_scale, void* C, rosko_dtype c_dt, int64_t ldc,
                          const rosko_tile* t, cudaStream_t st);
 rosko_status schedule_analytic(int64_t M, int64_t K, int64_t N, int64_t nnz, int32_t m_r,
-                               rosko_dtype dt, int sms, rosko_tile* t, bool few = true);
+                               rosko_dtype dt, int sms, rosko_tile* t, bool few = true,
+                               bool c16 = true);
 
 // autotune.cu
 int num_candidates();

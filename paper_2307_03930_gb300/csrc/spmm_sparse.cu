@@ -1312,8 +1312,10 @@ int narrow_chunks(rosko_dtype p_dt, int64_t K, int64_t N) {
 // General: a record of a 256-column strip costs an SM ~9 cycles (BF16, INT8;
 // 14.5 for FP32's two chunks per lane), whatever of the strip lies inside N; a
 // row's records are one chain of L2 latencies, or (long rows of few items, see
-// direct_pick) cut into short ones after a memset; and every wave of resident
-// warps costs ~1.4 us however short its rows are.
+// direct_pick) cut into short ones after a memset, whose additions into C cost
+// ~5.5 us a million (185x5088x245 at 79 %: 21.6 us; without them the model said
+// 14.2, and the tensor cores' 13.5 were passed over); and every wave of
+// resident warps costs ~1.4 us however short its rows are.
 // What a problem adds to a batch's shared launch: its records' or its work
 // items' share of the GPU.
 double direct_work_us(int64_t M, int64_t N, int64_t nnz, rosko_dtype dt, int sms) {
@@ -1330,7 +1332,8 @@ double direct_time_us(int64_t M, int64_t N, int64_t nnz, rosko_dtype dt, int sms
   const bool cut = 2.0 * mean >= kCutRecords && waves < 1.0;
   const double per_record = dt == ROSKO_F32 ? 0.075 : (dt == ROSKO_BF16 ? 0.05 : 0.03);
   const double chain = (cut ? kSegRecords : mean) * per_record;
-  return 3.0 + std::max(work, chain) + (cut ? 5.0 : 0.0);
+  const double pieces = (double)nnz / kSegRecords + 0.5 * (double)M;
+  return 3.0 + std::max(work, chain) + (cut ? 5.0 + 5.5e-6 * pieces * (double)N : 0.0);
 }
 
 // Narrow: per block the load of its strip (~60 KB a microsecond), the records
