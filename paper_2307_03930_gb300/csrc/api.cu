@@ -219,12 +219,12 @@ static double convert_us(int64_t K, int64_t N) {
 // BF16 layers of little work stay with the FMAs, whatever the tensor cores
 // would save: the tensor core truncates every addition where an FMA rounds,
 // and its sums are 1.1 to 6 times as far from the 64-bit result (176x1465x29
-// at 58 %: 8.1e-8 / 4.9e-7; 1053x148x8325 at 76 %: 1.3e-8 / 1.6e-8).  The line
-// is where the time that is saved gets to several times the launch: it
-// compares the multiply-adds of the whole layer with those of its nonzeros.
-// (Letting 16 uneven layers of a batch cross it takes 102 us, 135 with it, and
-// up to 5 times the error in the layers that cross; a caller who wants that
-// gives dense_split_pm.)
+// at 58 %: 8.1e-8 / 4.9e-7; 1053x148x8325 at 76 %: 1.3e-8 / 1.6e-8).  Both
+// sides are rough times of the engines (the multiply-adds of the whole layer
+// against those of its nonzeros, and what a launch costs); the line is where
+// the tensor cores have always begun to be taken.  16 uneven layers in a batch:
+// 133 us, 102 with every layer on the tensor cores, at up to 5 times the error
+// of those that cross (a caller who wants that gives dense_split_pm).
 static bool bf16_little_work(int64_t M, int64_t K, int64_t N, int64_t nnz) {
   const double all = 10.8 + 2.0 * (double)M * (double)K * (double)N / 0.58e15 * 1e6;
   const double nonzeros = 5.3 + (double)nnz * (double)N * 2.0 / 10.9e12 * 1e6;

@@ -927,8 +927,8 @@ __global__ void __launch_bounds__(256, 3)
 // The bound is shared memory: four records with 32-byte rows meet in a
 // 128-byte phase, whose bank conflicts double it (measured: 8.1 wavefronts per
 // 512-byte request), i.e. about half a cycle per record and SM.
-// 11008 x 4096 at 90 %, N = 16, BF16: 18.5 us on the tensor cores (90 MB of
-// dense copies), 155 row-direct, 14.4 here.
+// 11008 x 4096 at 90 %, N = 16, BF16: 20 us on the tensor cores (90 MB of
+// dense copies), 165 row-direct, 14.4 here.
 constexpr int kNarrowSmem = 200 * 1024;
 constexpr int kNarrowWarps = 32;
 
