@@ -245,9 +245,10 @@ static bool bf16_little_work(int64_t M, int64_t K, int64_t N, int64_t nnz) {
 // needed to put ~2 CTAs on every SM.
 // ---------------------------------------------------------------------------
 // few: the caller can run the few-column kernel, which n_r does not describe;
-// c16: rows of C are 16-byte aligned.
+// c16: rows of C are 16-byte aligned; skewed: see direct_time_us.
 rosko_status schedule_analytic(int64_t M, int64_t K, int64_t N, int64_t nnz, int32_t m_r,
-                               rosko_dtype dt, int sms, rosko_tile* t, bool few, bool c16) {
+                               rosko_dtype dt, int sms, rosko_tile* t, bool few, bool c16,
+                               bool skewed) {
   if (m_r <= 0) m_r = 16;
   const double d = (M * K > 0) ? (double)nnz / ((double)M * (double)K) : 0.0;
   // Traversal: row-direct (each C row walks its own nonzeros, k ascending,
@@ -307,7 +308,7 @@ rosko_status schedule_analytic(int64_t M, int64_t K, int64_t N, int64_t nnz, int
     // predicted faster.  INT8 pays the conversion of B besides.
     double t_dense = dense_time_us((M + 127) / 128, N, K, TN, ds, dt == ROSKO_I8, c16);
     if (dt == ROSKO_I8) t_dense += convert_us(K, N);
-    double t_direct = direct_time_us(M, N, nnz, dt, sms);
+    double t_direct = direct_time_us(M, N, nnz, dt, sms, skewed);
     const int lpr = few ? narrow_pick(M, K, N, nnz, dt, sms) : 0;
     if (lpr > 0) t_direct = std::min(t_direct, narrow_time_us(M, K, N, nnz, dt, lpr, sms));
     if (t_direct < t_dense || (dt == ROSKO_BF16 && bf16_little_work(M, K, N, nnz)))
@@ -520,10 +521,11 @@ rosko_status spmm_run(rosko_packed_s* A, const void* B_dev, rosko_dtype b_dtype,
   // few-column, 20 tensor cores, 165 general).
   bool few = !(tile && tile->order > 0 && tile->order != 4);
   const bool c16 = reinterpret_cast<uintptr_t>(C_dev) % 16 == 0 && ldc * (int64_t)csz % 16 == 0;
-  schedule_analytic(A->M, A->K, N, A->nnz, A->m_r, p, sms, &t, few, c16);
+  const bool skewed = direct_skewed(A);
+  schedule_analytic(A->M, A->K, N, A->nnz, A->m_r, p, sms, &t, few, c16, skewed);
   if (few && tile && tile->n_r > 0 && (forced || tile->n_r != t.n_r)) {
     few = false;
-    schedule_analytic(A->M, A->K, N, A->nnz, A->m_r, p, sms, &t, few, c16);
+    schedule_analytic(A->M, A->K, N, A->nnz, A->m_r, p, sms, &t, few, c16, skewed);
   }
   if (tile) {
     if (tile->m_r > 0 && tile->m_r != A->m_r) return ROSKO_ERR_INVALID_ARG;
@@ -574,7 +576,7 @@ rosko_status spmm_run(rosko_packed_s* A, const void* B_dev, rosko_dtype b_dtype,
     int TN = 256, ds = 1, mc = 128;
     dense_config(n_dense, N, A->K, sms, &TN, &ds, &mc, p == ROSKO_I8);
     auto sparse_us = [&](int64_t rows, int64_t nnz) {
-      const double us = direct_time_us(rows, N, nnz, p, sms);
+      const double us = direct_time_us(rows, N, nnz, p, sms, skewed);
       const int lpr = few ? narrow_pick(rows, A->K, N, nnz, p, sms) : 0;
       return lpr > 0 ? std::min(us, narrow_time_us(rows, A->K, N, nnz, p, lpr, sms)) : us;
     };

@@ -92,7 +92,8 @@ int candidate_index(const rosko_tile* t, rosko_dtype dt) {
 // (few columns of C, INT8 on the tensor cores).
 int analytic_candidate(const rosko_packed_s* h, int64_t N) {
   rosko_tile a;
-  schedule_analytic(h->M, h->K, N, h->nnz, h->m_r, h->dt, num_sms(), &a);
+  schedule_analytic(h->M, h->K, N, h->nnz, h->m_r, h->dt, num_sms(), &a, true, true,
+                    direct_skewed(h));
   if (a.order == 4 && a.dense_split_pm > 1000 &&
       narrow_pick(h->M, h->K, N, h->nnz, h->dt, num_sms()) > 0)
     return -1;

@@ -179,7 +179,12 @@ struct SparseLaunch {
 int narrow_chunks(rosko_dtype p_dt, int64_t K, int64_t N);
 double narrow_time_us(int64_t M, int64_t K, int64_t N, int64_t nnz, rosko_dtype dt, int lpr,
                       int sms);
-double direct_time_us(int64_t M, int64_t N, int64_t nnz, rosko_dtype dt, int sms);
+double direct_time_us(int64_t M, int64_t N, int64_t nnz, rosko_dtype dt, int sms,
+                      bool skewed = false);
+// Rows of h so uneven that the coarse list cuts some.
+inline bool direct_skewed(const rosko_packed_s* h) {
+  return !h->segs[1].split.empty() && h->segs[1].split.back() > 0;
+}
 double direct_work_us(int64_t M, int64_t N, int64_t nnz, rosko_dtype dt, int sms);
 // The narrow kernel's chunks per strip where it is predicted faster than the
 // general row-direct kernel, else 0.
@@ -292,7 +297,7 @@ rosko_status spmm_forced(rosko_packed_s* h, const void* B, rosko_dtype b_dt, int
                          const rosko_tile* t, cudaStream_t st);
 rosko_status schedule_analytic(int64_t M, int64_t K, int64_t N, int64_t nnz, int32_t m_r,
                                rosko_dtype dt, int sms, rosko_tile* t, bool few = true,
-                               bool c16 = true);
+                               bool c16 = true, bool skewed = false);
 
 // autotune.cu
 int num_candidates();

@@ -1041,8 +1041,9 @@ int64_t dense_pieces(int64_t n_tiles, int64_t N, int64_t K, int TN, int ctas) {
 // pipe needs, a 128-column one at ~350: it moves 96 bytes per pipe cycle into
 // each SM), the last tile's epilogue, the zero fill of cut tiles (a launch),
 // INT8 into rows of C that are not 16-byte aligned (~4.5 us: dequantised
-// 2543x5414x14 / x16 at 96 % 20.1 / 15.6), and no less than the memory needs.  Called on every product: the split's
-// sizes without its positions.
+// 2543x5414x14 / x16 at 96 % 20.1 / 15.6; more where many are added in pieces:
+// 1443x3491x907 31 against 28 row-direct), and no less than the memory needs.
+// Called on every product: the split's sizes without its positions.
 double dense_time_us(int64_t n_tiles, int64_t N, int64_t K, int TN, int ctas, bool i8, bool c16) {
   if (n_tiles <= 0 || N <= 0 || K <= 0) return 0.0;
   if (ctas <= 0) ctas = num_sms();
@@ -1057,7 +1058,9 @@ double dense_time_us(int64_t n_tiles, int64_t N, int64_t K, int TN, int ctas, bo
   const double mem = (2.0 * (double)n_tiles * kTM * K + 2.0 * (double)K * N +
                       4.0 * (double)n_tiles * kTM * N) / 6.5e6;
   return 4.6 + std::max(share * (TN == 256 ? 0.275 : 0.185), mem) + (TN == 256 ? 3.7 : 1.9) +
-         (cut && !i8 ? 4.0 : 0.0) + (i8 && !c16 ? 4.5 : 0.0);
+         (cut && !i8 ? 4.0 : 0.0) +
+         (i8 && !c16 ? 4.5 + (cut && rounds == 0 ? 2e-6 * (double)n_tiles * kTM * (double)N : 0.0)
+                     : 0.0);
 }
 
 rosko_status dense_batch_launch(const DenseJob* jobs, int count, int TN, int cg, cudaStream_t st) {

@@ -1324,16 +1324,21 @@ double direct_work_us(int64_t M, int64_t N, int64_t nnz, rosko_dtype dt, int sms
                   (double)M * strips / (24.0 * sms) * 1.4);
 }
 
-double direct_time_us(int64_t M, int64_t N, int64_t nnz, rosko_dtype dt, int sms) {
+// skewed: rows are cut in the coarse list too, whose longest pieces are twice
+// the mean, and C is zero-filled for them (2119x711x224 at 79 % with power-law
+// rows: 17 us, 9 on the tensor cores; 9 by the mean row).
+double direct_time_us(int64_t M, int64_t N, int64_t nnz, rosko_dtype dt, int sms, bool skewed) {
   const double mean = (double)nnz / (double)std::max<int64_t>(M, 1);
   const double strips = (double)((N + 255) / 256);
   const double waves = (double)M * strips / (24.0 * sms);
   const double work = direct_work_us(M, N, nnz, dt, sms);
   const bool cut = 2.0 * mean >= kCutRecords && waves < 1.0;
   const double per_record = dt == ROSKO_F32 ? 0.075 : (dt == ROSKO_BF16 ? 0.05 : 0.03);
-  const double chain = (cut ? kSegRecords : mean) * per_record;
+  const double chain = (cut ? kSegRecords : skewed ? 2.0 * mean : mean) * per_record;
+  // (FP32's multiplies take long enough to hide them: 816x938x989 at 65 % 56 us)
   const double pieces = (double)nnz / kSegRecords + 0.5 * (double)M;
-  return 3.0 + std::max(work, chain) + (cut ? 5.0 + 5.5e-6 * pieces * (double)N : 0.0);
+  const double adds = dt == ROSKO_F32 ? 0.0 : 5.5e-6 * pieces * (double)N;
+  return 3.0 + std::max(work, chain) + (cut ? 5.0 + adds : skewed ? 3.0 : 0.0);
 }
 
 // Narrow: per block the load of its strip (~60 KB a microsecond), the records
@@ -1349,8 +1354,9 @@ double narrow_time_us(int64_t M, int64_t K, int64_t N, int64_t nnz, rosko_dtype 
   const double waves = (double)((strips * parts + sms - 1) / sms);
   const double wf = lpr == 1 ? 0.36 : (lpr == 2 ? 0.57 : (lpr == 4 ? 0.9 : 1.3));
   const double rows = (double)((M + parts * kNarrowWarps - 1) / (parts * kNarrowWarps));
-  const double block = (double)(K * lpr) * 16.0 / 60e3 +
-                       (double)nnz / (double)parts * wf / 1.93e3 + rows * 0.9;
+  const double records = (double)nnz / (double)parts * wf / 1.93e3;
+  const bool is_long = 2 * nnz * lpr > 32 * kNarrowChain * M;   // (the second set of sums)
+  const double block = (double)(K * lpr) * 16.0 / 60e3 + records * (is_long ? 1.07 : 1.0) + rows * 0.9;
   return 3.0 + waves * block;
 }
 

@@ -1,6 +1,6 @@
 """The default schedule where the time models had been wrong: long rows cut into
-many pieces that are added, few tiles above the threshold, and many tiles of
-which only a last few are cut.  The default takes at most 1.25 times the faster
+many pieces that are added, few tiles above the threshold, many tiles of which
+only a last few are cut, and rows of very uneven length.  The default takes at most 1.25 times the faster
 of both engines (the models' spread; they were 1.25 to 1.7 off here).  GPU only."""
 import pytest
 import torch
@@ -22,7 +22,8 @@ def _powerlaw(M, K, d, seed):
 
 @pytest.mark.parametrize("M,K,N,d,int8", [(185, 5088, 245, 0.21, False),
                                           (7911, 810, 4934, 0.0095, True),
-                                          (5692, 1522, 3505, 0.0203, True)])
+                                          (5692, 1522, 3505, 0.0203, True),
+                                          (2119, 711, 224, 0.2137, False)])
 def test_default_is_near_the_faster_engine(M, K, N, d, int8):
     rosko = built()
     h = rosko.rosko_pack(_powerlaw(M, K, d, 3), rosko.I8 if int8 else rosko.BF16)
