@@ -55,8 +55,8 @@
 //
 // Accumulators end every kChunkSlabs K slabs (kShortSlabs in a short range);
 // the epilogue adds each chunk to its sums in registers while the next chunk's
-// MMAs run, and writes C once per range.  INT8 packs run through the same BF16 pipe (GB300's INT8 tensor
-// rate is far below it): the codes are exact in BF16, every chunk's FP32 sum
+// MMAs run, and writes C once per range.  INT8 packs run through the same BF16
+// pipe (GB300's INT8 tensor rate is far below it): the codes are exact in BF16, every chunk's FP32 sum
 // is still an exact integer and is converted and summed in INT32; C is INT32,
 // or FP32 times the row and column scales.  (Adding every chunk into INT32 C in
 // global memory instead cost an epilogue per 1,024 K: 162 against 115 us for
@@ -118,11 +118,11 @@ static_assert(128 * kRegsRest + 32 * kEpiWarps * kRegsEpi <= kThreads * kRegsLau
 // no split of a single product cuts, 7 % (7541x545x6775 184 -> 198 us).
 constexpr int kChunkSlabs = 16;
 constexpr int kShortSlabs = 8;
-template <int NP, bool I8>
-__device__ __forceinline__ int chunk_slabs(int range, bool whole) {
-  const bool is_short = NP > 1 ? range > kShortSlabs
-                               : whole ? range >= kChunkSlabs && range <= 2 * kChunkSlabs
-                                       : range <= kChunkSlabs;
+template <bool I8>
+__device__ __forceinline__ int chunk_slabs(int range, bool whole, bool batch) {
+  const bool is_short = batch ? range > kShortSlabs
+                              : whole ? range >= kChunkSlabs && range <= 2 * kChunkSlabs
+                                      : range <= kChunkSlabs;
   if (I8 || !is_short) return kChunkSlabs;
   const int n = (range + kShortSlabs - 1) / kShortSlabs;   // equal chunks
   return (range + n - 1) / n;
@@ -189,6 +189,7 @@ struct DenseTable {
   // 1: the launch follows a zero fill of C that started after everything
   // before it had completed, so A and B may be read at once
   int early_ab;
+  int batch;   // the launch is (part of) a batch, of one problem or more
   int* status;
 };
 
@@ -439,7 +440,7 @@ __global__ void __cluster_dims__(CG, 1, 1) __maxnreg__(kRegsLaunch)
     uint32_t used0 = 0, used1 = 0;       // chunks given to each group so far
     while (rank == 0 && ok && it.next(sg)) {
       if (kParts == 1) grp ^= 1;
-      const int slabs = chunk_slabs<NP, I8>(sg.s1 - sg.s0, sg.whole);
+      const int slabs = chunk_slabs<I8>(sg.s1 - sg.s0, sg.whole, NP > 1 || T.batch);
       for (int c0 = sg.s0; ok && c0 < sg.s1;) {
         // slabs [c0, c1) sum in one accumulator
         const int c1 = min(sg.s1, c0 + slabs);
@@ -539,7 +540,7 @@ __global__ void __cluster_dims__(CG, 1, 1) __maxnreg__(kRegsLaunch)
       for (int cc = 0; cc < kChunks; ++cc)
 #pragma unroll
         for (int j = 0; j < 32; ++j) sum[cc][j] = 0;
-      const int slabs = chunk_slabs<NP, I8>(sg.s1 - sg.s0, sg.whole);
+      const int slabs = chunk_slabs<I8>(sg.s1 - sg.s0, sg.whole, NP > 1 || T.batch);
       for (int c0 = sg.s0; c0 < sg.s1; c0 += slabs) {
         if (!wait_acc()) break;
 #pragma unroll
@@ -915,7 +916,7 @@ rosko_status encode_dense_maps(const DenseJob& j, CUtensorMap* mA, CUtensorMap* 
 
 template <int TN, int NP, int CG, bool I8>
 rosko_status run_jobs(const DenseJob* jobs, int count, int ctas, bool zero_cut, bool after_fill,
-                      cudaStream_t st) {
+                      bool batch, cudaStream_t st) {
   static_assert(sizeof(DenseTable<NP>) <= 32 * 1024 - 256, "kernel parameter table too large");
   DenseTable<NP> T;
   std::memset(static_cast<void*>(&T), 0, sizeof(T));
@@ -943,6 +944,7 @@ rosko_status run_jobs(const DenseJob* jobs, int count, int ctas, bool zero_cut, 
   for (int b = 0; b <= T.split.workers; ++b) T.start[b] = dense_pos(T.split, T.p, b);
   T.row_scale = jobs[0].row_scale;
   T.col_scale = jobs[0].col_scale;
+  T.batch = batch ? 1 : 0;
   T.early_ab = !I8 && (zero_cut || after_fill) ? 1 : 0;
   T.status = device_status_word();
   if (!T.status) return ROSKO_ERR_CUDA;
@@ -980,26 +982,26 @@ int group_of(int64_t n_tiles, int ctas) { return n_tiles >= 2 && ctas >= 2 ? 2 :
 
 template <int TN, int NP, bool I8>
 rosko_status dispatch_group(const DenseJob* jobs, int count, int cg, int ctas, bool zero_cut,
-                            bool after_fill, cudaStream_t st) {
-  return cg == 2 ? run_jobs<TN, NP, 2, I8>(jobs, count, ctas, zero_cut, after_fill, st)
-                 : run_jobs<TN, NP, 1, I8>(jobs, count, ctas, zero_cut, after_fill, st);
+                            bool after_fill, bool batch, cudaStream_t st) {
+  return cg == 2 ? run_jobs<TN, NP, 2, I8>(jobs, count, ctas, zero_cut, after_fill, batch, st)
+                 : run_jobs<TN, NP, 1, I8>(jobs, count, ctas, zero_cut, after_fill, batch, st);
 }
 
 rosko_status dispatch_jobs(const DenseJob* jobs, int count, int TN, int cg, int ctas,
-                           bool zero_cut, bool after_fill, cudaStream_t st) {
+                           bool zero_cut, bool after_fill, bool batch, cudaStream_t st) {
   if (count <= 0) return ROSKO_OK;
   if ((TN != 128 && TN != 256) || count > 64) return ROSKO_ERR_INVALID_ARG;
   if (count == 1 && jobs[0].i8)
     return TN == 256
-               ? dispatch_group<256, 1, true>(jobs, 1, cg, ctas, zero_cut, after_fill, st)
-               : dispatch_group<128, 1, true>(jobs, 1, cg, ctas, zero_cut, after_fill, st);
+               ? dispatch_group<256, 1, true>(jobs, 1, cg, ctas, zero_cut, after_fill, batch, st)
+               : dispatch_group<128, 1, true>(jobs, 1, cg, ctas, zero_cut, after_fill, batch, st);
   if (count == 1)
     return TN == 256
-               ? dispatch_group<256, 1, false>(jobs, 1, cg, ctas, zero_cut, after_fill, st)
-               : dispatch_group<128, 1, false>(jobs, 1, cg, ctas, zero_cut, after_fill, st);
+               ? dispatch_group<256, 1, false>(jobs, 1, cg, ctas, zero_cut, after_fill, batch, st)
+               : dispatch_group<128, 1, false>(jobs, 1, cg, ctas, zero_cut, after_fill, batch, st);
   return TN == 256
-             ? dispatch_group<256, 64, false>(jobs, count, cg, ctas, zero_cut, after_fill, st)
-             : dispatch_group<128, 64, false>(jobs, count, cg, ctas, zero_cut, after_fill, st);
+             ? dispatch_group<256, 64, false>(jobs, count, cg, ctas, zero_cut, after_fill, batch, st)
+             : dispatch_group<128, 64, false>(jobs, count, cg, ctas, zero_cut, after_fill, batch, st);
 }
 
 }  // namespace
@@ -1064,7 +1066,7 @@ double dense_time_us(int64_t n_tiles, int64_t N, int64_t K, int TN, int ctas, bo
 }
 
 rosko_status dense_batch_launch(const DenseJob* jobs, int count, int TN, int cg, cudaStream_t st) {
-  return dispatch_jobs(jobs, count, TN, cg, num_sms(), false, false, st);
+  return dispatch_jobs(jobs, count, TN, cg, num_sms(), false, false, true, st);
 }
 
 // Which jobs of a batch have a tile cut between workers (job order as given;
@@ -1158,7 +1160,7 @@ rosko_status dense_spmm_i8_launch(const rosko_packed_s* h, int64_t n_tiles, cons
     j.src_ld = ldb;
     j.row_scale = col_scale ? h->row_scale : nullptr;
     j.col_scale = col_scale;
-    s = dispatch_jobs(&j, 1, TN, group_of(n_tiles, ctas), ctas, zero_cut, zf != nullptr, st);
+    s = dispatch_jobs(&j, 1, TN, group_of(n_tiles, ctas), ctas, zero_cut, zf != nullptr, false, st);
   }
   pool_free(scratch, st);
   return s;
@@ -1190,7 +1192,7 @@ rosko_status dense_spmm_launch(const rosko_packed_s* h, int64_t n_tiles, const v
   j.accumulate = accumulate;
   // (after its zero fill the launch reads A and B before any wait: the fill
   // started after every earlier launch had completed)
-  return dispatch_jobs(&j, 1, TN, group_of(n_tiles, ctas), ctas, zero_cut, zf != nullptr, st);
+  return dispatch_jobs(&j, 1, TN, group_of(n_tiles, ctas), ctas, zero_cut, zf != nullptr, false, st);
 }
 
 }  // namespace rosko
