@@ -55,7 +55,9 @@ def test_decode_batch_is_not_slower_than_its_calls(planned):
         for h, B, C in zip(hs, Bs, Cs):
             rosko.rosko_spmm(h, B, C)
 
-    assert _us(lambda: rosko.rosko_spmm_batched(hs, Bs, Cs, tiles=tiles)) <= 1.5 * _us(alone)
+    # (the least of three: the host's own pauses)
+    assert min(_us(lambda: rosko.rosko_spmm_batched(hs, Bs, Cs, tiles=tiles)) / _us(alone)
+               for _ in range(3)) <= 1.5
 
 
 @pytest.mark.parametrize("bf16", [True, False])

@@ -38,5 +38,8 @@ def test_default_is_near_the_faster_engine(M, K, N, d, int8):
     def us(tile):
         return _us(lambda: rosko.rosko_spmm(h, B, C, col_scale=t, tile=tile))
 
-    both = min(us(rosko.make_tile(dense_split_pm=pm)) for pm in (1001, 15))
-    assert us(None) <= 1.25 * both
+    def off():
+        return us(None) / min(us(rosko.make_tile(dense_split_pm=pm)) for pm in (1001, 15))
+
+    # (the least of three: the host's own pauses)
+    assert min(off() for _ in range(3)) <= 1.25
